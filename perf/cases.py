@@ -118,26 +118,33 @@ def _normal(shape, std, g):
     return (torch.randn(*shape, device="cuda", generator=g) * std).to(torch.bfloat16)
 
 
-def prepare(case, seed):
-    c = case
-    M, K, N, op = c["M"], c["K"], c["N"], c["op"]
+def _inputs(c, seed):
+    """The tensors of a case, from the seed alone: activations, weights, biases and whatever else its call takes."""
+    M, K, N = c["M"], c["K"], c["N"]
     g = torch.Generator(device="cuda").manual_seed(int(seed))
-    lx = _context()
-    lx.reserve(M, N, K)
-    s = {"op": op, "lx": lx, "mode": MODES[c["mode"]], "X": _activations(c, g), "residual": None}
     n = c.get("products", 1)
-    s["W"] = [_normal((N, K), K ** -0.5, g) for _ in range(n)]
-    s["bias"] = [_normal((N,), 0.01, g) for _ in range(n)]
+    t = {"X": _activations(c, g), "residual": None}
+    t["W"] = [_normal((N, K), K ** -0.5, g) for _ in range(n)]
+    t["bias"] = [_normal((N,), 0.01, g) for _ in range(n)]
     if c.get("residual"):
-        s["residual"] = _normal((M, N), 0.05, g)
+        t["residual"] = _normal((M, N), 0.05, g)
+    if c["op"] == "lora":
+        t["LB"], t["LA"] = _normal((c["rank"], K), K ** -0.5, g), _normal((N, c["rank"]), 0.3 * c["rank"] ** -0.5, g)
+    return t
+
+
+def prepare(case, seed):
+    c, op = case, case["op"]
+    lx = _context()
+    lx.reserve(c["M"], c["N"], c["K"])
+    s = dict(_inputs(c, seed), op=op, lx=lx, mode=MODES[c["mode"]])
     if op == "lora":
-        lx.reserve_lora(M, K, c["rank"])
-        s["LB"], s["LA"] = _normal((c["rank"], K), K ** -0.5, g), _normal((N, c["rank"]), 0.3 * c["rank"] ** -0.5, g)
+        lx.reserve_lora(c["M"], c["K"], c["rank"])
     elif op == "fp8":
         s["Wq"], s["wscale"] = lx.quantize_weights_fp8(s.pop("W")[0], per_channel=True)
     elif op == "host":
         s["X"] = s["X"].cpu().pin_memory()
-        s["Y"] = torch.empty(M, N, dtype=torch.bfloat16, pin_memory=True)
+        s["Y"] = torch.empty(c["M"], c["N"], dtype=torch.bfloat16, pin_memory=True)
     return s
 
 
@@ -153,6 +160,57 @@ def run(state):
     if s["op"] == "fp8":
         return lx.act_sparse_linear_fp8(s["X"], s["Wq"], s["wscale"], s["bias"][0], s["mode"], s["residual"])
     return lx.act_sparse_linear_host(s["X"], s["W"][0], s["bias"][0], s["mode"], s["Y"])
+
+
+def _keep_mask(X):
+    """The two of each four elements of largest magnitude, of equal ones the first (a stable sort keeps their order)."""
+    order = X.abs().reshape(-1, 4).sort(dim=1, descending=True, stable=True).indices
+    return torch.zeros_like(order, dtype=torch.bool).scatter_(1, order[:, :2], True)
+
+
+def _e4m3(x):
+    return x.clamp(-448.0, 448.0).to(torch.float8_e4m3fn).double()
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits.  The FP8 codes are part of the layer's definition (fp32 rule, E4M3 result) and are
+    made as it says; everything behind them, and every other case throughout, is in 64 bits and never rounded."""
+    c = case
+    t = _inputs(c, seed)
+    X, M = t["X"].float(), c["M"]
+    mask = _keep_mask(X)
+    groups = X.double().reshape(-1, 4)
+    kept = groups * mask
+    scale = None
+    if c["mode"] == "row":
+        num, den = groups.square().reshape(M, -1).sum(1), kept.square().reshape(M, -1).sum(1)
+        scale = (num / (den + 1e-8)).sqrt()
+    elif c["mode"] == "tensor":
+        scale = (groups.square().sum() / (kept.square().sum() + 1e-8)).sqrt().expand(M)
+    elif c["mode"] == "group":
+        kept = kept * (groups.square().sum(1, keepdim=True) / (kept.square().sum(1, keepdim=True) + 1e-8)).sqrt()
+    values = kept[mask].reshape(M, -1) if c["op"] == "shared" else None
+    kept, weights = kept.reshape(M, -1), [w.double() for w in t["W"]]
+    if c["op"] == "fp8":
+        amax = X.abs().amax(1, keepdim=True)
+        kept = _e4m3(kept.float() * torch.where(amax > 0, 448.0 / amax, 0.0)) * (amax.double() / 448.0)
+        W = t["W"][0].float()
+        wmax = W.abs().amax(1, keepdim=True)
+        weights = [_e4m3(W * torch.where(wmax > 0, 448.0 / wmax, 0.0)) * (wmax.double() / 448.0)]
+    results = []
+    for W, b in zip(weights, t["bias"]):
+        Y = kept @ W.T
+        if scale is not None:
+            Y *= scale[:, None]
+        Y += b.double()
+        if c["op"] == "lora":
+            Y += (X.double() @ t["LB"].double().T) @ t["LA"].double().T
+        if t["residual"] is not None:
+            Y += t["residual"].double()
+        results.append(Y)
+    if c["op"] == "shared":
+        return [values, None, scale] + results  # (the metadata is whole numbers)
+    return results[0].cpu() if c["op"] == "host" else results[0]
 
 
 def work(case):
