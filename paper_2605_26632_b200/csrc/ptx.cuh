@@ -89,6 +89,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return mbar_wait_limit(bar, parity, cta_abort, dev_error, WAIT_LIMIT_NS);
 }
 
+// The same wait by a whole converged warp.  The vote makes the result warp-uniform, so that the code
+// behind it (the producer and MMA issue loops) stays convergent and its operands can live in uniform
+// registers; see the note on the issue loop in sparse_gemm.cuh.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* cta_abort,
+                                               uint32_t* dev_error) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, cta_abort, dev_error));
+}
+
+// One lane of a converged warp (always the same one).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t pred;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
+    return pred != 0;
+}
+
 // Bounded wait for a global-memory word (written with release semantics by another CTA) to reach
 // `want`.  Same time limit and abort protocol as mbar_wait.
 __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {

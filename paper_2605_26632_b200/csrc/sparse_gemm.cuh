@@ -6,7 +6,7 @@
 //   warp 0      producer: TMA loads of the compressed-A tile (128 rows x 64 stored values =
 //               128 logical K), the metadata block (2048 bytes) and the W tile into a ring of
 //               STAGES shared-memory stages guarded by full/empty mbarriers
-//   warp 1      MMA issuer (one thread): copies the stage's metadata into tensor memory
+//   warp 1      MMA issuer (one elected lane): copies the stage's metadata into tensor memory
 //               (tcgen05.cp), issues four tcgen05.mma.sp kind::f16 (K = 32 logical each) into a
 //               tensor-memory fp32 accumulator, commits to the stage's empty barrier; after the
 //               last K block commits to the accumulator's full barrier
@@ -14,6 +14,13 @@
 //               row scale / bias / residual, round to bf16, stage in swizzled shared memory and
 //               TMA-store 32 x 64 boxes
 // With two accumulator buffers the epilogue of tile i overlaps the main loop of tile i+1.
+//
+// The producer and the issuer are whole warps that run their loops converged; waits end in a vote and
+// one elected lane issues.  The operands of tcgen05.mma / tcgen05.cp / TMA live in uniform registers,
+// and inside a branch that only one lane takes every one of them has to be moved there again: a
+// stage's issue (wait, copy, four MMAs, commit, loop) cost 755 cycles that way and bounded the loop
+// (755 cycles per K block with or without the A and W loads; the four MMAs of a 240-wide tile take
+// 480).  Converged, the issue takes ~240 cycles and a K block ~510-600, bound by the operand stream.
 //
 // Low-rank branch (Algorithm 1 lines 5-6, Y = Y_s + X (L_A L_B)^T): when lora_steps > 0 every
 // tile gets lora_steps extra ring stages after its last K block.  Such a stage holds a 128 x 64
@@ -272,7 +279,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + (sBar - smem_base) + 8 * Cfg::NUM_BARS);
     volatile uint32_t* cta_abort = tmem_slot + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t rank = (CG == 2) ? cluster_ctarank() : 0u;
     const bool leader = rank == 0;
     const int cluster_id = blockIdx.x / CG, num_clusters = gridDim.x / CG;
@@ -317,17 +324,17 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
     __syncthreads();
     if constexpr (CG == 2) cluster_sync_all();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     // W tiles of the first stages of the first tile, before the wait for the previous kernel
     int npre = 0;
-    if (warp == 0 && lane == 0 && p.w_prefetch && num_items > 0 && l0_n == 0) {
+    if (warp == 0 && p.w_prefetch && num_items > 0 && l0_n == 0) {
         const WorkItem w = sched.get(cluster_id, 0);
         int tm, tn;
         tile_coords(w.tile, p.tiles_m, p.tiles_n, p.group_m, tm, tn);
         const int n0 = tn * BN + (int)rank * Cfg::BN_CTA;
         npre = (w.kb1 - w.kb0 < STAGES) ? w.kb1 - w.kb0 : STAGES;
         const uint32_t full0 = (CG == 2) ? mapa(bar_full, 0) : bar_full;
-        for (int s = 0; s < npre; ++s) {
+        if (elect_one()) for (int s = 0; s < npre; ++s) {
             const int kb = w.kb0 + s;
             const uint32_t b_dst = sB + s * Cfg::B_BYTES;
             if constexpr (CG == 1) {
@@ -346,7 +353,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer ----------
-        if (lane == 0) {
+        {
             uint32_t stage = 0, phase = 0;
             uint32_t issued = 0;
             bool ok = true;
@@ -363,13 +370,14 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     const int k0 = split * p.l0_kb_per_split;
                     const int k1 = (k0 + p.l0_kb_per_split < kblocks) ? k0 + p.l0_kb_per_split : kblocks;
                     for (int kb = k0; kb < k1; ++kb) {
-                        if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error)) {
+                        if (!mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error)) {
                             ok = false;
                             break;
                         }
                         const uint32_t a_dst = sA + stage * Cfg::A_BYTES;
                         const uint32_t b_dst = sB + stage * Cfg::B_BYTES;
-                        if constexpr (CG == 1) {
+                        if (!elect_one()) {
+                        } else if constexpr (CG == 1) {
                             const uint32_t bar = bar_full + 8 * stage;
                             mbar_arrive_expect_tx(bar, Cfg::L0_STAGE_BYTES);
                             tma_load_2d(a_dst, &tmap_x, kb * 128, m0, bar);
@@ -397,7 +405,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 const int n0 = tn * BN + (int)rank * Cfg::BN_CTA;
                 const int eblk = (tm * CG + (int)rank) * kblocks;
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                    if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error)) {
+                    if (!mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error)) {
                         ok = false;
                         break;
                     }
@@ -406,7 +414,8 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     const uint32_t e_dst = sE + stage * Cfg::E_BYTES;
                     // (the W tiles and the byte count of the first npre stages were issued before the wait)
                     const bool pre = wi == 0 && kb - w.kb0 < npre;
-                    if constexpr (CG == 1) {
+                    if (!elect_one()) {
+                        } else if constexpr (CG == 1) {
                         const uint32_t bar = bar_full + 8 * stage;
                         if (!pre) mbar_arrive_expect_tx(bar, Cfg::STAGE_BYTES);
                         tma_load_2d(a_dst, &tmap_a, kb * Cfg::A_BOX_X, m0, bar);
@@ -433,7 +442,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 // low-rank stages: T box in the A slot, L_A box in the first half of the W slot
                 if (w.kb1 == kblocks) {
                     for (int j = 0; j < lora_steps && ok; ++j) {
-                        if (!mbar_wait(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error)) {
+                        if (!mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error)) {
                             ok = false;
                             break;
                         }
@@ -441,15 +450,18 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                             // T rows of this CTA's 128 rows come from phase 0 of this launch: one look at
                             // the count of published groups (once complete, no tile looks again), else
                             // wait for the four ready words of these rows
-                            if (ld_acquire_gpu(p.l0_done) == p.l0_done_target) l0_all_done = true;
-                            else ok = flag_wait4(p.l0_ready + (tm * CG + (int)rank) * 4, p.l0_epoch, cta_abort, p.dev_error);
+                            // (every lane looks, the votes keep the warp together)
+                            if (__all_sync(0xffffffffu, ld_acquire_gpu(p.l0_done) == p.l0_done_target)) l0_all_done = true;
+                            else ok = __all_sync(0xffffffffu, flag_wait4(p.l0_ready + (tm * CG + (int)rank) * 4, p.l0_epoch,
+                                                                         cta_abort, p.dev_error));
                             if (!ok) break;
                             fence_proxy_async_global();
                         }
                         constexpr uint32_t LORA_BYTES = Cfg::A_BYTES + Cfg::B_HALF_BYTES;
                         const uint32_t a_dst = sA + stage * Cfg::A_BYTES;
                         const uint32_t b_dst = sB + stage * Cfg::B_BYTES;
-                        if constexpr (CG == 1) {
+                        if (!elect_one()) {
+                        } else if constexpr (CG == 1) {
                             const uint32_t bar = bar_full + 8 * stage;
                             mbar_arrive_expect_tx(bar, LORA_BYTES);
                             tma_load_2d(a_dst, &tmap_t, j * 64, m0, bar);
@@ -469,7 +481,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer --------
-        if (leader && lane == 0) {
+        if (leader) {
             constexpr uint32_t idesc0 = make_idesc_sp_bf16(Cfg::BM * CG, BN), idesc1 = idesc0 | 1u;
             // descriptor words: low = start address (16-byte units) | LBO, high = SBO | version | swizzle
             const uint64_t d0 = make_desc_sw128(sA);
@@ -489,7 +501,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     const int k1 = (k0 + p.l0_kb_per_split < kblocks) ? k0 + p.l0_kb_per_split : kblocks;
                     const int acc = (Cfg::ACC_STAGES == 2) ? (li & 1) : 0;
                     const uint32_t acc_phase = (Cfg::ACC_STAGES == 2) ? ((li >> 1) & 1) : (li & 1);
-                    if (!mbar_wait(bar_tempty + 8 * acc, acc_phase ^ 1, cta_abort, p.dev_error)) {
+                    if (!mbar_wait_warp(bar_tempty + 8 * acc, acc_phase ^ 1, cta_abort, p.dev_error)) {
                         ok = false;
                         break;
                     }
@@ -497,7 +509,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     const uint32_t d_tmem = tmem_base + acc * BN;
                     uint32_t accumulate = 0;
                     for (int kb = k0; kb < k1; ++kb) {
-                        if (!mbar_wait(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) {
+                        if (!mbar_wait_warp(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) {
                             ok = false;
                             break;
                         }
@@ -506,21 +518,24 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                         const uint32_t b_lo = b_lo0 + stage * (Cfg::B_BYTES >> 4);
                         const uint32_t a2_lo = b_lo + (Cfg::L0_X2_OFF >> 4);
                         const uint32_t b2_lo = b_lo + (Cfg::L0_LB_BYTES >> 4);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            mma_bf16_lh<CG>(d_tmem, a_lo + 2 * i, b_lo + 2 * i, desc_hi, idesc_l0, accumulate);
-                            accumulate = 1u;
+                            for (int i = 0; i < 4; ++i)
+                                mma_bf16_lh<CG>(d_tmem, a_lo + 2 * i, b_lo + 2 * i, desc_hi, idesc_l0, i ? 1u : accumulate);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                mma_bf16_lh<CG>(d_tmem, a2_lo + 2 * i, b2_lo + 2 * i, desc_hi, idesc_l0, 1u);
+                            if constexpr (CG == 1) tc_commit(bar_empty + 8 * stage);
+                            else tc_commit_pair(bar_empty + 8 * stage, 0x3);
                         }
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            mma_bf16_lh<CG>(d_tmem, a2_lo + 2 * i, b2_lo + 2 * i, desc_hi, idesc_l0, 1u);
-                        if constexpr (CG == 1) tc_commit(bar_empty + 8 * stage);
-                        else tc_commit_pair(bar_empty + 8 * stage, 0x3);
+                        accumulate = 1u;
                         if (++stage == STAGES) { stage = 0; phase ^= 1; }
                     }
                     if (!ok) break;
-                    if constexpr (CG == 1) tc_commit(bar_tfull + 8 * acc);
-                    else tc_commit_pair(bar_tfull + 8 * acc, 0x3);
+                    if (elect_one()) {
+                        if constexpr (CG == 1) tc_commit(bar_tfull + 8 * acc);
+                        else tc_commit_pair(bar_tfull + 8 * acc, 0x3);
+                    }
                 }
             }
             int it = 0;
@@ -529,12 +544,12 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 const int gi = l0_n + it;  // accumulator buffers alternate over phase 0 items and tiles alike
                 const int acc = (Cfg::ACC_STAGES == 2) ? (gi & 1) : 0;
                 const uint32_t acc_phase = (Cfg::ACC_STAGES == 2) ? ((gi >> 1) & 1) : (gi & 1);
-                if (!mbar_wait(bar_tempty + 8 * acc, acc_phase ^ 1, cta_abort, p.dev_error)) break;
+                if (!mbar_wait_warp(bar_tempty + 8 * acc, acc_phase ^ 1, cta_abort, p.dev_error)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 uint32_t accumulate = 0;
                 for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                    if (!mbar_wait(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) {
+                    if (!mbar_wait_warp(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) {
                         ok = false;
                         break;
                     }
@@ -542,33 +557,35 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     const uint32_t e_tmem = tmem_base + Cfg::E_COL0 + Cfg::E_COLS * stage;
                     const uint32_t a_lo = a_lo0 + stage * (Cfg::A_BYTES >> 4);
                     const uint32_t b_lo = b_lo0 + stage * (Cfg::B_BYTES >> 4);
-                    tmem_cp_128x128b<CG>(e_tmem, e_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4)));
-                    if constexpr (Cfg::FP8) {
-                        // second 128 x 128 metadata block of the stage, then four K steps of 64 logical
-                        // elements: A advances 32 bytes, W 64 bytes, metadata two columns
-                        tmem_cp_128x128b<CG>(e_tmem + 4, e_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4) + (2048 >> 4)));
-                        constexpr uint32_t idesc8 = make_idesc_sp_e4m3(Cfg::BM * CG, BN);
-                        mma_sp_f8_lh<CG>(d_tmem, a_lo, b_lo, desc_hi, e_tmem, idesc8, accumulate);
-                        mma_sp_f8_lh<CG>(d_tmem, a_lo + 2, b_lo + 4, desc_hi, e_tmem + 2, idesc8, 1u);
-                        mma_sp_f8_lh<CG>(d_tmem, a_lo + 4, b_lo + BH, desc_hi, e_tmem + 4, idesc8, 1u);
-                        mma_sp_f8_lh<CG>(d_tmem, a_lo + 6, b_lo + BH + 4, desc_hi, e_tmem + 6, idesc8, 1u);
-                    } else {
-                        // four K steps of 32 logical elements: A advances 32 bytes, W 64 bytes (steps 2, 3
-                        // in the second 64-element slice); metadata column pair + sparse_id2 = step parity
-                        mma_sp_bf16_lh<CG>(d_tmem, a_lo, b_lo, desc_hi, e_tmem, idesc0, accumulate);
-                        mma_sp_bf16_lh<CG>(d_tmem, a_lo + 2, b_lo + 4, desc_hi, e_tmem, idesc1, 1u);
-                        mma_sp_bf16_lh<CG>(d_tmem, a_lo + 4, b_lo + BH, desc_hi, e_tmem + 2, idesc0, 1u);
-                        mma_sp_bf16_lh<CG>(d_tmem, a_lo + 6, b_lo + BH + 4, desc_hi, e_tmem + 2, idesc1, 1u);
+                    if (elect_one()) {
+                        tmem_cp_128x128b<CG>(e_tmem, e_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4)));
+                        if constexpr (Cfg::FP8) {
+                            // second 128 x 128 metadata block of the stage, then four K steps of 64 logical
+                            // elements: A advances 32 bytes, W 64 bytes, metadata two columns
+                            tmem_cp_128x128b<CG>(e_tmem + 4, e_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4) + (2048 >> 4)));
+                            constexpr uint32_t idesc8 = make_idesc_sp_e4m3(Cfg::BM * CG, BN);
+                            mma_sp_f8_lh<CG>(d_tmem, a_lo, b_lo, desc_hi, e_tmem, idesc8, accumulate);
+                            mma_sp_f8_lh<CG>(d_tmem, a_lo + 2, b_lo + 4, desc_hi, e_tmem + 2, idesc8, 1u);
+                            mma_sp_f8_lh<CG>(d_tmem, a_lo + 4, b_lo + BH, desc_hi, e_tmem + 4, idesc8, 1u);
+                            mma_sp_f8_lh<CG>(d_tmem, a_lo + 6, b_lo + BH + 4, desc_hi, e_tmem + 6, idesc8, 1u);
+                        } else {
+                            // four K steps of 32 logical elements: A advances 32 bytes, W 64 bytes (steps 2, 3
+                            // in the second 64-element slice); metadata column pair + sparse_id2 = step parity
+                            mma_sp_bf16_lh<CG>(d_tmem, a_lo, b_lo, desc_hi, e_tmem, idesc0, accumulate);
+                            mma_sp_bf16_lh<CG>(d_tmem, a_lo + 2, b_lo + 4, desc_hi, e_tmem, idesc1, 1u);
+                            mma_sp_bf16_lh<CG>(d_tmem, a_lo + 4, b_lo + BH, desc_hi, e_tmem + 2, idesc0, 1u);
+                            mma_sp_bf16_lh<CG>(d_tmem, a_lo + 6, b_lo + BH + 4, desc_hi, e_tmem + 2, idesc1, 1u);
+                        }
+                        if constexpr (CG == 1) tc_commit(bar_empty + 8 * stage);
+                        else tc_commit_pair(bar_empty + 8 * stage, 0x3);
                     }
                     accumulate = 1u;
-                    if constexpr (CG == 1) tc_commit(bar_empty + 8 * stage);
-                    else tc_commit_pair(bar_empty + 8 * stage, 0x3);
                     if (++stage == STAGES) { stage = 0; phase ^= 1; }
                 }
                 if (ok && w.kb1 == kblocks) {
                     constexpr uint32_t idesc_dense = idesc0 & ~(1u << 2);
                     for (int j = 0; j < lora_steps; ++j) {
-                        if (!mbar_wait(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) {
+                        if (!mbar_wait_warp(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) {
                             ok = false;
                             break;
                         }
@@ -576,19 +593,23 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                         const uint32_t a_lo = a_lo0 + stage * (Cfg::A_BYTES >> 4);
                         const uint32_t b_lo = b_lo0 + stage * (Cfg::B_BYTES >> 4);
                         // dense K steps of 16 elements: both operands advance 32 bytes
-                        mma_bf16_lh<CG>(d_tmem, a_lo, b_lo, desc_hi, idesc_dense, accumulate);
-                        mma_bf16_lh<CG>(d_tmem, a_lo + 2, b_lo + 2, desc_hi, idesc_dense, 1u);
-                        mma_bf16_lh<CG>(d_tmem, a_lo + 4, b_lo + 4, desc_hi, idesc_dense, 1u);
-                        mma_bf16_lh<CG>(d_tmem, a_lo + 6, b_lo + 6, desc_hi, idesc_dense, 1u);
+                        if (elect_one()) {
+                            mma_bf16_lh<CG>(d_tmem, a_lo, b_lo, desc_hi, idesc_dense, accumulate);
+                            mma_bf16_lh<CG>(d_tmem, a_lo + 2, b_lo + 2, desc_hi, idesc_dense, 1u);
+                            mma_bf16_lh<CG>(d_tmem, a_lo + 4, b_lo + 4, desc_hi, idesc_dense, 1u);
+                            mma_bf16_lh<CG>(d_tmem, a_lo + 6, b_lo + 6, desc_hi, idesc_dense, 1u);
+                            if constexpr (CG == 1) tc_commit(bar_empty + 8 * stage);
+                            else tc_commit_pair(bar_empty + 8 * stage, 0x3);
+                        }
                         accumulate = 1u;
-                        if constexpr (CG == 1) tc_commit(bar_empty + 8 * stage);
-                        else tc_commit_pair(bar_empty + 8 * stage, 0x3);
                         if (++stage == STAGES) { stage = 0; phase ^= 1; }
                     }
                 }
                 if (!ok) break;
-                if constexpr (CG == 1) tc_commit(bar_tfull + 8 * acc);
-                else tc_commit_pair(bar_tfull + 8 * acc, 0x3);
+                if (elect_one()) {
+                    if constexpr (CG == 1) tc_commit(bar_tfull + 8 * acc);
+                    else tc_commit_pair(bar_tfull + 8 * acc, 0x3);
+                }
             }
         }
     } else {

@@ -181,7 +181,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + (sBar - smem_base) + 8 * Cfg::NUM_BARS);
     volatile uint32_t* cta_abort = tmem_slot + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
     const int cluster_id = blockIdx.x / 2;
@@ -221,11 +221,11 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     __syncthreads();
     cluster_sync_all();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     // W tiles of the first stages of the first item, before the wait for the previous kernel (W is
     // not its output in a layer call); the producer below skips them
     int npre = 0;
-    if (warp == 0 && lane == 0 && p.w_prefetch && num_items > 0) {
+    if (warp == 0 && p.w_prefetch && num_items > 0) {
         int tm0, tn, rows, ordinal;
         sched.item(cluster_id, 0, tm0, tn, rows, ordinal);
         const bool r1 = rows == 1;
@@ -235,7 +235,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         const uint32_t full0 = mapa(bfull, 0);
         const int n0 = tn * BN + (int)rank * Cfg::BN_CTA;
         const uint32_t tx = r1 ? (uint32_t)Cfg::SINGLE_TX : (uint32_t)Cfg::STAGE_BYTES;
-        for (int s = 0; s < npre; ++s) {
+        if (elect_one()) for (int s = 0; s < npre; ++s) {
             const uint32_t b_dst = r1 ? sA + Cfg::RING1_B + s * Cfg::B_BYTES : sB + s * Cfg::B_BYTES;
             if (leader) mbar_arrive_expect_tx(bfull + 8 * s, 2 * tx);
             tma_load_2d_pair(b_dst, &tmap_b, s * Cfg::BK, n0, full0 + 8 * s);
@@ -247,7 +247,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer ----------
-        if (lane == 0) {
+        {
             uint32_t stage = 0, phase = 0, issued = 0;
             bool ok = true;
             bool ring1 = false;  // false: the 3 x 66 KB ring of the doubles, true: the 4 x 48 KB ring of the singles
@@ -259,7 +259,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     // ring has to be released first (the stages below `stage` were last used in this
                     // round of the ring, the others in the round before; a fresh barrier passes).
                     for (int s = 0; s < STAGES && ok; ++s)
-                        ok = mbar_wait(bar_empty + 8 * s, ((uint32_t)s < stage) ? phase : (phase ^ 1u), cta_abort, p.dev_error);
+                        ok = mbar_wait_warp(bar_empty + 8 * s, ((uint32_t)s < stage) ? phase : (phase ^ 1u), cta_abort, p.dev_error);
                     if (!ok) break;
                     ring1 = true;
                     stage = 0;
@@ -272,7 +272,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                 const int n0 = tn * BN + (int)rank * Cfg::BN_CTA;
                 const uint32_t tx = (rows == 2) ? (uint32_t)Cfg::STAGE_BYTES : (uint32_t)Cfg::SINGLE_TX;
                 for (int kb = 0; kb < kblocks + lora_steps; ++kb) {
-                    if (!mbar_wait(bempty + 8 * stage, phase ^ 1, cta_abort, p.dev_error)) {
+                    if (!mbar_wait_warp(bempty + 8 * stage, phase ^ 1, cta_abort, p.dev_error)) {
                         ok = false;
                         break;
                     }
@@ -280,7 +280,8 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     const uint32_t b_dst = ring1 ? sA + Cfg::RING1_B + stage * Cfg::B_BYTES : sB + stage * Cfg::B_BYTES;
                     const uint32_t e_dst = ring1 ? sA + Cfg::RING1_E + stage * Cfg::E_BYTES : sE + stage * 2 * Cfg::E_BYTES;
                     const uint32_t bar = full0 + 8 * stage;
-                    if (kb < kblocks) {
+                    if (!elect_one()) {
+                    } else if (kb < kblocks) {
                         const bool pre = it == 0 && kb < npre;  // W tile and byte count went out before the wait
                         // the leader announces the bytes of both CTAs; the peer's bytes may land first
                         if (leader && !pre) mbar_arrive_expect_tx(bfull + 8 * stage, 2 * tx);
@@ -310,7 +311,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer --------
-        if (leader && lane == 0) {
+        if (leader) {
             constexpr uint32_t idesc0 = make_idesc_sp_bf16(Cfg::BM * 2, BN), idesc1 = idesc0 | 1u;
             constexpr uint32_t idesc_dense = idesc0 & ~(1u << 2);
             const uint64_t d0 = make_desc_sw128(sA);
@@ -337,14 +338,14 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                 const int acc0 = (rows == 2) ? 0 : (ordinal & 1);
                 for (int r = 0; r < rows && ok; ++r) {
                     const int a = acc0 + r;
-                    ok = mbar_wait(bar_tempty + 8 * a, (uses[a] & 1u) ^ 1u, cta_abort, p.dev_error);
+                    ok = mbar_wait_warp(bar_tempty + 8 * a, (uses[a] & 1u) ^ 1u, cta_abort, p.dev_error);
                 }
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc0 * BN;
                 uint32_t accumulate = 0;
                 for (int kb = 0; kb < kblocks + lora_steps; ++kb) {
-                    if (!mbar_wait(bfull + 8 * stage, phase, cta_abort, p.dev_error)) {
+                    if (!mbar_wait_warp(bfull + 8 * stage, phase, cta_abort, p.dev_error)) {
                         ok = false;
                         break;
                     }
@@ -353,42 +354,44 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                                                 : ring_lo0 + stage * (2 * Cfg::A_BYTES >> 4);
                     const uint32_t b_lo = ring1 ? ring_lo0 + ((Cfg::RING1_B + stage * Cfg::B_BYTES) >> 4)
                                                 : b_lo0 + stage * (Cfg::B_BYTES >> 4);
-                    if (kb < kblocks) {
-                        const uint32_t e_tmem = tmem_base + Cfg::E_COL0 + (ring1 ? 4 * stage : Cfg::E_COLS * stage);
-                        const uint64_t e_desc = ring1 ? e1_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4))
-                                                      : e_d0 + (uint64_t)(stage * (2 * Cfg::E_BYTES >> 4));
-                        tmem_cp_128x128b<2>(e_tmem, e_desc);
-                        if (rows == 2) tmem_cp_128x128b<2>(e_tmem + 4, e_desc + (uint64_t)(Cfg::E_BYTES >> 4));
-                        // four K steps of 32 logical elements per row tile: A advances 32 bytes, W 64 bytes
-                        // (steps 2, 3 in the second 64-element slice); metadata column pair + step parity
-                        mma_sp_bf16_lh<2>(d_tmem, a_lo, b_lo, desc_hi, e_tmem, idesc0, accumulate);
-                        mma_sp_bf16_lh<2>(d_tmem, a_lo + 2, b_lo + 4, desc_hi, e_tmem, idesc1, 1u);
-                        mma_sp_bf16_lh<2>(d_tmem, a_lo + 4, b_lo + BH, desc_hi, e_tmem + 2, idesc0, 1u);
-                        mma_sp_bf16_lh<2>(d_tmem, a_lo + 6, b_lo + BH + 4, desc_hi, e_tmem + 2, idesc1, 1u);
-                        if (rows == 2) {
-                            constexpr uint32_t A1 = Cfg::A_BYTES >> 4;
-                            mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1, b_lo, desc_hi, e_tmem + 4, idesc0, accumulate);
-                            mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 2, b_lo + 4, desc_hi, e_tmem + 4, idesc1, 1u);
-                            mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 4, b_lo + BH, desc_hi, e_tmem + 6, idesc0, 1u);
-                            mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 6, b_lo + BH + 4, desc_hi, e_tmem + 6, idesc1, 1u);
+                    if (elect_one()) {
+                        if (kb < kblocks) {
+                            const uint32_t e_tmem = tmem_base + Cfg::E_COL0 + (ring1 ? 4 * stage : Cfg::E_COLS * stage);
+                            const uint64_t e_desc = ring1 ? e1_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4))
+                                                          : e_d0 + (uint64_t)(stage * (2 * Cfg::E_BYTES >> 4));
+                            tmem_cp_128x128b<2>(e_tmem, e_desc);
+                            if (rows == 2) tmem_cp_128x128b<2>(e_tmem + 4, e_desc + (uint64_t)(Cfg::E_BYTES >> 4));
+                            // four K steps of 32 logical elements per row tile: A advances 32 bytes, W 64 bytes
+                            // (steps 2, 3 in the second 64-element slice); metadata column pair + step parity
+                            mma_sp_bf16_lh<2>(d_tmem, a_lo, b_lo, desc_hi, e_tmem, idesc0, accumulate);
+                            mma_sp_bf16_lh<2>(d_tmem, a_lo + 2, b_lo + 4, desc_hi, e_tmem, idesc1, 1u);
+                            mma_sp_bf16_lh<2>(d_tmem, a_lo + 4, b_lo + BH, desc_hi, e_tmem + 2, idesc0, 1u);
+                            mma_sp_bf16_lh<2>(d_tmem, a_lo + 6, b_lo + BH + 4, desc_hi, e_tmem + 2, idesc1, 1u);
+                            if (rows == 2) {
+                                constexpr uint32_t A1 = Cfg::A_BYTES >> 4;
+                                mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1, b_lo, desc_hi, e_tmem + 4, idesc0, accumulate);
+                                mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 2, b_lo + 4, desc_hi, e_tmem + 4, idesc1, 1u);
+                                mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 4, b_lo + BH, desc_hi, e_tmem + 6, idesc0, 1u);
+                                mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 6, b_lo + BH + 4, desc_hi, e_tmem + 6, idesc1, 1u);
+                            }
+                        } else {
+                            // low-rank stage: dense K steps of 16 elements, both operands advance 32 bytes
+                            for (int r = 0; r < rows; ++r) {
+                                const uint32_t dt = d_tmem + r * BN, al = a_lo + r * (Cfg::A_BYTES >> 4);
+                                mma_bf16_lh<2>(dt, al, b_lo, desc_hi, idesc_dense, accumulate);
+                                mma_bf16_lh<2>(dt, al + 2, b_lo + 2, desc_hi, idesc_dense, 1u);
+                                mma_bf16_lh<2>(dt, al + 4, b_lo + 4, desc_hi, idesc_dense, 1u);
+                                mma_bf16_lh<2>(dt, al + 6, b_lo + 6, desc_hi, idesc_dense, 1u);
+                            }
                         }
-                    } else {
-                        // low-rank stage: dense K steps of 16 elements, both operands advance 32 bytes
-                        for (int r = 0; r < rows; ++r) {
-                            const uint32_t dt = d_tmem + r * BN, al = a_lo + r * (Cfg::A_BYTES >> 4);
-                            mma_bf16_lh<2>(dt, al, b_lo, desc_hi, idesc_dense, accumulate);
-                            mma_bf16_lh<2>(dt, al + 2, b_lo + 2, desc_hi, idesc_dense, 1u);
-                            mma_bf16_lh<2>(dt, al + 4, b_lo + 4, desc_hi, idesc_dense, 1u);
-                            mma_bf16_lh<2>(dt, al + 6, b_lo + 6, desc_hi, idesc_dense, 1u);
-                        }
+                        tc_commit_pair(bempty + 8 * stage, 0x3);
                     }
                     accumulate = 1u;
-                    tc_commit_pair(bempty + 8 * stage, 0x3);
                     if (++stage == nst) { stage = 0; phase ^= 1; }
                 }
                 if (!ok) break;
                 for (int r = 0; r < rows; ++r) {
-                    tc_commit_pair(bar_tfull + 8 * (acc0 + r), 0x3);
+                    if (elect_one()) tc_commit_pair(bar_tfull + 8 * (acc0 + r), 0x3);
                     ++uses[acc0 + r];
                 }
             }
