@@ -1,0 +1,136 @@
+// Epilogue pieces shared by the two sparse GEMM kernels: accumulator chunk -> scale, bias, residual ->
+// packed bf16 registers -> staging box -> TMA store.
+//
+// What bounds it.  A launch's last tile has nothing left to hide its epilogue behind, and the 512-row
+// items of the two-row-tile kernel hold both accumulators until theirs are read.  With four warps per
+// tile, a shuffle per bias value and one staging box per warp, the epilogue of a 128 x 192 tile took
+// 5300 cycles on an idle GPU and 8100 with every SM storing (13500 with a residual, whose loads were
+// fetched chunk by chunk).  Hence: eight warps per tile (two per tensor-memory lane quarter); all chunks of
+// a warp converted to packed bf16 registers before the first is stored (the accumulator goes back
+// after the tensor-memory reads); packed fp32 multiply-adds; the residual fetched into the output registers
+// during the main loop and replaced there; and for the last item a staging box per chunk in the ring's
+// memory, which nothing uses any more, so that no store waits for another.
+//
+// Layout.  The accumulators are read in the 16 x 256-bit shape: of a 16-row x 8-column block lane t holds rows
+// t / 4 and t / 4 + 8, columns 2 (t % 4) and + 1.  A lane then needs two bias values per eight columns
+// for its four rows; in the row-per-lane shape every lane needs every column's value, and those broadcast
+// loads alone occupied the shared memory for 1900 cycles per 512 x 240 item.  The blocks go to the
+// staging box with stmatrix.
+#pragma once
+
+#include "ptx.cuh"
+
+namespace lynx {
+
+constexpr int GEMM_EPI_WARPS = 8;
+constexpr int GEMM_EPI_WARP0 = 4;         // first epilogue warp: the producer, the issuer and two idle warps come before
+constexpr uint32_t GEMM_EPI_BARRIER = 1;  // named barrier of the epilogue warps
+constexpr int GEMM_THREADS = 32 * (GEMM_EPI_WARP0 + GEMM_EPI_WARPS);
+// Register shares (per thread) of the two kinds of warpgroups; 128 * 72 + 256 * 216 = the 384 * 168 the block is
+// launched with.  An epilogue warp holds up to five packed chunks beside the one it converts.
+constexpr int GEMM_REGS_ISSUE = 72, GEMM_REGS_EPI = 216;
+static_assert(128 * GEMM_REGS_ISSUE + 32 * GEMM_EPI_WARPS * GEMM_REGS_EPI <= GEMM_THREADS * 168, "register pool of the block");
+
+// One 32-row x CH-column chunk: v[half][4 g + 2 k + e] = row 16 half + 8 k + lane / 4, column 8 g + 2 (lane % 4) + e
+template <int CH>
+__device__ __forceinline__ void epi_tmem_ld(uint32_t taddr, uint32_t (&v)[2][CH / 2]) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+        const uint32_t t = taddr + ((uint32_t)(16 * half) << 16);
+        if constexpr (CH == 64) {
+            tmem_ld_16x256b_x8(t, v[half]);
+        } else {
+            tmem_ld_16x256b_x4(t, *reinterpret_cast<uint32_t(*)[16]>(&v[half][0]));
+            tmem_ld_16x256b_x2(t + 32, *reinterpret_cast<uint32_t(*)[8]>(&v[half][16]));
+        }
+    }
+}
+
+// The chunk's residual values in the layout of the packed results (columns past N and rows past M: zero)
+template <int CH>
+__device__ __forceinline__ void epi_load_residual(const uint16_t* residual, int64_t ldr, int64_t row0, int64_t M, int n0, int64_t N,
+                                                  int lane, uint32_t (&out)[2][CH / 4]) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int64_t row = row0 + 16 * half + 8 * k + (lane >> 2);
+            const uint16_t* src = residual + row * ldr + n0 + 2 * (lane & 3);
+#pragma unroll
+            for (int g = 0; g < CH / 8; ++g)
+                out[half][2 * g + k] = (row < M && n0 + 8 * g < N) ? __ldg(reinterpret_cast<const uint32_t*>(src + 8 * g)) : 0u;
+        }
+}
+
+// out[half][2 g + k] = bf16(fma(s [* col_scale], v, bias) [+ the residual that `out` holds]); s[2 half + k]: the
+// lane's rows' scales; sb / sc: shared-memory addresses of the chunk's fp32 bias values and weight scales.
+template <int CH, bool COL_SCALE, bool RES>
+__device__ __forceinline__ void epi_convert(const uint32_t (&v)[2][CH / 2], const float (&s)[4], uint32_t sb, uint32_t sc, int lane,
+                                            uint32_t (&out)[2][CH / 4]) {
+    const uint32_t col = 8 * (lane & 3);
+#pragma unroll
+    for (int g = 0; g < CH / 8; ++g) {
+        const uint64_t b = lds64(sb + g * 32 + col);
+        uint64_t c = 0;
+        if constexpr (COL_SCALE) c = lds64(sc + g * 32 + col);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int half = i >> 1, k = i & 1;
+            uint64_t m = pack_f32x2(s[i], s[i]);
+            if constexpr (COL_SCALE) m = mul_f32x2(m, c);
+            uint64_t y = fma_f32x2(m, pack_b32x2(v[half][4 * g + 2 * k], v[half][4 * g + 2 * k + 1]), b);
+            if constexpr (RES) {
+                const uint32_t r = out[half][2 * g + k];
+                y = add_f32x2(y, pack_f32x2(bf16_lo_f(r), bf16_hi_f(r)));
+            }
+            out[half][2 * g + k] = pack_bf16x2_of(y);
+        }
+    }
+}
+
+// One chunk to the output through a staging box of shared memory (64-column boxes: 128-byte rows with the
+// 128-byte swizzle; 48: dense 96-byte rows).  BOX_ROWS: rows of the tensor map's box and of the warp's own box.
+// fresh: `box` holds 32 rows and nothing has used it; else it is the warp's own, whose previous store must have read it.
+template <int CH, int BOX_ROWS>
+__device__ __forceinline__ void epi_store(const CUtensorMap* tmap, const uint32_t (&o)[2][CH / 4], int n0, int m0, uint32_t box,
+                                          bool fresh, int lane) {
+    constexpr int ROW_BYTES = CH * 2;
+    // lane l addresses row l % 8 of 8 x 8 matrix l / 8: rows 0-7 and 8-15 of column group g, then of g + 1
+    const uint32_t r = (lane & 7) + (lane & 8), gl = lane >> 4;
+    auto put = [&](const uint32_t (&h)[CH / 4], uint32_t base) {
+#pragma unroll
+        for (int g = 0; g < CH / 8; g += 2)
+            stmatrix_x4(base + r * ROW_BYTES + ((CH == 64 ? ((g + gl) ^ (r & 7)) : (g + gl)) << 4), h[2 * g], h[2 * g + 1], h[2 * g + 2],
+                        h[2 * g + 3]);
+    };
+    if (fresh || BOX_ROWS == 32) {
+        if (!fresh) {
+            if (lane == 0) tma_store_wait_read<0>();
+            __syncwarp();
+        }
+        put(o[0], box);
+        put(o[1], box + 16 * ROW_BYTES);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+#pragma unroll
+            for (int i = 0; i < 32; i += BOX_ROWS) tma_store_2d(tmap, n0, m0 + i, box + i * ROW_BYTES);
+            tma_store_commit();
+        }
+        return;
+    }
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {  // 16-row boxes
+        if (lane == 0) tma_store_wait_read<0>();
+        __syncwarp();
+        put(o[half], box);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_2d(tmap, n0, m0 + 16 * half, box);
+            tma_store_commit();
+        }
+    }
+}
+
+}  // namespace lynx

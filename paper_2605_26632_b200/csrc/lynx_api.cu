@@ -323,7 +323,7 @@ lynx_status launch_gemm_cfg(lynx_ctx* ctx, const void* values, const void* meta,
         !make_tmap_2d(ctx, &te, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, meta, rb * kblocks * 2, 256, 1024, 256, 2,
                       CU_TENSOR_MAP_SWIZZLE_NONE) ||
         !make_tmap_2d(ctx, &ty, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, (uint64_t)M, (uint64_t)N, (uint64_t)ldy * 2, Cfg::CH,
-                      32, Cfg::CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE))
+                      Cfg::BOX_ROWS, Cfg::CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE))
         return LYNX_ERR_CUDA;
     if (lora) {
         if (!make_tmap_2d(ctx, &tt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->T, (uint64_t)M, (uint64_t)lora->R,
@@ -603,14 +603,14 @@ lynx_status launch_gemm(lynx_ctx* ctx, const void* values, const void* meta, int
     if (cfg == 0) cfg = pick_gemm_cfg(ctx, M, N, K, lora_steps);
 #define LYNX_GEMM_ARGS ctx, values, meta, M, K, W, N, ldw, bias, comp, lora, Y, ldy, st, ss, layer_call
     switch (cfg) {
-        case 1: return launch_gemm_cfg<GemmCfg<128, 1, 4, 1>>(LYNX_GEMM_ARGS);
-        case 2: return launch_gemm_cfg<GemmCfg<192, 1, 3, 1>>(LYNX_GEMM_ARGS);
-        case 3: return launch_gemm_cfg<GemmCfg<256, 1, 2, 1>>(LYNX_GEMM_ARGS);
-        case 4: return launch_gemm_cfg<GemmCfg<192, 2, 4, 2>>(LYNX_GEMM_ARGS);
-        case 5: return launch_gemm_cfg<GemmCfg<256, 2, 4, 1>>(LYNX_GEMM_ARGS);
-        case 6: return launch_gemm_cfg<GemmCfg<128, 2, 5, 2>>(LYNX_GEMM_ARGS);
-        case 7: return launch_gemm_cfg<GemmCfg<240, 2, 4, 2>>(LYNX_GEMM_ARGS);
-        case 8: return launch_gemm_cfg<GemmCfg<192, 2, 5, 1, false, 48>>(LYNX_GEMM_ARGS);  // five stages: one-round launches
+        case 1: return launch_gemm_cfg<GemmCfg<128, 1, 4, 16>>(LYNX_GEMM_ARGS);
+        case 2: return launch_gemm_cfg<GemmCfg<192, 1, 3, 16>>(LYNX_GEMM_ARGS);
+        case 3: return launch_gemm_cfg<GemmCfg<256, 1, 2, 32>>(LYNX_GEMM_ARGS);
+        case 4: return launch_gemm_cfg<GemmCfg<192, 2, 4, 32>>(LYNX_GEMM_ARGS);
+        case 5: return launch_gemm_cfg<GemmCfg<256, 2, 4, 16>>(LYNX_GEMM_ARGS);
+        case 6: return launch_gemm_cfg<GemmCfg<128, 2, 5, 32>>(LYNX_GEMM_ARGS);
+        case 7: return launch_gemm_cfg<GemmCfg<240, 2, 4, 32>>(LYNX_GEMM_ARGS);
+        case 8: return launch_gemm_cfg<GemmCfg<192, 2, 5, 16, false, 48>>(LYNX_GEMM_ARGS);  // five stages: one-round launches
         default: return LYNX_ERR_INVALID_ARG;
     }
 #undef LYNX_GEMM_ARGS
@@ -631,7 +631,7 @@ lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void*
         !make_tmap_2d(ctx, &te, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, meta, rb * kb128 * 2, 256, 1024, 256,
                       Cfg::E_BYTES / 1024, CU_TENSOR_MAP_SWIZZLE_NONE) ||
         !make_tmap_2d(ctx, &ty, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, (uint64_t)M, (uint64_t)N, (uint64_t)ldy * 2, Cfg::CH,
-                      32, Cfg::CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE))
+                      Cfg::BOX_ROWS, Cfg::CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE))
         return LYNX_ERR_CUDA;
     GemmParams p = {};
     p.M = M; p.N = N; p.K = K;
@@ -683,9 +683,9 @@ lynx_status launch_gemm_fp8(lynx_ctx* ctx, const void* values_q, const void* met
     }
 #define LYNX_FP8_ARGS ctx, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, Y, ldy, st
     switch (cfg) {
-        case 4: return launch_gemm_fp8_cfg<GemmCfg<192, 2, 4, 2, true>>(LYNX_FP8_ARGS);
-        case 6: return launch_gemm_fp8_cfg<GemmCfg<128, 2, 5, 2, true>>(LYNX_FP8_ARGS);
-        default: return launch_gemm_fp8_cfg<GemmCfg<240, 2, 4, 2, true>>(LYNX_FP8_ARGS);
+        case 4: return launch_gemm_fp8_cfg<GemmCfg<192, 2, 4, 32, true>>(LYNX_FP8_ARGS);
+        case 6: return launch_gemm_fp8_cfg<GemmCfg<128, 2, 5, 32, true>>(LYNX_FP8_ARGS);
+        default: return launch_gemm_fp8_cfg<GemmCfg<240, 2, 4, 16, true>>(LYNX_FP8_ARGS);
     }
 #undef LYNX_FP8_ARGS
 }

@@ -44,6 +44,9 @@
 // cta_group::2 MMAs, and each CTA drains its own 128 accumulator rows.
 #pragma once
 
+#include <type_traits>
+
+#include "epilogue.cuh"
 #include "ptx.cuh"
 #include "prune_compress.cuh"  // row_scale_from_partials
 
@@ -190,9 +193,10 @@ struct L0Schedule {
 // (a 128-byte swizzled row of compressed A is then 256 logical K instead of 128, a 128-byte row of
 // W 128 K instead of 64), the metadata of a stage doubles (two 128 x 128 blocks), and the four MMAs
 // of a stage are kind::f8f6f4 with K = 64 each.
-template <int BN_, int CG_, int STAGES_, int CBUFS_, bool FP8_ = false, int CH_ = 0>
+// BOX_ROWS: rows of an epilogue warp's own staging box (16 where the ring leaves no room for 32).
+template <int BN_, int CG_, int STAGES_, int BOX_ROWS_, bool FP8_ = false, int CH_ = 0>
 struct GemmCfg {
-    static constexpr int BN = BN_, CG = CG_, STAGES = STAGES_, CBUFS = CBUFS_;
+    static constexpr int BN = BN_, CG = CG_, STAGES = STAGES_, BOX_ROWS = BOX_ROWS_;
     static constexpr bool FP8 = FP8_;
     static constexpr int BM = 128;  // rows per CTA
     static constexpr int BK = FP8 ? 256 : 128;  // logical K per stage
@@ -209,24 +213,22 @@ struct GemmCfg {
     // (96-byte unswizzled rows) -- BN = 240 is the widest tile that leaves room for two
     // accumulator buffers plus the metadata columns in the 512 columns of tensor memory
     static constexpr int CH = CH_ ? CH_ : ((BN % 64 == 0) ? 64 : 48);  // (CH_: narrower staging boxes where shared memory is short)
-    static constexpr int C_BOX_BYTES = 32 * CH * 2;  // one warp's 32 x CH bf16 store box
-    static constexpr int C_BYTES = 4 * CBUFS * C_BOX_BYTES;
+    static constexpr int NCH = BN / CH;              // chunks of a tile, dealt to the two warps of a lane quarter:
+    static constexpr int SLOTS = (NCH + 1) / 2;      // the first takes SLOTS of them, the second the rest
+    static constexpr int EPI_WARPS = GEMM_EPI_WARPS;
+    static constexpr int BOX_BYTES = BOX_ROWS * CH * 2;
+    static constexpr int C_BYTES = EPI_WARPS * BOX_BYTES;
+    static constexpr int STRIP_BYTES = BN * 4 * (FP8 ? 2 : 1);  // a tile's bias (and weight scales) as fp32
     static constexpr int ACC_STAGES = (2 * BN + E_COLS * STAGES <= 512) ? 2 : 1;
     static constexpr int E_COL0 = ACC_STAGES * BN;  // metadata columns start after accumulators
     static constexpr int TMEM_COLS = 512;
     static constexpr int NUM_BARS = 2 * STAGES + 2 * ACC_STAGES;
-    static constexpr int SMEM_BYTES = 1024 /*align slack*/ + STAGES * STAGE_BYTES + C_BYTES + 256;
-    // Epilogue warps: four (one per tensor-memory lane quarter), or eight for FP8 -- two per quarter
-    // that take alternate column chunks, each with one staging box.  A tile's epilogue takes ~6 us
-    // with four warps, which an FP8 main loop at K = 3072 (6.5 us) no longer hides.
-    static constexpr int EPI_WARPS = FP8 ? 8 : 4;
-    static constexpr int EPI_SPLIT = EPI_WARPS / 4;          // warps per lane quarter
-    static constexpr int CBUFS_W = 4 * CBUFS / EPI_WARPS;    // staging boxes per epilogue warp
-    static constexpr int THREADS = 64 + 32 * EPI_WARPS;
-    static_assert(CBUFS_W >= 1, "every epilogue warp needs a staging box");
+    static constexpr int SMEM_BYTES = 1024 /*align slack*/ + STAGES * STAGE_BYTES + C_BYTES + 2 * STRIP_BYTES + 256;
+    static constexpr int THREADS = GEMM_THREADS;
     static_assert(BN % 16 == 0 && (BN / CG) % 8 == 0 && BN <= 256, "tile N");
     static_assert(BN % CH == 0, "epilogue works on whole chunks");
-    static_assert(C_BOX_BYTES % 1024 == 0, "staging boxes stay 1024-byte aligned");
+    static_assert(CH == 48 || BOX_BYTES % 1024 == 0, "swizzled staging boxes stay 1024-byte aligned");
+    static_assert(EPI_WARPS * SLOTS * 32 * CH * 2 <= STAGES * STAGE_BYTES, "last tile: a staging box per chunk in the ring");
     static_assert(B_HALF_BYTES % 1024 == 0, "swizzle atoms need 1024-byte aligned tiles");
     static_assert(E_COL0 % 4 == 0 && E_COL0 + E_COLS * STAGES <= TMEM_COLS, "tensor memory budget");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
@@ -273,7 +275,8 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
     const uint32_t sB = sA + STAGES * Cfg::A_BYTES;
     const uint32_t sE = sB + STAGES * Cfg::B_BYTES;
     const uint32_t sC = sE + STAGES * Cfg::E_BYTES;
-    const uint32_t sBar = sC + Cfg::C_BYTES;
+    const uint32_t sStrip = sC + Cfg::C_BYTES;  // [item parity] STRIP_BYTES
+    const uint32_t sBar = sStrip + 2 * Cfg::STRIP_BYTES;
     const uint32_t bar_full = sBar, bar_empty = sBar + 8 * STAGES;
     const uint32_t bar_tfull = sBar + 16 * STAGES, bar_tempty = bar_tfull + 8 * Cfg::ACC_STAGES;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + (sBar - smem_base) + 8 * Cfg::NUM_BARS);
@@ -322,7 +325,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
     }
     tc_fence_before();
     __syncthreads();
-    if constexpr (CG == 2) cluster_sync_all();
+    if constexpr (CG == 2) cluster_sync_relaxed();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     // W tiles of the first stages of the first tile, before the wait for the previous kernel
@@ -351,6 +354,8 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
     // everything above overlapped the previous kernel's tail; its results are needed from here on
     griddep_wait();
 
+    if (warp < GEMM_EPI_WARP0) {
+    setmaxnreg_dec<GEMM_REGS_ISSUE>();
     if (warp == 0) {
         // ------------------------------------------------------------------ producer ----------
         {
@@ -612,16 +617,18 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 }
             }
         }
+    }
     } else {
+        setmaxnreg_inc<GEMM_REGS_EPI>();
         // ------------------------------------------------------------------ epilogue ----------
         const int q = warp & 3;  // tensor-memory lane quarter this warp may read
-        const uint32_t cbuf0 = sC + (warp - 2) * Cfg::CBUFS_W * Cfg::C_BOX_BYTES;
-        const int c_first = (warp - 2) >> 2;  // with two warps per quarter: even or odd chunks
+        const int h = (warp - GEMM_EPI_WARP0) >> 2;  // which of the quarter's two warps
+        const uint32_t own_box = sC + (warp - GEMM_EPI_WARP0) * Cfg::BOX_BYTES;
         const uint32_t tempty0 = (CG == 2) ? mapa(bar_tempty, 0) : bar_tempty;
-        int it = 0, cb = 0;
         bool alive = true;
         if constexpr (L0) {
-            // ---- phase 0: drain the 64-column accumulator of each (row block, K split) item ----
+            // ---- phase 0: drain the 64-column accumulator of each (row block, K split) item (the first
+            //      four warps; the others only hand the accumulator back) ----
             constexpr int PIECES = Cfg::L0_R / 4;  // float4 pieces per row
             constexpr int BLOCK_ROWS = Cfg::BM * CG;
             for (int li = 0; li < l0_n && alive; ++li) {
@@ -634,7 +641,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 // the row's scale is fetched while the item's K loop runs (a global load costs over a
                 // microsecond once the main loops saturate the memory system); T = acc * (1 / s)
                 float inv_s = 1.0f;
-                if (row < p.M && (p.scale_partial != nullptr || p.row_scale != nullptr)) {
+                if (h == 0 && row < p.M && (p.scale_partial != nullptr || p.row_scale != nullptr)) {
                     const float sc = (p.scale_partial != nullptr) ? row_scale_from_partials(p.scale_partial, row, p.scale_ks)
                                                                   : __ldg(p.row_scale + row);
                     inv_s = (sc == 0.0f) ? 0.0f : __frcp_rn(sc);
@@ -644,6 +651,15 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     break;
                 }
                 tc_fence_after();
+                if (h != 0) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if constexpr (CG == 1) mbar_arrive(bar_tempty + 8 * acc);
+                        else mbar_arrive_cluster(tempty0 + 8 * acc);
+                    }
+                    continue;
+                }
                 const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN;
                 uint32_t v[64];
                 tmem_ld_32x32b_x32(t_row, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
@@ -723,188 +739,141 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 }
             }
         }
-        for (; it < num_items && alive; ++it) {
+        constexpr int CH = Cfg::CH, SLOTS = Cfg::SLOTS;
+        const int slots = h == 0 ? SLOTS : Cfg::NCH - SLOTS, c0 = h == 0 ? 0 : SLOTS;  // this warp's chunks
+        for (int it = 0; it < num_items; ++it) {
             const WorkItem w = sched.get(cluster_id, it);
             int tm, tn;
             tile_coords(w.tile, p.tiles_m, p.tiles_n, p.group_m, tm, tn);
+            const bool last = it == num_items - 1;
             const int gi = l0_n + it;
             const int acc = (Cfg::ACC_STAGES == 2) ? (gi & 1) : 0;
             const uint32_t acc_phase = (Cfg::ACC_STAGES == 2) ? ((gi >> 1) & 1) : (gi & 1);
+            // the tile's per-column terms as fp32, for all epilogue warps (the other parity's may still be read)
+            const uint32_t sb = sStrip + (it & 1) * Cfg::STRIP_BYTES, sc = sb + BN * 4;
+            if (const int c = (int)threadIdx.x - 32 * GEMM_EPI_WARP0; c < BN) {
+                const int n = tn * BN + c;
+                sts32f(sb + c * 4, (p.bias != nullptr && n < p.N) ? __uint_as_float((uint32_t)__ldg(p.bias + n) << 16) : 0.0f);
+                if constexpr (Cfg::FP8) sts32f(sc + c * 4, (p.col_scale != nullptr && n < p.N) ? __ldg(p.col_scale + n) : 1.0f);
+            }
+            bar_sync_named(GEMM_EPI_BARRIER, 32 * Cfg::EPI_WARPS);  // every warp passes it once per item, whatever became of its waits
+            if (!alive) continue;
             const int m0 = (tm * CG + (int)rank) * Cfg::BM + q * 32;
             const int64_t row = m0 + lane;
-            const bool row_ok = row < p.M;
             // the row's scale is fetched (or summed from the prune launch's partial sums) while the
             // tile's main loop still runs
-            float s = 1.0f;
-            if (row_ok) {
-                if (p.scale_partial != nullptr) s = row_scale_from_partials(p.scale_partial, row, p.scale_ks);
-                else if (p.row_scale != nullptr) s = __ldg(p.row_scale + row);
+            float sl = 1.0f, s[4];
+            if (row < p.M) {
+                if (p.scale_partial != nullptr) sl = row_scale_from_partials(p.scale_partial, row, p.scale_ks);
+                else if (p.row_scale != nullptr) sl = __ldg(p.row_scale + row);
             }
-            // the tile's per-column terms (bias, FP8 weight scale), one column per lane and round,
-            // fetched while the main loop runs and handed round by shuffles in the chunk loop: no
-            // dependent global load is left between the accumulator and the store
-            constexpr int CH = Cfg::CH;
-            float bl_all[BN / CH][2], cl_all[BN / CH][2];
 #pragma unroll
-            for (int c = 0; c < BN / CH; ++c)
+            for (int i = 0; i < 4; ++i) s[i] = __shfl_sync(0xffffffffu, sl, 8 * i + (lane >> 2));
+            // stream-K pieces: fp32 partial slot of a cluster, [32-row quarter][CH-column chunk][half][8-column
+            // group][lane] float4 (512 contiguous bytes per group); one ready word per epilogue warp
+            constexpr size_t SLOT_FLOATS = (size_t)Cfg::BM * CG * BN;
+            auto piece = [&](int cluster, int c) {
+                return reinterpret_cast<float4*>(p.sk_partial + (size_t)cluster * SLOT_FLOATS) +
+                       (size_t)(((int)rank * 4 + q) * Cfg::NCH + c) * (CH / 4) * 32 + lane;
+            };
+            constexpr int FLAGS = CG * Cfg::EPI_WARPS;
+            const int my_flag = (int)rank * Cfg::EPI_WARPS + warp - GEMM_EPI_WARP0;
+            uint32_t packed[SLOTS][2][CH / 4];
+            auto convert = [&](auto has_residual) {
+                constexpr bool RES = decltype(has_residual)::value;
+                if constexpr (RES) {  // the residual arrives during the main loop, in the registers of the results
+                    if (w.kind != 1) {
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int idx = u * 32 + lane, n = tn * BN + c * CH + idx;
-                    bl_all[c][u] = 0.f;
-                    cl_all[c][u] = 1.f;
-                    if (idx < CH && n < p.N) {
-                        if (p.bias != nullptr) bl_all[c][u] = __uint_as_float((uint32_t)__ldg(p.bias + n) << 16);
-                        if constexpr (Cfg::FP8)
-                            if (p.col_scale != nullptr) cl_all[c][u] = __ldg(p.col_scale + n);
+                        for (int slot = 0; slot < SLOTS; ++slot)
+                            if (slot < slots)
+                                epi_load_residual<CH>(p.residual, p.ldr, m0, p.M, tn * BN + (c0 + slot) * CH, p.N, lane, packed[slot]);
                     }
                 }
-            if (!mbar_wait(bar_tfull + 8 * acc, acc_phase, cta_abort, p.dev_error)) break;
-            tc_fence_after();
-            const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN;
-            // stream-K pieces: this thread's row of the pair tile inside an fp32 partial slot
-            const size_t slot_floats = (size_t)Cfg::BM * CG * BN;
-            // layout of a slot: [CH-column chunk][16-byte piece j][row of the pair tile] float4, so a
-            // warp's 32 rows of one piece are 512 contiguous bytes
-            constexpr int SLOT_ROWS = Cfg::BM * CG;
-            const size_t my_row_off = (size_t)((int)rank * Cfg::BM + q * 32 + lane);
-            const int my_flag = (int)rank * 4 + q;
-            if (w.kind == 2) {
-                // wait until every contributing cluster's matching warp has published its rows
-                if (lane == 0) {
+                alive = mbar_wait_warp(bar_tfull + 8 * acc, acc_phase, cta_abort, p.dev_error);
+                if (!alive) return;
+                tc_fence_after();
+                if (w.kind == 2) {
+                    // wait until every contributing cluster's matching warp has published its rows
                     for (int cc = w.first_contrib; cc < cluster_id && alive; ++cc)
                         if (sched.has_tail(cc))
-                            alive = flag_wait(p.sk_flags + cc * 8 + my_flag, p.sk_epoch, cta_abort, p.dev_error);
+                            alive = __all_sync(0xffffffffu, flag_wait(p.sk_flags + cc * FLAGS + my_flag, p.sk_epoch, cta_abort, p.dev_error));
+                    if (!alive) return;
                 }
-                alive = __shfl_sync(0xffffffffu, (int)alive, 0) != 0;
-                if (!alive) break;
-            }
-            constexpr int NCH = BN / CH;
-            // this warp's last chunk: after reading it the accumulator goes back to the issuer
-            const int c_last = NCH - 1 - ((NCH - 1 - c_first) % Cfg::EPI_SPLIT);
-#pragma unroll 1
-            for (int c = c_first; c < NCH; c += Cfg::EPI_SPLIT) {
-                const int n0 = tn * BN + c * CH;
-                // this chunk's two rounds, picked with selects so that the arrays stay in registers
-                // (an index that depends on the loop counter would put them into local memory and
-                // force every load above to complete before the wait)
-                float bl[2] = {bl_all[0][0], bl_all[0][1]}, cl[2] = {cl_all[0][0], cl_all[0][1]};
+                const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN;
 #pragma unroll
-                for (int cc = 1; cc < BN / CH; ++cc)
-                    if (c == cc) {
-                        bl[0] = bl_all[cc][0]; bl[1] = bl_all[cc][1];
-                        cl[0] = cl_all[cc][0]; cl[1] = cl_all[cc][1];
-                    }
-                uint32_t v[CH];
-                tmem_ld_32x32b_x32(t_row + c * CH, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-                if constexpr (CH == 64)
-                    tmem_ld_32x32b_x32(t_row + c * CH + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-                else
-                    tmem_ld_32x32b_x16(t_row + c * CH + 32, *reinterpret_cast<uint32_t(*)[16]>(&v[32]));
-                tmem_ld_wait();
-                if (c == c_last) {
-                    // accumulator fully read: hand it back to the MMA issuer
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if constexpr (CG == 1) mbar_arrive(bar_tempty + 8 * acc);
-                        else mbar_arrive_cluster(tempty0 + 8 * acc);
-                    }
-                }
-                if (w.kind == 1) {
-                    // partial piece: raw fp32 accumulators to this cluster's slot
-                    float4* dst = reinterpret_cast<float4*>(p.sk_partial + (size_t)cluster_id * slot_floats) +
-                                  (size_t)c * (CH / 4) * SLOT_ROWS + my_row_off;
-#pragma unroll
-                    for (int j = 0; j < CH / 4; ++j)
-                        __stcg(dst + (size_t)j * SLOT_ROWS, make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                                    __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])));
-                    continue;
-                }
-                if (w.kind == 2) {
-                    // owner piece: add the partials in ascending cluster order
-                    for (int cc = w.first_contrib; cc < cluster_id; ++cc) {
-                        if (!sched.has_tail(cc)) continue;
-                        const float4* src = reinterpret_cast<const float4*>(p.sk_partial + (size_t)cc * slot_floats) +
-                                            (size_t)c * (CH / 4) * SLOT_ROWS + my_row_off;
-                        float4 pa[CH / 4];
-#pragma unroll
-                        for (int j = 0; j < CH / 4; ++j) pa[j] = __ldcg(src + (size_t)j * SLOT_ROWS);
-#pragma unroll
-                        for (int j = 0; j < CH / 4; ++j) {
-                            const float4 a = pa[j];
-                            v[4 * j] = __float_as_uint(__uint_as_float(v[4 * j]) + a.x);
-                            v[4 * j + 1] = __float_as_uint(__uint_as_float(v[4 * j + 1]) + a.y);
-                            v[4 * j + 2] = __float_as_uint(__uint_as_float(v[4 * j + 2]) + a.z);
-                            v[4 * j + 3] = __float_as_uint(__uint_as_float(v[4 * j + 3]) + a.w);
+                for (int slot = 0; slot < SLOTS; ++slot) {
+                    if (slot >= slots) break;
+                    const int c = c0 + slot;
+                    uint32_t v[2][CH / 2];
+                    epi_tmem_ld<CH>(t_row + c * CH, v);
+                    tmem_ld_wait();
+                    if (slot == slots - 1) {
+                        // this warp's share of the accumulator is read: hand it back to the MMA issuer
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if constexpr (CG == 1) mbar_arrive(bar_tempty + 8 * acc);
+                            else mbar_arrive_cluster(tempty0 + 8 * acc);
                         }
                     }
-                }
-                if (n0 >= p.N) continue;
-                // staging buffer must have been read by its previous TMA store
-                if (lane == 0) tma_store_wait_read<Cfg::CBUFS_W - 1>();
-                __syncwarp();
-                const uint32_t cbuf = cbuf0 + cb * Cfg::C_BOX_BYTES;
+                    if (w.kind == 1) {
+                        // partial piece: raw fp32 accumulators to this cluster's slot
+                        float4* dst = piece(cluster_id, c);
 #pragma unroll
-                for (int j = 0; j < CH / 8; ++j) {  // 8 columns (16 bytes of output) at a time
-                    const int n = n0 + j * 8;
-                    float b[8];
-                    float r[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int col = j * 8 + e;
-                        b[e] = __shfl_sync(0xffffffffu, bl[col >> 5], col & 31);
+                        for (int i = 0; i < CH / 4; ++i) {
+                            const uint32_t* x = &v[i / (CH / 8)][4 * (i % (CH / 8))];
+                            __stcg(dst + i * 32, make_float4(__uint_as_float(x[0]), __uint_as_float(x[1]), __uint_as_float(x[2]),
+                                                             __uint_as_float(x[3])));
+                        }
+                        continue;
                     }
-                    if (n < p.N) {
-                        if (p.residual != nullptr && row_ok) {
-                            const uint4 rv = __ldg(reinterpret_cast<const uint4*>(p.residual + row * p.ldr + n));
-                            r[0] = bf16_lo_f(rv.x); r[1] = bf16_hi_f(rv.x);
-                            r[2] = bf16_lo_f(rv.y); r[3] = bf16_hi_f(rv.y);
-                            r[4] = bf16_lo_f(rv.z); r[5] = bf16_hi_f(rv.z);
-                            r[6] = bf16_lo_f(rv.w); r[7] = bf16_hi_f(rv.w);
+                    if (w.kind == 2) {
+                        // owner piece: add the partials in ascending cluster order
+                        for (int cc = w.first_contrib; cc < cluster_id; ++cc) {
+                            if (!sched.has_tail(cc)) continue;
+                            const float4* src = piece(cc, c);
+#pragma unroll
+                            for (int i = 0; i < CH / 4; ++i) {
+                                const float4 a = __ldcg(src + i * 32);
+                                uint32_t* x = &v[i / (CH / 8)][4 * (i % (CH / 8))];
+                                x[0] = __float_as_uint(__uint_as_float(x[0]) + a.x);
+                                x[1] = __float_as_uint(__uint_as_float(x[1]) + a.y);
+                                x[2] = __float_as_uint(__uint_as_float(x[2]) + a.z);
+                                x[3] = __float_as_uint(__uint_as_float(x[3]) + a.w);
+                            }
                         }
                     }
-                    float cs[8] = {s, s, s, s, s, s, s, s};  // row scale (x per-channel weight scale)
-                    if constexpr (Cfg::FP8) {
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const int col = j * 8 + e;
-                            cs[e] = s * __shfl_sync(0xffffffffu, cl[col >> 5], col & 31);
-                        }
-                    }
-                    uint32_t o[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float y0 = fmaf(cs[2 * e], __uint_as_float(v[j * 8 + 2 * e]), b[2 * e]) + r[2 * e];
-                        const float y1 = fmaf(cs[2 * e + 1], __uint_as_float(v[j * 8 + 2 * e + 1]), b[2 * e + 1]) + r[2 * e + 1];
-                        o[e] = pack_bf16x2(y0, y1);
-                    }
-                    if constexpr (CH == 64)  // 128-byte rows, 16-byte chunk index XOR (row % 8): the 128-byte swizzle
-                        sts128(cbuf + lane * 128 + ((j ^ (lane & 7)) << 4), o[0], o[1], o[2], o[3]);
-                    else  // dense 96-byte rows for the unswizzled 48-column box
-                        sts128(cbuf + lane * (CH * 2) + (j << 4), o[0], o[1], o[2], o[3]);
+                    epi_convert<CH, Cfg::FP8, RES>(v, s, sb + c * (CH * 4), sc + c * (CH * 4), lane, packed[slot]);
                 }
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    tma_store_2d(&tmap_y, n0, m0, cbuf);
-                    tma_store_commit();
-                }
-                cb = (cb + 1 == Cfg::CBUFS_W) ? 0 : cb + 1;
-            }
+            };
+            if (p.residual != nullptr) convert(std::true_type{});
+            else convert(std::false_type{});
+            if (!alive) continue;
             if (w.kind == 1) {
                 // publish: all lanes' stores (ordered before lane 0 by the warp barrier), then the
                 // releasing store of the ready word of this (slot, warp)
                 __syncwarp();
-                if (lane == 0) st_release_gpu(p.sk_flags + cluster_id * 8 + my_flag, p.sk_epoch);
+                if (lane == 0) st_release_gpu(p.sk_flags + cluster_id * FLAGS + my_flag, p.sk_epoch);
+                continue;
+            }
+#pragma unroll
+            for (int slot = 0; slot < SLOTS; ++slot) {
+                if (slot >= slots) break;
+                const int n0 = tn * BN + (c0 + slot) * CH;
+                // rows past M and columns past N are clipped by the store.  The last tile stages in the ring:
+                // its MMAs are done (the wait above) and nothing is loaded any more.
+                if (n0 < p.N)
+                    epi_store<CH, Cfg::BOX_ROWS>(&tmap_y, packed[slot], n0, m0,
+                                                 last ? smem_base + ((warp - GEMM_EPI_WARP0) * SLOTS + slot) * (32 * CH * 2) : own_box, last, lane);
             }
         }
-        if (lane == 0) tma_store_wait_all<0>();
+        if (lane == 0) tma_store_wait_read<0>();  // (the end of the grid makes the stores visible)
     }
 
     // ---------------------------------------------------------------------- teardown ----------
     tc_fence_before();
     __syncthreads();
-    if constexpr (CG == 2) cluster_sync_all();
+    if constexpr (CG == 2) cluster_sync_relaxed();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc<CG>(tmem_base, Cfg::TMEM_COLS);

@@ -28,6 +28,7 @@
 
 #include "ptx.cuh"
 #include "prune_compress.cuh"  // row_scale_from_partials
+#include "epilogue.cuh"
 #include "sparse_gemm.cuh"     // make_idesc_sp_bf16
 
 namespace lynx {
@@ -139,8 +140,8 @@ struct Gemm2Cfg {
     static constexpr int E_COL0 = 2 * BN;              // metadata columns behind the two accumulators
     static constexpr int E_COLS = 8;                   // per stage: 4 per row tile
     static constexpr int TMEM_COLS = 512;
-    static constexpr int EPI_WARPS = 8;
-    static constexpr int THREADS = 64 + 32 * EPI_WARPS;
+    static constexpr int EPI_WARPS = GEMM_EPI_WARPS;
+    static constexpr int THREADS = GEMM_THREADS;
     // the single-tile items run on a ring of their own over the same shared memory: four stages of
     // 48 KB (A 16 KB, metadata 2 KB, W 30 KB) instead of three of 66 KB
     static constexpr int STAGES1 = 4;
@@ -148,9 +149,10 @@ struct Gemm2Cfg {
     static constexpr int NUM_BARS = 2 * STAGES + 2 * STAGES1 + 4;
     static constexpr int C_BOX_BYTES = 32 * CH * 2;    // one epilogue warp's staging box: 32 rows x 48 columns
     static constexpr int C_BYTES = EPI_WARPS * C_BOX_BYTES;
-    static constexpr int BIAS_BYTES = BN * 2;          // one epilogue warp's copy of the item's bias values (bf16)
-    static constexpr int SMEM_BYTES = 1024 /*align slack*/ + STAGES * STAGE_BYTES + C_BYTES + EPI_WARPS * BIAS_BYTES + 256;
-    static_assert(BN % CH == 0 && BN % 16 == 0 && BN_CTA % 8 == 0, "tile N");
+    static constexpr int BIAS_BYTES = BN * 4;          // the item's bias values (fp32), two items' worth
+    static constexpr int SMEM_BYTES = 1024 /*align slack*/ + STAGES * STAGE_BYTES + C_BYTES + 2 * BIAS_BYTES + 256;
+    static_assert(NCH == 5 && BN % CH == 0 && BN_CTA % 8 == 0, "tile N: the epilogue deals five chunks per accumulator");
+    static_assert(EPI_WARPS * 5 * C_BOX_BYTES <= STAGES * STAGE_BYTES, "last item: a staging box per chunk in the ring");
     static_assert(B_HALF_BYTES % 1024 == 0, "swizzle atoms need 1024-byte aligned tiles");
     static_assert(E_COL0 + E_COLS * STAGES <= TMEM_COLS && 4 * STAGES1 <= E_COLS * STAGES, "tensor memory budget");
     static_assert(RING1_E + STAGES1 * E_BYTES <= STAGES * STAGE_BYTES, "the single-tile ring fits into the double ring's memory");
@@ -173,8 +175,8 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     const uint32_t sB = sA + STAGES * 2 * Cfg::A_BYTES;         // [stage] B_BYTES
     const uint32_t sE = sB + STAGES * Cfg::B_BYTES;             // [stage][row tile] E_BYTES
     const uint32_t sC = sE + STAGES * 2 * Cfg::E_BYTES;         // [epilogue warp] C_BOX_BYTES
-    const uint32_t sBias = sC + Cfg::C_BYTES;                   // [epilogue warp] BIAS_BYTES
-    const uint32_t sBar = sBias + Cfg::EPI_WARPS * Cfg::BIAS_BYTES;
+    const uint32_t sBias = sC + Cfg::C_BYTES;                   // [item parity] BIAS_BYTES
+    const uint32_t sBar = sBias + 2 * Cfg::BIAS_BYTES;
     const uint32_t bar_full = sBar, bar_empty = sBar + 8 * STAGES;
     const uint32_t bar_tfull = sBar + 16 * STAGES, bar_tempty = bar_tfull + 16;
     const uint32_t bar_full1 = bar_tempty + 16, bar_empty1 = bar_full1 + 8 * Cfg::STAGES1;  // single-tile ring
@@ -201,7 +203,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(bar_tfull + 8 * a, 1);   // one tcgen05.commit
-            mbar_init(bar_tempty + 8 * a, 8);  // the accumulator's four epilogue warps in both CTAs
+            mbar_init(bar_tempty + 8 * a, 2 * Cfg::EPI_WARPS);  // the epilogue warps of both CTAs
         }
         fence_mbar_init();
         prefetch_tmap(&tmap_a);
@@ -219,7 +221,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     }
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();
+    cluster_sync_relaxed();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     // W tiles of the first stages of the first item, before the wait for the previous kernel (W is
@@ -245,6 +247,8 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     // everything above overlapped the previous kernel's tail; its results are needed from here on
     griddep_wait();
 
+    if (warp < GEMM_EPI_WARP0) {
+    setmaxnreg_dec<GEMM_REGS_ISSUE>();
     if (warp == 0) {
         // ------------------------------------------------------------------ producer ----------
         {
@@ -336,15 +340,14 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                 const uint32_t bfull = ring1 ? bar_full1 : bar_full, bempty = ring1 ? bar_empty1 : bar_empty;
                 // accumulators of this item: a double fills both, the k-th single accumulator k % 2
                 const int acc0 = (rows == 2) ? 0 : (ordinal & 1);
-                for (int r = 0; r < rows && ok; ++r) {
-                    const int a = acc0 + r;
-                    ok = mbar_wait_warp(bar_tempty + 8 * a, (uses[a] & 1u) ^ 1u, cta_abort, p.dev_error);
-                }
-                if (!ok) break;
+                // (a double's second accumulator is waited for behind the first one's MMAs: the epilogue
+                // hands them back one after the other)
+                if (!mbar_wait_warp(bar_tempty + 8 * acc0, (uses[acc0] & 1u) ^ 1u, cta_abort, p.dev_error)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc0 * BN;
+                const int ksteps = kblocks + lora_steps;
                 uint32_t accumulate = 0;
-                for (int kb = 0; kb < kblocks + lora_steps; ++kb) {
+                for (int kb = 0; kb < ksteps; ++kb) {
                     if (!mbar_wait_warp(bfull + 8 * stage, phase, cta_abort, p.dev_error)) {
                         ok = false;
                         break;
@@ -354,204 +357,168 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                                                 : ring_lo0 + stage * (2 * Cfg::A_BYTES >> 4);
                     const uint32_t b_lo = ring1 ? ring_lo0 + ((Cfg::RING1_B + stage * Cfg::B_BYTES) >> 4)
                                                 : b_lo0 + stage * (Cfg::B_BYTES >> 4);
-                    if (elect_one()) {
-                        if (kb < kblocks) {
-                            const uint32_t e_tmem = tmem_base + Cfg::E_COL0 + (ring1 ? 4 * stage : Cfg::E_COLS * stage);
-                            const uint64_t e_desc = ring1 ? e1_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4))
-                                                          : e_d0 + (uint64_t)(stage * (2 * Cfg::E_BYTES >> 4));
-                            tmem_cp_128x128b<2>(e_tmem, e_desc);
-                            if (rows == 2) tmem_cp_128x128b<2>(e_tmem + 4, e_desc + (uint64_t)(Cfg::E_BYTES >> 4));
-                            // four K steps of 32 logical elements per row tile: A advances 32 bytes, W 64 bytes
-                            // (steps 2, 3 in the second 64-element slice); metadata column pair + step parity
-                            mma_sp_bf16_lh<2>(d_tmem, a_lo, b_lo, desc_hi, e_tmem, idesc0, accumulate);
-                            mma_sp_bf16_lh<2>(d_tmem, a_lo + 2, b_lo + 4, desc_hi, e_tmem, idesc1, 1u);
-                            mma_sp_bf16_lh<2>(d_tmem, a_lo + 4, b_lo + BH, desc_hi, e_tmem + 2, idesc0, 1u);
-                            mma_sp_bf16_lh<2>(d_tmem, a_lo + 6, b_lo + BH + 4, desc_hi, e_tmem + 2, idesc1, 1u);
-                            if (rows == 2) {
-                                constexpr uint32_t A1 = Cfg::A_BYTES >> 4;
-                                mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1, b_lo, desc_hi, e_tmem + 4, idesc0, accumulate);
-                                mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 2, b_lo + 4, desc_hi, e_tmem + 4, idesc1, 1u);
-                                mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 4, b_lo + BH, desc_hi, e_tmem + 6, idesc0, 1u);
-                                mma_sp_bf16_lh<2>(d_tmem + BN, a_lo + A1 + 6, b_lo + BH + 4, desc_hi, e_tmem + 6, idesc1, 1u);
-                            }
+                    const uint32_t e_tmem = tmem_base + Cfg::E_COL0 + (ring1 ? 4 * stage : Cfg::E_COLS * stage);
+                    const uint64_t e_desc = ring1 ? e1_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4))
+                                                  : e_d0 + (uint64_t)(stage * (2 * Cfg::E_BYTES >> 4));
+                    const bool sparse = kb < kblocks;
+                    // one row tile's MMAs of this stage
+                    auto issue = [&](int r) {
+                        const uint32_t dt = d_tmem + r * BN, al = a_lo + r * (Cfg::A_BYTES >> 4), et = e_tmem + 4 * r;
+                        if (sparse) {
+                            // four K steps of 32 logical elements: A advances 32 bytes, W 64 bytes (steps 2, 3 in
+                            // the second 64-element slice); metadata column pair + step parity
+                            mma_sp_bf16_lh<2>(dt, al, b_lo, desc_hi, et, idesc0, accumulate);
+                            mma_sp_bf16_lh<2>(dt, al + 2, b_lo + 4, desc_hi, et, idesc1, 1u);
+                            mma_sp_bf16_lh<2>(dt, al + 4, b_lo + BH, desc_hi, et + 2, idesc0, 1u);
+                            mma_sp_bf16_lh<2>(dt, al + 6, b_lo + BH + 4, desc_hi, et + 2, idesc1, 1u);
                         } else {
                             // low-rank stage: dense K steps of 16 elements, both operands advance 32 bytes
-                            for (int r = 0; r < rows; ++r) {
-                                const uint32_t dt = d_tmem + r * BN, al = a_lo + r * (Cfg::A_BYTES >> 4);
-                                mma_bf16_lh<2>(dt, al, b_lo, desc_hi, idesc_dense, accumulate);
-                                mma_bf16_lh<2>(dt, al + 2, b_lo + 2, desc_hi, idesc_dense, 1u);
-                                mma_bf16_lh<2>(dt, al + 4, b_lo + 4, desc_hi, idesc_dense, 1u);
-                                mma_bf16_lh<2>(dt, al + 6, b_lo + 6, desc_hi, idesc_dense, 1u);
-                            }
+                            mma_bf16_lh<2>(dt, al, b_lo, desc_hi, idesc_dense, accumulate);
+                            mma_bf16_lh<2>(dt, al + 2, b_lo + 2, desc_hi, idesc_dense, 1u);
+                            mma_bf16_lh<2>(dt, al + 4, b_lo + 4, desc_hi, idesc_dense, 1u);
+                            mma_bf16_lh<2>(dt, al + 6, b_lo + 6, desc_hi, idesc_dense, 1u);
                         }
-                        tc_commit_pair(bempty + 8 * stage, 0x3);
+                    };
+                    if (elect_one()) {
+                        if (sparse) {
+                            tmem_cp_128x128b<2>(e_tmem, e_desc);
+                            if (rows == 2) tmem_cp_128x128b<2>(e_tmem + 4, e_desc + (uint64_t)(Cfg::E_BYTES >> 4));
+                        }
+                        issue(0);
+                        if (kb == ksteps - 1) tc_commit_pair(bar_tfull + 8 * acc0, 0x3);
                     }
+                    if (rows == 2) {
+                        if (kb == 0) {
+                            if (!mbar_wait_warp(bar_tempty + 8, (uses[1] & 1u) ^ 1u, cta_abort, p.dev_error)) {
+                                ok = false;
+                                break;
+                            }
+                            tc_fence_after();
+                        }
+                        if (elect_one()) {
+                            issue(1);
+                            if (kb == ksteps - 1) tc_commit_pair(bar_tfull + 8, 0x3);
+                        }
+                    }
+                    if (elect_one()) tc_commit_pair(bempty + 8 * stage, 0x3);
                     accumulate = 1u;
                     if (++stage == nst) { stage = 0; phase ^= 1; }
                 }
-                if (!ok) break;
-                for (int r = 0; r < rows; ++r) {
-                    if (elect_one()) tc_commit_pair(bar_tfull + 8 * (acc0 + r), 0x3);
-                    ++uses[acc0 + r];
-                }
+                for (int r = 0; r < rows; ++r) ++uses[acc0 + r];
             }
         }
+    }
     } else {
+        setmaxnreg_inc<GEMM_REGS_EPI>();
         // ------------------------------------------------------------------ epilogue ----------
-        const int g = (warp - 2) >> 2;  // the accumulator this warp drains
+        // Both warps of a lane quarter drain every accumulator.  An accumulator's five chunks are dealt
+        // 3 + 2, a double's second accumulator 2 + 3, so a warp holds at most five chunks.
+        const int h = (warp - GEMM_EPI_WARP0) >> 2;  // which of the quarter's two warps
         const int q = warp & 3;         // tensor-memory lane quarter this warp may read
         const uint32_t tempty0 = mapa(bar_tempty, 0);
-        const uint32_t cbuf = sC + (warp - 2) * Cfg::C_BOX_BYTES;
-        uint32_t uses = 0;
+        const uint32_t own_box = sC + (warp - GEMM_EPI_WARP0) * Cfg::C_BOX_BYTES;
         constexpr int CH = Cfg::CH, NCH = Cfg::NCH;
+        const int n_first = h == 0 ? 3 : 2;  // chunks of the item's first accumulator
+        uint32_t uses[2] = {0u, 0u};
+        bool alive = true;
         for (int it = 0; it < num_items; ++it) {
             int tm0, tn, rows, ordinal;
             sched.item(cluster_id, it, tm0, tn, rows, ordinal);
-            int tm;
-            if (rows == 2) tm = tm0 + g;
-            else if ((ordinal & 1) == g) tm = tm0;
-            else continue;
-            const int m0 = (tm * 2 + (int)rank) * Cfg::BM + q * 32;
-            const int64_t row = m0 + lane;
-            const bool row_ok = row < p.M;
-            // the row's scale (or its sum from the prune launch's partial sums) and the tile's bias
-            // values, one column per lane and round, are fetched while the main loop still runs
-            float s = 1.0f;
-            if (row_ok) {
-                if (p.scale_partial != nullptr) s = row_scale_from_partials(p.scale_partial, row, p.scale_ks);
-                else if (p.row_scale != nullptr) s = __ldg(p.row_scale + row);
+            const bool last = it == num_items - 1;
+            const int acc0 = (rows == 2) ? 0 : (ordinal & 1);
+            // the item's bias values as fp32, for all epilogue warps (the other parity's may still be read)
+            const uint32_t sb = sBias + (it & 1) * Cfg::BIAS_BYTES;
+            if (const int c = (int)threadIdx.x - 32 * GEMM_EPI_WARP0; c < BN) {
+                const int n = tn * BN + c;
+                sts32f(sb + c * 4, (p.bias != nullptr && n < p.N) ? __uint_as_float((uint32_t)__ldg(p.bias + n) << 16) : 0.0f);
             }
-            // the item's bias values go to this warp's own strip of shared memory (30 lanes x 8 bf16);
-            // the conversion below reads them back as broadcast 16-byte loads (a shuffle per value
-            // made the shuffle unit the bottleneck of the five conversion rounds)
-            const uint32_t sb = sBias + (warp - 2) * Cfg::BIAS_BYTES;
-            if (lane < BN / 8) {
-                const int n = tn * BN + lane * 8;
-                uint4 bq = make_uint4(0u, 0u, 0u, 0u);
-                if (p.bias != nullptr && n < p.N) bq = __ldg(reinterpret_cast<const uint4*>(p.bias + n));
-                sts128(sb + lane * 16, bq.x, bq.y, bq.z, bq.w);
-            }
-            __syncwarp();
-            if (!mbar_wait(bar_tfull + 8 * g, uses & 1u, cta_abort, p.dev_error)) break;
-            ++uses;
-            tc_fence_after();
-            const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + g * BN;
-            const uint16_t* rrow = (p.residual != nullptr) ? p.residual + row * p.ldr : nullptr;
-            if (rrow == nullptr) {
-                // Fast path (no residual addend): the whole accumulator row is converted to packed
-                // bf16 in registers first, so the accumulator goes back to the MMA issuer after five
-                // tcgen05.ld round trips; the stores follow while the next main loop already runs.
-                uint32_t packed[NCH][CH / 2];
+            bar_sync_named(GEMM_EPI_BARRIER, 32 * Cfg::EPI_WARPS);  // every warp passes it once per item, whatever became of its waits
+            if (!alive) continue;
+            // the rows' scales (or their sums from the prune launch's partial sums) are fetched while
+            // the main loop still runs
+            const int m0 = (tm0 * 2 + (int)rank) * Cfg::BM + q * 32;  // this warp's rows in the first row tile; the second: + 256
+            float s[2][4];
 #pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    uint32_t v[CH];
-                    tmem_ld_32x32b_x32(t_row + c * CH, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-                    tmem_ld_32x32b_x16(t_row + c * CH + 32, *reinterpret_cast<uint32_t(*)[16]>(&v[32]));
+            for (int r = 0; r < 2; ++r) {
+                const int64_t row = m0 + r * 256 + lane;
+                float sl = 1.0f;
+                if (r < rows && row < p.M) {
+                    if (p.scale_partial != nullptr) sl = row_scale_from_partials(p.scale_partial, row, p.scale_ks);
+                    else if (p.row_scale != nullptr) sl = __ldg(p.row_scale + row);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) s[r][i] = __shfl_sync(0xffffffffu, sl, 8 * i + (lane >> 2));
+            }
+            const int slots = rows == 2 ? NCH : n_first;
+            // slot -> row tile of the item and chunk
+            auto chunk_of = [&](int slot, int& r, int& c) {
+                r = slot >= n_first;
+                c = h == 0 ? (r ? slot - 3 : slot) : (r ? slot : 3 + slot);
+            };
+            // All chunks are converted to packed bf16 first, so an accumulator goes back after its
+            // tensor-memory reads; the stores follow while the next main loop already runs.
+            uint32_t packed[NCH][2][CH / 4];
+            auto convert = [&](auto has_residual) {
+                constexpr bool RES = decltype(has_residual)::value;
+                if constexpr (RES) {  // the residual arrives during the main loop, in the registers of the results
+#pragma unroll
+                    for (int slot = 0; slot < NCH; ++slot) {
+                        if (slot >= slots) break;
+                        int r, c;
+                        chunk_of(slot, r, c);
+                        epi_load_residual<CH>(p.residual, p.ldr, m0 + r * 256, p.M, tn * BN + c * CH, p.N, lane, packed[slot]);
+                    }
+                }
+#pragma unroll
+                for (int slot = 0; slot < NCH; ++slot) {
+                    if (slot >= slots || !alive) break;
+                    int r, c;
+                    chunk_of(slot, r, c);
+                    const int acc = acc0 + r;
+                    if (slot == 0 || slot == n_first) {
+                        alive = mbar_wait_warp(bar_tfull + 8 * acc, uses[acc] & 1u, cta_abort, p.dev_error);
+                        if (!alive) break;
+                        ++uses[acc];
+                        tc_fence_after();
+                    }
+                    uint32_t v[2][CH / 2];
+                    epi_tmem_ld<CH>(tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + c * CH, v);
                     tmem_ld_wait();
-                    if (c == NCH - 1) {
-                        // accumulator fully read: hand it back to the MMA issuer
+                    if (slot == n_first - 1 || slot == slots - 1) {
+                        // this warp's share of the accumulator is read: hand it back to the MMA issuer
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive_cluster(tempty0 + 8 * g);
+                        if (lane == 0) mbar_arrive_cluster(tempty0 + 8 * acc);
                     }
+                    float sr[4];
 #pragma unroll
-                    for (int j = 0; j < CH / 8; ++j) {
-                        uint32_t bq[4];
-                        lds128(sb + c * (CH * 2) + j * 16, bq[0], bq[1], bq[2], bq[3]);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            packed[c][4 * j + e] = pack_bf16x2(fmaf(s, __uint_as_float(v[8 * j + 2 * e]), bf16_lo_f(bq[e])),
-                                                               fmaf(s, __uint_as_float(v[8 * j + 2 * e + 1]), bf16_hi_f(bq[e])));
-                    }
+                    for (int i = 0; i < 4; ++i) sr[i] = r ? s[1][i] : s[0][i];
+                    epi_convert<CH, false, RES>(v, sr, sb + c * (CH * 4), 0u, lane, packed[slot]);
                 }
+            };
+            if (p.residual != nullptr) convert(std::true_type{});
+            else convert(std::false_type{});
+            if (!alive) continue;
 #pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    const int n0 = tn * BN + c * CH;
-                    if (n0 >= p.N) continue;
-                    // the staging box must have been read by this warp's previous TMA store
-                    if (lane == 0) tma_store_wait_read<0>();
-                    __syncwarp();
-#pragma unroll
-                    for (int j = 0; j < CH / 8; ++j)  // dense 96-byte rows
-                        sts128(cbuf + lane * (CH * 2) + (j << 4), packed[c][4 * j], packed[c][4 * j + 1], packed[c][4 * j + 2],
-                               packed[c][4 * j + 3]);
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) {
-                        tma_store_2d(&tmap_y, n0, m0, cbuf);  // rows past M and columns past N are clipped
-                        tma_store_commit();
-                    }
-                }
-                continue;
-            }
-            // With a residual addend (its values have to be fetched per chunk): chunk by chunk, the
-            // next chunk's accumulators travelling while the current one is converted and stored.
-            uint32_t v[2][CH];
-            tmem_ld_32x32b_x32(t_row, *reinterpret_cast<uint32_t(*)[32]>(&v[0][0]));
-            tmem_ld_32x32b_x16(t_row + 32, *reinterpret_cast<uint32_t(*)[16]>(&v[0][32]));
-#pragma unroll
-            for (int c = 0; c < NCH; ++c) {
-                tmem_ld_wait();
-                if (c + 1 < NCH) {
-                    tmem_ld_32x32b_x32(t_row + (c + 1) * CH, *reinterpret_cast<uint32_t(*)[32]>(&v[(c + 1) & 1][0]));
-                    tmem_ld_32x32b_x16(t_row + (c + 1) * CH + 32, *reinterpret_cast<uint32_t(*)[16]>(&v[(c + 1) & 1][32]));
-                } else {
-                    // accumulator fully read: hand it back to the MMA issuer
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(tempty0 + 8 * g);
-                }
+            for (int slot = 0; slot < NCH; ++slot) {
+                if (slot >= slots) break;
+                int r, c;
+                chunk_of(slot, r, c);
                 const int n0 = tn * BN + c * CH;
-                if (n0 >= p.N) continue;
-                const uint32_t* vc = v[c & 1];
-                // the staging box must have been read by this warp's previous TMA store
-                if (lane == 0) tma_store_wait_read<0>();
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < CH / 8; ++j) {  // 8 columns (16 bytes of output) at a time
-                    const int n = n0 + j * 8;
-                    float bv[8];
-                    {
-                        uint32_t bq[4];
-                        lds128(sb + c * (CH * 2) + j * 16, bq[0], bq[1], bq[2], bq[3]);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            bv[2 * e] = bf16_lo_f(bq[e]);
-                            bv[2 * e + 1] = bf16_hi_f(bq[e]);
-                        }
-                    }
-                    float r[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                    if (n < p.N && row_ok) {
-                        const uint4 rv = __ldg(reinterpret_cast<const uint4*>(rrow + n));
-                        r[0] = bf16_lo_f(rv.x); r[1] = bf16_hi_f(rv.x);
-                        r[2] = bf16_lo_f(rv.y); r[3] = bf16_hi_f(rv.y);
-                        r[4] = bf16_lo_f(rv.z); r[5] = bf16_hi_f(rv.z);
-                        r[6] = bf16_lo_f(rv.w); r[7] = bf16_hi_f(rv.w);
-                    }
-                    uint32_t o[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float y0 = fmaf(s, __uint_as_float(vc[j * 8 + 2 * e]), bv[2 * e]) + r[2 * e];
-                        const float y1 = fmaf(s, __uint_as_float(vc[j * 8 + 2 * e + 1]), bv[2 * e + 1]) + r[2 * e + 1];
-                        o[e] = pack_bf16x2(y0, y1);
-                    }
-                    sts128(cbuf + lane * (CH * 2) + (j << 4), o[0], o[1], o[2], o[3]);  // dense 96-byte rows
-                }
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    tma_store_2d(&tmap_y, n0, m0, cbuf);  // rows past M and columns past N are clipped
-                    tma_store_commit();
-                }
+                // rows past M and columns past N are clipped by the store.  The last item stages in the ring:
+                // its MMAs are done (the wait above) and nothing is loaded any more.
+                if (n0 < p.N)
+                    epi_store<CH, 32>(&tmap_y, packed[slot], n0, m0 + r * 256,
+                                      last ? smem_base + ((warp - GEMM_EPI_WARP0) * NCH + slot) * Cfg::C_BOX_BYTES : own_box, last, lane);
             }
         }
-        if (lane == 0) tma_store_wait_all<0>();
+        if (lane == 0) tma_store_wait_read<0>();  // (the end of the grid makes the stores visible)
     }
 
     // ---------------------------------------------------------------------- teardown ----------
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();
+    cluster_sync_relaxed();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc<2>(tmem_base, Cfg::TMEM_COLS);
