@@ -443,21 +443,21 @@ lynx_status launch_gemm_cfg(lynx_ctx* ctx, const void* values, const void* meta,
 
 using Rt2Cfg = Gemm2Cfg<240, 3>;
 
-// Modelled time (us) of the slowest cluster for a schedule with D doubles.  Per-K-block times are
-// measured B200 figures: 0.69 us for a 512 x 240 stage (66 KB in flight per CTA and stage, three
-// stages) against 0.465 us for a 256 x 240 stage of sparse_gemm_kernel (0.49 us here); a double's
-// epilogue is exposed (the accumulators are not double-buffered: ~5 us per double including the
-// refill of the ring), a single's hides behind the next single; the switch between the two
-// rings costs a pipeline fill.  Within each class of clusters the one at the first position carries the
-// most singles, so two clusters decide the maximum.
-constexpr double RT2_T1 = 0.49, RT2_T2 = 0.69, RT2_E1 = 0.8, RT2_E2 = 5.0, RT2_SWITCH = 2.0;
+// Modelled time (us) of the slowest cluster for a schedule with D doubles.  The figures are fits to
+// measured B200 launches (back to back, clocks as they settle): 0.41 us per K block of a 256 x 240 single
+// (its epilogue hides behind the next one), 0.63 us per 512 x 240 K block, and 4.5 us per double from
+// its last MMA until the next item runs at full rate (both accumulators are read one after the other, and the
+// stores of 122 KB per CTA slow the next item's first loads).  4352 x 3072 x 3072: one double + one single per
+// cluster 34.9 us, three singles 36.2; 4096 x 3072 x 12288: doubles 121.7, singles 127.1.  Within each class of
+// clusters the one at the first position carries the most singles, so two clusters decide the maximum.
+constexpr double RT2_T1 = 0.41, RT2_T2 = 0.63, RT2_E1 = 0.3, RT2_E2 = 4.5;
 double rt2_makespan(const PairSchedule& sc, double kb) {
     double worst = 0.0;
     const int probe[2] = {sc.b % sc.C, 0};  // position 0 (first light cluster), position L (first heavy one)
     for (int i = 0; i < 2; ++i) {
         const int c = probe[i];
         const int nd = sc.num_doubles(c), ns = sc.num_singles(c);
-        const double t = nd * (kb * RT2_T2 + RT2_E2) + ns * (kb * RT2_T1 + RT2_E1) + ((nd && ns) ? RT2_SWITCH : 0.0);
+        const double t = nd * (kb * RT2_T2 + RT2_E2) + ns * (kb * RT2_T1 + RT2_E1);
         if (t > worst) worst = t;
     }
     return worst;
@@ -555,17 +555,17 @@ lynx_status launch_gemm_rt2(lynx_ctx* ctx, const Rt2Plan& plan, const void* valu
 }
 
 // Tile configuration for (M, N, K): the development override, else the smallest modelled time.
-// CTA-pair tiles 256 x {256, 240, 192, 128}.  A sparse MMA takes the same time whatever its N
-// (up to 256), so wide tiles win; 240 is the widest that still double-buffers the accumulator.
-// Model: rounds of tiles over the CTA pairs x (K blocks x measured time per K block + exposed
-// epilogue).  Per-K-block times (us) are measured B200 figures for each tile shape; the 256-wide
-// tile has one accumulator buffer, so its epilogue is not hidden.
+// CTA-pair tiles 256 x {256, 240, 192, 128}.
+// Model: rounds of tiles over the CTA pairs x (K blocks x time per K block + what a tile adds), fits to
+// measured B200 launches of each tile (us): 1024 x 3072 x 3072 14.5 with 192 against 16.1 with 240,
+// 4352 x 3072 x 3072 37.4 against 36.2, 1024 x 3072 x 9216 28.6 with 256 (two rounds) against 30.0 with
+// 192 (three).  The 256-wide tile has one accumulator buffer, so its epilogue is not hidden.
 int pick_gemm_cfg_model(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, double* t_us = nullptr) {
     const int pairs = num_sms / 2;
     const double kb = (double)(K / 128) + lora_steps;
-    // (the 192-wide tile runs with five stages of 42 KB, id 8: measured 4-7 % faster than with four)
+    // (the 192-wide tile runs with five stages of 42 KB, id 8)
     struct { int id, bn; double t_kb, epi; } cand[4] = {
-        {7, 240, 0.465, 0.6}, {5, 256, 0.50, 3.0}, {8, 192, 0.39, 0.8}, {6, 128, 0.345, 0.5}};
+        {7, 240, 0.41, 0.3}, {5, 256, 0.425, 2.0}, {8, 192, 0.325, 0.7}, {6, 128, 0.27, 0.6}};
     double best = 1e30;
     int cfg = 7;
     for (auto& c : cand) {
