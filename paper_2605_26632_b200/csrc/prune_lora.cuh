@@ -15,9 +15,16 @@
 // free again when the MMAs have retired and all eight tiles are in registers.  Warps 2..5 drain
 // the accumulator into the CTA's own shared memory at the end (the L_B half of the ring is free
 // by then); after a cluster barrier every CTA finishes 128 / splits rows of T: it reads those rows
-// of every split's partial through distributed shared memory, adds them in split order (the
-// result does not depend on timing), divides by the row scale -- summed from all splits' row sums
-// exactly as the GEMM epilogue will sum them -- and writes T.  No global round trip, no ticket.
+// of every split's partial and row sums through distributed shared memory, adds them in split order
+// (the result does not depend on timing), divides by the row scale -- the sums added exactly as the
+// GEMM epilogue will add them -- and writes T.  No global round trip, no ticket.
+//
+// What bounds it: the stream over X is at the HBM rate; what follows the last stage was half of the kernel
+// on 4352 x 3072 (cycles): 2700 in the cluster barrier, whose release waited for every value store of the
+// CTA, and 6400 in the finish, which 4 warps did after a global round trip for the row sums, one
+// dependent load at a time.  Now only the four drain warps release -- the prune warps hand them their row
+// sums in shared memory through a CTA barrier --, twelve warps finish T, and a thread's loads from all splits
+// are in flight together.
 #pragma once
 
 #include "lora_down.cuh"
@@ -50,7 +57,7 @@ struct PruneLoraCfg {
     static constexpr int PRUNERS = 8;                 // warps, one 16 x 128 tile each per stage
     static constexpr int THREADS = 64 + 128 + 32 * PRUNERS;
     static constexpr int TAIL_THREADS = 128 + 32 * PRUNERS;  // drain + prune warps meet once at the end
-    static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 1024;
+    static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 1536;
     static constexpr int TMEM_COLS = R;
     static constexpr int PARTIAL_BYTES = BM * R * 4;  // the drained accumulator, kept in the L_B ring
     static_assert(PARTIAL_BYTES <= STAGES * B_BYTES, "the partial fits where the L_B stages were");
@@ -74,7 +81,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     uint8_t* tail = smem_gen + (sBar - smem_base);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 128);
     volatile uint32_t* cta_abort = tmem_slot + 1;
-    float* s_scale = reinterpret_cast<float*>(tail + 256);  // [128] row scales of the finishing CTA
+    const uint32_t s_sums = sBar + 256;  // [128] (sum x^2, sum kept^2) of this split's rows
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles_m = (int)((p.M + Cfg::BM - 1) / Cfg::BM);
@@ -105,6 +112,8 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     griddep_wait();  // X comes from the kernels before this one
+    // the GEMM behind this launch may place its CTAs on the SMs left over and run its prologue
+    griddep_launch_dependents();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer ----------
@@ -206,8 +215,12 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 float* mine = p.scale_partial + (((int64_t)tm * 8 + pw) * p.splits + split) * 32;
                 *reinterpret_cast<float2*>(mine + 2 * r) = make_float2(numA, denA);
                 *reinterpret_cast<float2*>(mine + 2 * (r + 8)) = make_float2(numB, denB);
+                sts64f(s_sums + rowA_in * 8, numA, denA);
+                sts64f(s_sums + (rowA_in + 8) * 8, numB, denB);
             }
+            __syncwarp();
         }
+        bar_sync_named(3, Cfg::TAIL_THREADS);
     } else {
         // ------------------------------------------------------------------ drain -------------
         // accumulator -> this CTA's shared memory, float4 (row, 4 columns j) at (j * 128 + row) * 16:
@@ -229,46 +242,53 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                            v[4 * j + 3]);
             }
         }
+        __syncwarp();
+        bar_sync_named(3, Cfg::TAIL_THREADS);
     }
 
-    // every split's partial (shared memory) and row sums (global) are written: cluster-wide hand-over
+    // every split's partial and row sums are in shared memory: cluster-wide hand-over.  The drain warps
+    // release them (the prune warps' sums came to them through the barrier above); the others have nothing to
+    // release, in particular not their value stores.
     __syncwarp();
-    cluster_sync_all();
-    if (warp >= 2 && warp < 6) {
+    if (warp >= 2 && warp < 6) cluster_arrive_release();
+    else cluster_arrive_relaxed();
+    cluster_wait();
+    if (warp >= 2) {
         // this CTA finishes rows [split * 128 / splits, (split + 1) * 128 / splits) of the row block
         // (integer division: the shares differ by a row when splits does not divide 128)
-        const int t = threadIdx.x - 64;  // 0..127
+        const int t = threadIdx.x - 64;
         const int row_first = split * Cfg::BM / p.splits;
         const int rows_per = (split + 1) * Cfg::BM / p.splits - row_first;
-        if (t < rows_per) {
-            const int64_t grow = (int64_t)tm * Cfg::BM + row_first + t;
-            float s = 1.0f;
-            if constexpr (SUMS) {
-                // (the same additions, in the same order, as the GEMM epilogue that multiplies by s)
-                if (grow < p.M) s = row_scale_from_partials(p.scale_partial, grow, p.splits);
-            }
-            s_scale[t] = s;
-        }
-        bar_sync_named(2, 128);
         constexpr int PIECES_PER_ROW = R / 8;
         const int items = rows_per * PIECES_PER_ROW;
-        for (int idx = t; idx < items; idx += 128) {
+        for (int idx = t; idx < items; idx += Cfg::TAIL_THREADS) {
             const int r_l = idx / PIECES_PER_ROW, piece = idx % PIECES_PER_ROW;  // consecutive threads: one row's pieces
             const int r_t = row_first + r_l;
             const int64_t grow = (int64_t)tm * Cfg::BM + r_t;
             if (grow >= p.M) continue;
             const uint32_t a0 = sB + (uint32_t)(((2 * piece) * 128 + r_t) * 16);
             const uint32_t a1 = sB + (uint32_t)(((2 * piece + 1) * 128 + r_t) * 16);
-            float acc[8];
+            float4 a[8], b[8];
+            float2 q[8];
+#pragma unroll
+            for (int sp = 0; sp < 8; ++sp)  // every split's loads in flight together
+                if (sp < p.splits) {
+                    a[sp] = lds128_cluster_f32(mapa(a0, (uint32_t)sp));
+                    b[sp] = lds128_cluster_f32(mapa(a1, (uint32_t)sp));
+                    if constexpr (SUMS) q[sp] = lds64_cluster_f32(mapa(s_sums + r_t * 8, (uint32_t)sp));
+                }
+            float acc[8], num = 0.0f, den = 0.0f;
 #pragma unroll
             for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
-            for (int sp = 0; sp < p.splits; ++sp) {  // ascending split order, always
-                const float4 a = lds128_cluster_f32(mapa(a0, (uint32_t)sp));
-                const float4 b = lds128_cluster_f32(mapa(a1, (uint32_t)sp));
-                acc[0] += a.x; acc[1] += a.y; acc[2] += a.z; acc[3] += a.w;
-                acc[4] += b.x; acc[5] += b.y; acc[6] += b.z; acc[7] += b.w;
-            }
-            const float s = s_scale[r_l];
+#pragma unroll
+            for (int sp = 0; sp < 8; ++sp)  // ascending split order, always
+                if (sp < p.splits) {
+                    acc[0] += a[sp].x; acc[1] += a[sp].y; acc[2] += a[sp].z; acc[3] += a[sp].w;
+                    acc[4] += b[sp].x; acc[5] += b[sp].y; acc[6] += b[sp].z; acc[7] += b[sp].w;
+                    // (up to eight partial sums in ascending order: the additions of row_scale_from_partials)
+                    if constexpr (SUMS) { num += q[sp].x; den += q[sp].y; }
+                }
+            const float s = SUMS ? sqrtf(num / (den + 1e-8f)) : 1.0f;
             uint32_t o[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -281,7 +301,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     }
     // nobody leaves while a peer may still read its shared memory
     __syncwarp();
-    cluster_sync_all();
+    cluster_sync_relaxed();
 
     tc_fence_before();
     __syncthreads();
