@@ -10,9 +10,9 @@
 //               (tcgen05.cp), issues four tcgen05.mma.sp kind::f16 (K = 32 logical each) into a
 //               tensor-memory fp32 accumulator, commits to the stage's empty barrier; after the
 //               last K block commits to the accumulator's full barrier
-//   warps 2..5  epilogue: tcgen05.ld the accumulator (each warp its 32-lane quarter), apply
-//               row scale / bias / residual, round to bf16, stage in swizzled shared memory and
-//               TMA-store 32 x 64 boxes
+//   warps 4..11 epilogue (epilogue.cuh): read the accumulator (two warps per 32-lane quarter), apply
+//               row scale / bias / residual, round to bf16, stage in shared memory and TMA-store
+//   (warps 2, 3 only make the first warpgroup whole: register shares go by warpgroup)
 // With two accumulator buffers the epilogue of tile i overlaps the main loop of tile i+1.
 //
 // The producer and the issuer are whole warps that run their loops converged; waits end in a vote and

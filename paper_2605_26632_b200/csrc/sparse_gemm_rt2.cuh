@@ -1,19 +1,18 @@
 // 2:4 sparse x dense GEMM, "two row tiles per W stage" form (Algorithm 1 lines 5-6):
 //     Y[m, n] = bf16( s_m * sum_k X~[m,k] W[n,k] + bias[n] + Yr[m,n] )
 //
-// Why a second kernel.  The main loop of sparse_gemm_kernel is bound by the operand stream into
-// each SM, and that stream is bound by latency x bytes in flight (a load-only run of the same
-// loop delivers 89 / 134 / 165 GB/s per SM with 2 / 3 / 4 stages of 48 KB in flight: ~1.1 us per
-// round trip), while the sparse MMAs of a 256 x 240 stage need only 0.28 us.  Shared memory is
-// full, so the only lever left is flops per byte in flight.  Here a CTA pair works on TWO 256-row
-// tiles of the same 240 columns at once ("double"): a ring stage holds two compressed-A tiles and
-// two metadata blocks per CTA but ONE W tile, 66 KB for twice the MMAs of the 48 KB stage (-31 %
-// bytes per flop).  The two accumulators fill all of tensor memory (2 x 240 columns + metadata),
-// so the epilogue of a double is not hidden behind a following main loop; it is therefore made
-// short: eight epilogue warps (four per accumulator), tcgen05.ld of the next column chunk in flight
-// while the current one is converted; each warp stages its 32 x 48 chunk in a 3 KB box of its own
-// and hands it to a TMA store.  (Storing straight from registers -- 16 bytes per lane, every lane
-// another row -- was measured first: 5.6 us per 512-row item, more than the main loop gained.)
+// Why a second kernel.  A CTA pair works on TWO 256-row tiles of the same 240 columns at once
+// ("double"): a ring stage holds two compressed-A tiles and two metadata blocks per CTA but ONE W
+// tile, 66 KB for twice the MMAs of the single-tile kernel's 48 KB stage (-31 % bytes per flop).  The
+// eight MMAs of a stage take 960 cycles and the loop runs at 950-1050 per stage; a single's four take
+// 480 and its loop runs at 530-650, because 48 KB per 480 cycles is more than a CTA gets (84 B/clk with no
+// MMAs at all).  Under the power cap, which launches of this size reach within milliseconds, the bytes
+// not moved count again: 4096 x 3072 x 12288 runs 121.7 us in doubles, 127.1 us in singles
+// (sustained 140.8 against 148.1).
+// The two accumulators fill all of tensor memory (2 x 240 columns + metadata), so the epilogue
+// of a double is not hidden behind a following main loop: the eight epilogue warps read the first accumulator as
+// soon as its last MMA is done, then the second, and the issuer starts the next item on the first while
+// the second is read.  What remains is about 2500 cycles per double (24000 of MMAs at K = 3072).
 //
 // Work items of a cluster: "doubles" (512 x 240) first, then "singles" (256 x 240, the tile of
 // sparse_gemm_kernel; consecutive singles alternate between the two accumulators, so their
@@ -21,8 +20,8 @@
 // choice (PairSchedule, a cost model): doubles cost less per unit, singles fill the clusters that
 // would otherwise idle in the last round.
 //
-// Roles per CTA (320 threads): warp 0 TMA producer, warp 1 MMA issuer (leader CTA, one thread),
-// warps 2-5 epilogue of accumulator 0, warps 6-9 epilogue of accumulator 1.  Every wait is
+// Roles per CTA (384 threads): warp 0 TMA producer, warp 1 MMA issuer (leader CTA), both converged with
+// one elected lane issuing (see sparse_gemm.cuh), warps 2 and 3 idle, warps 4-11 epilogue.  Every wait is
 // bounded (mbar_wait): on expiry the kernel raises the error word and all roles leave.
 #pragma once
 
@@ -499,11 +498,21 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
             if (p.residual != nullptr) convert(std::true_type{});
             else convert(std::false_type{});
             if (!alive) continue;
+            // The stores compete with the operand stream of the next main loop, whose ring is too short to ride out
+            // 122 KB leaving at once: the 40 chunks of a CTA go one after the other, spread over 100 cycles per K
+            // block (a K block of a double takes 960), at most 3200.  4096 x 3072 x 12288 124.2 -> 122.2 us, 4352 x
+            // 3072 x 9216 101.4 -> 100.0; unlimited at K = 12288 the last stores delay what follows (layer + 1 %).
+            const long long t_store = clock64();
+            const int pace = (kblocks < 32 ? kblocks : 32) * 100 / Cfg::EPI_WARPS;
 #pragma unroll
             for (int slot = 0; slot < NCH; ++slot) {
                 if (slot >= slots) break;
                 int r, c;
                 chunk_of(slot, r, c);
+                if (!last) {
+                    const long long at = t_store + (long long)(slot * Cfg::EPI_WARPS + warp - GEMM_EPI_WARP0) * pace;
+                    for (int i = 0; i < 1000 && clock64() < at; ++i) __nanosleep(100);
+                }
                 const int n0 = tn * BN + c * CH;
                 // rows past M and columns past N are clipped by the store.  The last item stages in the ring:
                 // its MMAs are done (the wait above) and nothing is loaded any more.
