@@ -88,6 +88,7 @@ prune_compress_fp8_kernel(const uint16_t* __restrict__ X, int64_t M, int64_t K, 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid < 64) lut[tid] = prune_lut_entry(tid & 15, tid >> 4);
     griddep_wait();
+    griddep_launch_dependents();  // the GEMM's CTAs take the SMs as this grid's leave them and run their prologue
 
     const int64_t row0 = (int64_t)blockIdx.x * PRUNE_ROWS;
     const int r = lane >> 2, q = lane & 3;
@@ -261,6 +262,7 @@ prune_compress_fp8_ring_kernel(const uint16_t* __restrict__ X, int64_t M, int64_
     }
     __syncthreads();
     griddep_wait();
+    griddep_launch_dependents();  // the GEMM's CTAs take the SMs as this grid's leave them and run their prologue
 
     // this CTA's rows
     const int64_t G = gridDim.x, b = blockIdx.x;

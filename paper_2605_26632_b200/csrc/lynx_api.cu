@@ -620,7 +620,7 @@ lynx_status launch_gemm(lynx_ctx* ctx, const void* values, const void* meta, int
 template <class Cfg>
 lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void* meta, int64_t M, int64_t K,
                                 const void* Wq, int64_t N, int64_t ldwq, const float* wscale, const void* bias,
-                                const lynx_comp* comp, void* Y, int64_t ldy, cudaStream_t st) {
+                                const lynx_comp* comp, void* Y, int64_t ldy, cudaStream_t st, bool layer_call) {
     static_assert(Cfg::FP8, "FP8 configuration expected");
     CUtensorMap ta, tb, te, ty;
     const uint64_t rb = (uint64_t)((M + 127) / 128), kb128 = (uint64_t)(K / 128);
@@ -645,6 +645,7 @@ lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void*
     p.tiles_n = (int)((N + Cfg::BN - 1) / Cfg::BN);
     p.group_m = gemm_group_rows(ctx, p.tiles_m);
     p.l0_splits = 1;
+    p.w_prefetch = layer_call ? 1 : 0;
     auto kern = sparse_gemm_kernel<Cfg, false>;
     static bool attr_set[MAX_CTX_DEVICES] = {};  // per instantiation
     if (lynx_status as = allow_dynamic_smem(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
@@ -674,14 +675,14 @@ lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void*
 // choice among the same pair tiles (a stage is 256 K here; relative times as for bf16).
 lynx_status launch_gemm_fp8(lynx_ctx* ctx, const void* values_q, const void* meta, int64_t M, int64_t K,
                             const void* Wq, int64_t N, int64_t ldwq, const float* wscale, const void* bias,
-                            const lynx_comp* comp, void* Y, int64_t ldy, cudaStream_t st) {
+                            const lynx_comp* comp, void* Y, int64_t ldy, cudaStream_t st, bool layer_call = false) {
     int cfg = ctx->gemm_cfg;
     if (cfg != 4 && cfg != 6 && cfg != 7) {
         cfg = pick_gemm_cfg_model(ctx->num_sms, M, N, K / 2, 0);
         if (cfg == 8) cfg = 4;  // (FP8 stages are larger: four of them)
         if (cfg == 5) cfg = 7;  // the 256-wide tile has no FP8 instantiation (no tensor memory left for metadata)
     }
-#define LYNX_FP8_ARGS ctx, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, Y, ldy, st
+#define LYNX_FP8_ARGS ctx, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, Y, ldy, st, layer_call
     switch (cfg) {
         case 4: return launch_gemm_fp8_cfg<GemmCfg<192, 2, 4, 32, true>>(LYNX_FP8_ARGS);
         case 6: return launch_gemm_fp8_cfg<GemmCfg<128, 2, 5, 32, true>>(LYNX_FP8_ARGS);
@@ -1700,7 +1701,9 @@ lynx_status lynx_act_sparse_linear_fp8(lynx_ctx* ctx, const void* X, int64_t M, 
     comp.row_scale = scale;
     comp.residual = residual;
     comp.ldr = ldr;
-    return lynx_sparse_linear_fp8(ctx, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, &comp, Y, ldy, stream);
+    if ((s = check_device_error(ctx)) != LYNX_OK) return s;
+    return launch_gemm_fp8(ctx, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, &comp, Y, ldy,
+                           static_cast<cudaStream_t>(stream), true);
 }
 
 lynx_status lynx_meta_to_canonical(lynx_ctx* ctx, const void* meta, int64_t M, int64_t K, void* meta_canon,
