@@ -347,11 +347,15 @@ LYNX_API lynx_status lynx_selftest_wait_timeout(lynx_ctx* ctx, int64_t limit_us,
  * lynx_gemm_schedule_items lists the work items of CTA pair `cluster` for `tiles_m` x `tiles_n`
  * tiles of 256 x 240 over `clusters` pairs with `doubles` 512-row items: items[4i..4i+3] = first
  * row tile, column tile, row tiles (1 or 2), ordinal among the pair's single-tile items; returns
- * the item count (only the first `capacity` are written) or -1. */
+ * the item count (only the first `capacity` are written) or -1.
+ * lynx_gemm_accumulator_waits: the parities with which the MMA issuer waits for hand-backs when its items
+ * use the accumulator buffers order[0..n-1] (of `buffers`, 1 or 2): parities[i] before item i, then
+ * parities[n + a] for buffer a before the kernel ends; returns n + buffers or -1. */
 LYNX_API int lynx_gemm_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, int* doubles,
                             int* clusters);
 LYNX_API int lynx_gemm_schedule_items(int tiles_m, int tiles_n, int clusters, int doubles, int cluster,
                                       int* items, int capacity);
+LYNX_API int lynx_gemm_accumulator_waits(int buffers, const int* order, int n, int* parities);
 
 /* Number of kernels the library launched on this context since creation (for accounting). */
 LYNX_API int64_t lynx_launch_count(lynx_ctx* ctx);

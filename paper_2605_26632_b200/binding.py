@@ -24,7 +24,8 @@ EXPORTS = [
     "lynx_meta_to_canonical", "lynx_decompress", "lynx_launch_count", "lynx_prune_compress_static",
     "lynx_reserve_lora", "lynx_lora_down", "lynx_prune_compress_lora", "lynx_sparse_linear_lora", "lynx_act_sparse_linear_lora",
     "lynx_quantize_weights_fp8", "lynx_prune_compress_fp8", "lynx_sparse_linear_fp8",
-    "lynx_act_sparse_linear_fp8", "lynx_gemm_plan", "lynx_gemm_schedule_items", "lynx_selftest_wait_timeout",
+    "lynx_act_sparse_linear_fp8", "lynx_gemm_plan", "lynx_gemm_schedule_items", "lynx_gemm_accumulator_waits",
+    "lynx_selftest_wait_timeout",
 ]
 
 
@@ -102,6 +103,7 @@ def load_library() -> ctypes.CDLL:
                                                i64, vp]
     lib.lynx_gemm_plan.argtypes = [i32, i64, i64, i64, i32, ctypes.POINTER(i32), ctypes.POINTER(i32)]
     lib.lynx_gemm_schedule_items.argtypes = [i32, i32, i32, i32, i32, ctypes.POINTER(i32), i32]
+    lib.lynx_gemm_accumulator_waits.argtypes = [i32, ctypes.POINTER(i32), i32, ctypes.POINTER(i32)]
     lib.lynx_selftest_wait_timeout.argtypes = [vp, i64, vp]
     lib.lynx_launch_count.argtypes = [vp]
     lib.lynx_launch_count.restype = i64
@@ -138,6 +140,15 @@ def gemm_schedule_items(tiles_m: int, tiles_n: int, clusters: int, doubles: int,
     if n < 0:
         raise ValueError("lynx_gemm_schedule_items: bad arguments")
     return [tuple(buf[4 * i:4 * i + 4]) for i in range(n)]
+
+
+def gemm_accumulator_waits(buffers: int, order):
+    """-> parities of the MMA issuer's waits for hand-backs: one per item, then one per buffer (host only)."""
+    n = len(order)
+    src, out = (ctypes.c_int * max(n, 1))(*order), (ctypes.c_int * (n + buffers))()
+    if load_library().lynx_gemm_accumulator_waits(buffers, src, n, out) < 0:
+        raise ValueError("lynx_gemm_accumulator_waits: bad arguments")
+    return list(out)
 
 
 # Every call passes through these, and on the smallest layers (7 us of GPU work) the host side is what a caller waits

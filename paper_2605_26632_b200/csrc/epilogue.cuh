@@ -31,6 +31,31 @@ constexpr int GEMM_THREADS = 32 * (GEMM_EPI_WARP0 + GEMM_EPI_WARPS);
 constexpr int GEMM_REGS_ISSUE = 72, GEMM_REGS_EPI = 216;
 static_assert(128 * GEMM_REGS_ISSUE + 32 * GEMM_EPI_WARPS * GEMM_REGS_EPI <= GEMM_THREADS * 168, "register pool of the block");
 
+// Whose turn an accumulator buffer is: the issuer fills it once its previous contents were handed back, the
+// epilogue drains it once it is filled, and each of its two barriers completes one phase per use.  Bit a of the word
+// is the number of uses of buffer a so far, mod 2 (a bit each: an array with a run-time index lives in local memory).
+//
+// After its last item the issuer asks for every buffer once more, as if it were to fill it again.  The hand-backs
+// of CTA 1's epilogue warps are remote arrives on a barrier of CTA 0; without that wait nothing orders the last
+// of them before CTA 0 leaves and its shared memory is given away.  The producers do the same with the ring's stages,
+// whose release is a commit that arrives on both CTAs' barriers.  Neither is on the critical path: what they wait for
+// comes before the epilogue's last stores.
+struct AccTurns {
+    uint32_t odd = 0;
+    // parity of the hand-back barrier that lets the issuer fill buffer a (a fresh barrier passes)
+    __host__ __device__ uint32_t fill(int a) {
+        const uint32_t parity = ((odd >> a) & 1u) ^ 1u;
+        odd ^= 1u << a;
+        return parity;
+    }
+    // parity of the barrier that tells the epilogue that buffer a is filled
+    __host__ __device__ uint32_t drain(int a) {
+        const uint32_t parity = (odd >> a) & 1u;
+        odd ^= 1u << a;
+        return parity;
+    }
+};
+
 // One 32-row x CH-column chunk: v[half][4 g + 2 k + e] = row 16 half + 8 k + lane / 4, column 8 g + 2 (lane % 4) + e
 template <int CH>
 __device__ __forceinline__ void epi_tmem_ld(uint32_t taddr, uint32_t (&v)[2][CH / 2]) {

@@ -1749,6 +1749,17 @@ int lynx_gemm_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps,
     return (M > 256 && plan.t_us < gemm_model_time(num_sms, M, N, K, lora_steps)) ? 1 : 0;
 }
 
+int lynx_gemm_accumulator_waits(int buffers, const int* order, int n, int* parities) {
+    if (buffers < 1 || buffers > 2 || !order || n < 0 || !parities) return -1;
+    AccTurns turns;
+    for (int i = 0; i < n; ++i) {
+        if (order[i] < 0 || order[i] >= buffers) return -1;
+        parities[i] = (int)turns.fill(order[i]);
+    }
+    for (int a = 0; a < buffers; ++a) parities[n + a] = (int)turns.fill(a);
+    return n + buffers;
+}
+
 int lynx_gemm_schedule_items(int tiles_m, int tiles_n, int clusters, int doubles, int cluster, int* items, int capacity) {
     if (tiles_m < 1 || tiles_n < 1 || clusters < 1 || cluster < 0 || cluster >= clusters) return -1;
     PairSchedule sc;

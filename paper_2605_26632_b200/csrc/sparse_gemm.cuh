@@ -482,6 +482,10 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     }
                 }
             }
+            for (int s = 0; s < STAGES && ok; ++s) {  // the last releases of the stages (see AccTurns)
+                ok = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error);
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
             if (!ok && issued) bounded_delay_ns(200000);  // let the copies in flight land before teardown
         }
     } else if (warp == 1) {
@@ -496,6 +500,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
             constexpr uint32_t BH = Cfg::B_HALF_BYTES >> 4;
             uint32_t stage = 0, phase = 0;
             bool ok = true;
+            AccTurns turns;
             if constexpr (L0) {
                 // phase 0: eight dense K = 16 steps per stage into the first 64 accumulator columns
                 constexpr uint32_t idesc_l0 = make_idesc_sp_bf16(Cfg::BM * CG, Cfg::L0_R) & ~(1u << 2);
@@ -505,8 +510,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     const int k0 = split * p.l0_kb_per_split;
                     const int k1 = (k0 + p.l0_kb_per_split < kblocks) ? k0 + p.l0_kb_per_split : kblocks;
                     const int acc = (Cfg::ACC_STAGES == 2) ? (li & 1) : 0;
-                    const uint32_t acc_phase = (Cfg::ACC_STAGES == 2) ? ((li >> 1) & 1) : (li & 1);
-                    if (!mbar_wait_warp(bar_tempty + 8 * acc, acc_phase ^ 1, cta_abort, p.dev_error)) {
+                    if (!mbar_wait_warp(bar_tempty + 8 * acc, turns.fill(acc), cta_abort, p.dev_error)) {
                         ok = false;
                         break;
                     }
@@ -543,13 +547,12 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     }
                 }
             }
-            int it = 0;
-            for (; it < num_items && ok; ++it) {
+            for (int it = 0; it < num_items && ok; ++it) {
                 const WorkItem w = sched.get(cluster_id, it);
                 const int gi = l0_n + it;  // accumulator buffers alternate over phase 0 items and tiles alike
                 const int acc = (Cfg::ACC_STAGES == 2) ? (gi & 1) : 0;
-                const uint32_t acc_phase = (Cfg::ACC_STAGES == 2) ? ((gi >> 1) & 1) : (gi & 1);
-                if (!mbar_wait_warp(bar_tempty + 8 * acc, acc_phase ^ 1, cta_abort, p.dev_error)) break;
+                ok = mbar_wait_warp(bar_tempty + 8 * acc, turns.fill(acc), cta_abort, p.dev_error);
+                if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 uint32_t accumulate = 0;
@@ -616,6 +619,8 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     else tc_commit_pair(bar_tfull + 8 * acc, 0x3);
                 }
             }
+            for (int a = 0; a < Cfg::ACC_STAGES && ok; ++a)  // the last hand-backs (see AccTurns)
+                ok = mbar_wait_warp(bar_tempty + 8 * a, turns.fill(a), cta_abort, p.dev_error);
         }
     }
     } else {
@@ -626,6 +631,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
         const uint32_t own_box = sC + (warp - GEMM_EPI_WARP0) * Cfg::BOX_BYTES;
         const uint32_t tempty0 = (CG == 2) ? mapa(bar_tempty, 0) : bar_tempty;
         bool alive = true;
+        AccTurns turns;
         if constexpr (L0) {
             // ---- phase 0: drain the 64-column accumulator of each (row block, K split) item (the first
             //      four warps; the others only hand the accumulator back) ----
@@ -635,7 +641,6 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 const int item = l0s.item(cluster_id, li);
                 const int tmb = item % p.tiles_m, split = item / p.tiles_m;
                 const int acc = (Cfg::ACC_STAGES == 2) ? (li & 1) : 0;
-                const uint32_t acc_phase = (Cfg::ACC_STAGES == 2) ? ((li >> 1) & 1) : (li & 1);
                 const int row_in_block = (int)rank * Cfg::BM + q * 32 + lane;
                 const int64_t row = (int64_t)tmb * BLOCK_ROWS + row_in_block;
                 // the row's scale is fetched while the item's K loop runs (a global load costs over a
@@ -646,7 +651,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                                                                   : __ldg(p.row_scale + row);
                     inv_s = (sc == 0.0f) ? 0.0f : __frcp_rn(sc);
                 }
-                if (!mbar_wait(bar_tfull + 8 * acc, acc_phase, cta_abort, p.dev_error)) {
+                if (!mbar_wait(bar_tfull + 8 * acc, turns.drain(acc), cta_abort, p.dev_error)) {
                     alive = false;
                     break;
                 }
@@ -748,7 +753,6 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
             const bool last = it == num_items - 1;
             const int gi = l0_n + it;
             const int acc = (Cfg::ACC_STAGES == 2) ? (gi & 1) : 0;
-            const uint32_t acc_phase = (Cfg::ACC_STAGES == 2) ? ((gi >> 1) & 1) : (gi & 1);
             // the tile's per-column terms as fp32, for all epilogue warps (the other parity's may still be read)
             const uint32_t sb = sStrip + (it & 1) * Cfg::STRIP_BYTES, sc = sb + BN * 4;
             if (const int c = (int)threadIdx.x - 32 * GEMM_EPI_WARP0; c < BN) {
@@ -789,7 +793,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                                 epi_load_residual<CH>(p.residual, p.ldr, m0, p.M, tn * BN + (c0 + slot) * CH, p.N, lane, packed[slot]);
                     }
                 }
-                alive = mbar_wait_warp(bar_tfull + 8 * acc, acc_phase, cta_abort, p.dev_error);
+                alive = mbar_wait_warp(bar_tfull + 8 * acc, turns.drain(acc), cta_abort, p.dev_error);
                 if (!alive) return;
                 tc_fence_after();
                 if (w.kind == 2) {

@@ -310,6 +310,12 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     if (++stage == nst) { stage = 0; phase ^= 1; }
                 }
             }
+            // the last releases of the stages (see AccTurns; a switch of the rings has waited for the other one's)
+            const uint32_t nst = ring1 ? (uint32_t)Cfg::STAGES1 : (uint32_t)STAGES, bempty = ring1 ? bar_empty1 : bar_empty;
+            for (uint32_t s = 0; s < nst && ok; ++s) {
+                ok = mbar_wait_warp(bempty + 8 * stage, phase ^ 1, cta_abort, p.dev_error);
+                if (++stage == nst) { stage = 0; phase ^= 1; }
+            }
             if (!ok && issued) bounded_delay_ns(200000);  // let the copies in flight land before teardown
         }
     } else if (warp == 1) {
@@ -325,7 +331,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
             constexpr uint32_t BH = Cfg::B_HALF_BYTES >> 4;
             uint32_t stage = 0, phase = 0;
             bool ring1 = false;
-            uint32_t uses[2] = {0u, 0u};  // how often each accumulator has been handed to the epilogue
+            AccTurns turns;
             bool ok = true;
             for (int it = 0; it < num_items && ok; ++it) {
                 int tm0, tn, rows, ordinal;
@@ -341,7 +347,8 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                 const int acc0 = (rows == 2) ? 0 : (ordinal & 1);
                 // (a double's second accumulator is waited for behind the first one's MMAs: the epilogue
                 // hands them back one after the other)
-                if (!mbar_wait_warp(bar_tempty + 8 * acc0, (uses[acc0] & 1u) ^ 1u, cta_abort, p.dev_error)) break;
+                ok = mbar_wait_warp(bar_tempty + 8 * acc0, turns.fill(acc0), cta_abort, p.dev_error);
+                if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc0 * BN;
                 const int ksteps = kblocks + lora_steps;
@@ -388,7 +395,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     }
                     if (rows == 2) {
                         if (kb == 0) {
-                            if (!mbar_wait_warp(bar_tempty + 8, (uses[1] & 1u) ^ 1u, cta_abort, p.dev_error)) {
+                            if (!mbar_wait_warp(bar_tempty + 8, turns.fill(1), cta_abort, p.dev_error)) {
                                 ok = false;
                                 break;
                             }
@@ -403,8 +410,9 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     accumulate = 1u;
                     if (++stage == nst) { stage = 0; phase ^= 1; }
                 }
-                for (int r = 0; r < rows; ++r) ++uses[acc0 + r];
             }
+            for (int a = 0; a < 2 && ok; ++a)  // the last hand-backs (see AccTurns)
+                ok = mbar_wait_warp(bar_tempty + 8 * a, turns.fill(a), cta_abort, p.dev_error);
         }
     }
     } else {
@@ -418,7 +426,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         const uint32_t own_box = sC + (warp - GEMM_EPI_WARP0) * Cfg::C_BOX_BYTES;
         constexpr int CH = Cfg::CH, NCH = Cfg::NCH;
         const int n_first = h == 0 ? 3 : 2;  // chunks of the item's first accumulator
-        uint32_t uses[2] = {0u, 0u};
+        AccTurns turns;
         bool alive = true;
         for (int it = 0; it < num_items; ++it) {
             int tm0, tn, rows, ordinal;
@@ -475,9 +483,8 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     chunk_of(slot, r, c);
                     const int acc = acc0 + r;
                     if (slot == 0 || slot == n_first) {
-                        alive = mbar_wait_warp(bar_tfull + 8 * acc, uses[acc] & 1u, cta_abort, p.dev_error);
+                        alive = mbar_wait_warp(bar_tfull + 8 * acc, turns.drain(acc), cta_abort, p.dev_error);
                         if (!alive) break;
-                        ++uses[acc];
                         tc_fence_after();
                     }
                     uint32_t v[2][CH / 2];

@@ -35,6 +35,33 @@ def test_size_helpers():
     assert lib.lynx_workspace_bytes(256, 512, 512) >= 256 * 256 * 2 + 2 * 4 * 2048 + 256 * 4
 
 
+def test_no_accumulator_hand_back_is_outstanding_when_the_gemm_ends():
+    """The MMA issuer's waits, against barriers that complete a phase per hand-back and an epilogue that hands back as
+    late as it can: no buffer is filled before its contents were handed back, and when the issuer is through
+    every hand-back has arrived (they are remote arrives on its CTA's shared memory)."""
+    import random
+
+    from paper_2605_26632_b200 import binding
+
+    rng = random.Random(1)
+    orders = [(b, [i % b for i in range(n)]) for b in (1, 2) for n in range(6)]  # one after the other, as single tiles are
+    orders += [(2, [0, 1] * d + [i % 2 for i in range(s)]) for d in range(4) for s in range(4)]  # doubles, then singles
+    orders += [(2, [rng.randint(0, 1) for _ in range(rng.randint(1, 9))]) for _ in range(40)]
+    for buffers, order in orders:
+        waits = binding.gemm_accumulator_waits(buffers, order)
+        assert len(waits) == len(order) + buffers
+        filled, back = [0] * buffers, [0] * buffers
+        for i, parity in enumerate(waits):
+            a = order[i] if i < len(order) else i - len(order)
+            while (back[a] & 1) == parity:  # the phase with this parity is not complete: the issuer waits
+                assert back[a] < filled[a], ("waits for ever", buffers, order, i)
+                back[a] += 1
+            assert back[a] == filled[a], ("not handed back yet", buffers, order, i)
+            if i < len(order):
+                filled[a] += 1
+        assert back == filled, (buffers, order)
+
+
 def test_two_row_tile_schedule_covers_every_tile_exactly_once():
     """Host logic of the GEMM's work distribution: for any number of row tiles, column tiles,
     CTA pairs and 512-row items, every 256 x 240 tile is computed exactly once, doubles pair the
