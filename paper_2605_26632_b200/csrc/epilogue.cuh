@@ -29,7 +29,13 @@ constexpr int GEMM_THREADS = 32 * (GEMM_EPI_WARP0 + GEMM_EPI_WARPS);
 // Register shares (per thread) of the two kinds of warpgroups; 128 * 72 + 256 * 216 = the 384 * 168 the block is
 // launched with.  An epilogue warp holds up to five packed chunks beside the one it converts.
 constexpr int GEMM_REGS_ISSUE = 72, GEMM_REGS_EPI = 216;
-static_assert(128 * GEMM_REGS_ISSUE + 32 * GEMM_EPI_WARPS * GEMM_REGS_EPI <= GEMM_THREADS * 168, "register pool of the block");
+// Do the shares fit what a block launched with `regs` registers per thread owns?  If not, the epilogue's
+// setmaxnreg.inc waits for ever; how many a kernel is launched with is the compiler's choice, so the host asks
+// the built kernel before its first launch.
+constexpr bool gemm_register_shares_fit(int regs) {
+    return 128 * GEMM_REGS_ISSUE + 32 * GEMM_EPI_WARPS * GEMM_REGS_EPI <= GEMM_THREADS * regs;
+}
+static_assert(gemm_register_shares_fit(65536 / GEMM_THREADS / 8 * 8), "register pool of the block");
 
 // Whose turn an accumulator buffer is: the issuer fills it once its previous contents were handed back, the
 // epilogue drains it once it is filled, and each of its two barriers completes one phase per use.  Bit a of the word

@@ -149,6 +149,16 @@ lynx_status allow_dynamic_smem(Kernel kern, int bytes, int device, bool (&done)[
     return LYNX_OK;
 }
 
+// The same for the kernels that move registers between their warpgroups.
+template <class Kernel>
+lynx_status prepare_gemm_kernel(Kernel kern, int bytes, int device, bool (&done)[MAX_CTX_DEVICES]) {
+    if (device >= 0 && device < MAX_CTX_DEVICES && !done[device]) {
+        cudaFuncAttributes fa;
+        if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || !gemm_register_shares_fit(fa.numRegs)) return LYNX_ERR_CUDA;
+    }
+    return allow_dynamic_smem(kern, bytes, device, done);
+}
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 lynx_status check_device_error(lynx_ctx* ctx) {
@@ -382,7 +392,7 @@ lynx_status launch_gemm_cfg(lynx_ctx* ctx, const void* values, const void* meta,
 
     auto kern = lora ? sparse_gemm_kernel<Cfg, true> : sparse_gemm_kernel<Cfg, false>;
     static bool attr_set[2][MAX_CTX_DEVICES] = {};  // per instantiation (with / without the low-rank code)
-    if (lynx_status as = allow_dynamic_smem(kern, Cfg::SMEM_BYTES, ctx->device, attr_set[lora ? 1 : 0]); as != LYNX_OK)
+    if (lynx_status as = prepare_gemm_kernel(kern, Cfg::SMEM_BYTES, ctx->device, attr_set[lora ? 1 : 0]); as != LYNX_OK)
         return as;
     const int tiles = p.tiles_m * p.tiles_n;
     int clusters = ctx->num_sms / Cfg::CG;
@@ -534,7 +544,7 @@ lynx_status launch_gemm_rt2(lynx_ctx* ctx, const Rt2Plan& plan, const void* valu
     p.w_prefetch = layer_call ? 1 : 0;
     auto kern = sparse_gemm_rt2_kernel<Cfg, LORA>;
     static bool attr_set[MAX_CTX_DEVICES] = {};  // per instantiation
-    if (lynx_status as = allow_dynamic_smem(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
+    if (lynx_status as = prepare_gemm_kernel(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(plan.clusters * 2));
     cfg.blockDim = dim3(Cfg::THREADS);
@@ -648,7 +658,7 @@ lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void*
     p.w_prefetch = layer_call ? 1 : 0;
     auto kern = sparse_gemm_kernel<Cfg, false>;
     static bool attr_set[MAX_CTX_DEVICES] = {};  // per instantiation
-    if (lynx_status as = allow_dynamic_smem(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
+    if (lynx_status as = prepare_gemm_kernel(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
     const int tiles = p.tiles_m * p.tiles_n;
     int clusters = ctx->num_sms / Cfg::CG;
     if (clusters > tiles) clusters = tiles;
@@ -1748,6 +1758,8 @@ int lynx_gemm_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps,
     if (clusters) *clusters = plan.clusters;
     return (M > 256 && plan.t_us < gemm_model_time(num_sms, M, N, K, lora_steps)) ? 1 : 0;
 }
+
+int lynx_gemm_register_shares_fit(int regs_per_thread) { return gemm_register_shares_fit(regs_per_thread) ? 1 : 0; }
 
 int lynx_gemm_accumulator_waits(int buffers, const int* order, int n, int* parities) {
     if (buffers < 1 || buffers > 2 || !order || n < 0 || !parities) return -1;

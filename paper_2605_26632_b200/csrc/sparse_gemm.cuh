@@ -227,6 +227,7 @@ struct GemmCfg {
     static constexpr int THREADS = GEMM_THREADS;
     static_assert(BN % 16 == 0 && (BN / CG) % 8 == 0 && BN <= 256, "tile N");
     static_assert(BN % CH == 0, "epilogue works on whole chunks");
+    static_assert(NCH >= 2, "an epilogue warp without a chunk would never hand the accumulator back");
     static_assert(CH == 48 || BOX_BYTES % 1024 == 0, "swizzled staging boxes stay 1024-byte aligned");
     static_assert(EPI_WARPS * SLOTS * 32 * CH * 2 <= STAGES * STAGE_BYTES, "last tile: a staging box per chunk in the ring");
     static_assert(B_HALF_BYTES % 1024 == 0, "swizzle atoms need 1024-byte aligned tiles");

@@ -62,6 +62,20 @@ def test_no_accumulator_hand_back_is_outstanding_when_the_gemm_ends():
         assert back == filled, (buffers, order)
 
 
+def test_gemm_kernels_with_too_few_registers_are_refused():
+    """The GEMM's warps take 72 and 216 registers out of what 384 threads were launched with: 168 is the least."""
+    from paper_2605_26632_b200 import binding
+
+    fit = binding.load_library().lynx_gemm_register_shares_fit
+    assert fit(168) == 1 and fit(167) == 0 and fit(160) == 0 and fit(128) == 0
+    # every launch of such a kernel goes through the check
+    src = open(os.path.join(ROOT, "paper_2605_26632_b200", "csrc", "lynx_api.cu")).read()
+    for launch in ("launch_gemm_cfg", "launch_gemm_rt2", "launch_gemm_fp8_cfg"):
+        body = src[src.index(f"lynx_status {launch}(lynx_ctx"):]
+        body = body[:body.index("cudaLaunchKernelEx")]
+        assert "prepare_gemm_kernel(" in body and "allow_dynamic_smem(" not in body, launch
+
+
 def test_two_row_tile_schedule_covers_every_tile_exactly_once():
     """Host logic of the GEMM's work distribution: for any number of row tiles, column tiles,
     CTA pairs and 512-row items, every 256 x 240 tile is computed exactly once, doubles pair the
