@@ -322,7 +322,7 @@ prune_compress_fp8_ring_kernel(const uint16_t* __restrict__ X, int64_t M, int64_
             const float amax_given = amax_next;
             if (GIVEN && i + NG < count) amax_next = __ldg(row_amax + start + i + NG);
             const int slot = first + ls;
-            bool ok = mbar_wait(bar_full + 8 * slot, use & 1, cta_abort, dev_error);
+            bool ok = mbar_wait_warp(bar_full + 8 * slot, use & 1, cta_abort, dev_error);
             const uint32_t sbase = data + (uint32_t)slot * row_bytes;
             // ---- pass 1: the row's largest magnitude
             uint32_t m = 0;

@@ -171,7 +171,7 @@ fused_linear_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++it) {
             float num = 0.f, den = 0.f;
             for (int kb = 0; kb < kblocks; ++kb) {
-                if (!mbar_wait(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) { ok = false; break; }
+                if (!mbar_wait_warp(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) { ok = false; break; }
                 const uint32_t xrow = sX + stage * Cfg::X_BYTES + (uint32_t)r * 128;
                 const uint32_t erow = sE + stage * Cfg::E_BYTES + e_row;
 #pragma unroll
@@ -248,7 +248,7 @@ fused_linear_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         int it = 0;
         for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++it) {
             const int tm = t % p.tiles_m, tn = t / p.tiles_m;
-            if (!mbar_wait(bar_tfull, (uint32_t)(it & 1), cta_abort, p.dev_error)) break;
+            if (!mbar_wait_warp(bar_tfull, (uint32_t)(it & 1), cta_abort, p.dev_error)) break;
             tc_fence_after();
             const int m0 = tm * Cfg::BM + q * 32;
             const int64_t row = m0 + lane;

@@ -144,7 +144,7 @@ lora_down_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         const int r_in_tile = q * 32 + lane;
         const int64_t row = (int64_t)tm * Cfg::BM + r_in_tile;
         const bool row_ok = row < p.M;
-        bool alive = mbar_wait(bar_done, 0, cta_abort, p.dev_error);
+        bool alive = mbar_wait_warp(bar_done, 0, cta_abort, p.dev_error);
         if (alive) {
             tc_fence_after();
             const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);

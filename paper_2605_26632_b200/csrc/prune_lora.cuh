@@ -183,7 +183,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         float numA = 0.f, denA = 0.f, numB = 0.f, denB = 0.f;
         uint32_t stage = 0, phase = 0;
         for (int kb = kb0; kb < kb1; ++kb) {
-            if (!mbar_wait(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) break;
+            if (!mbar_wait_warp(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) break;
             const uint32_t base = sX + stage * Cfg::X_BYTES + offA;
             uint32_t a0[8], a1[8], b0[8], b1[8];
             lds128(base + (((c0 + 0) ^ sw) << 4), a0[0], a0[1], a0[2], a0[3]);
@@ -227,7 +227,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // consecutive lanes write consecutive 16-byte slots
         const int q = warp & 3;  // tensor-memory lane quarter this warp may read
         const int r_in_tile = q * 32 + lane;
-        const bool alive = mbar_wait(bar_done, 0, cta_abort, p.dev_error);  // every MMA has retired: sB is free
+        const bool alive = mbar_wait_warp(bar_done, 0, cta_abort, p.dev_error);  // every MMA has retired: sB is free
         if (alive) {
             tc_fence_after();
             const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);

@@ -652,7 +652,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                                                                   : __ldg(p.row_scale + row);
                     inv_s = (sc == 0.0f) ? 0.0f : __frcp_rn(sc);
                 }
-                if (!mbar_wait(bar_tfull + 8 * acc, turns.drain(acc), cta_abort, p.dev_error)) {
+                if (!mbar_wait_warp(bar_tfull + 8 * acc, turns.drain(acc), cta_abort, p.dev_error)) {
                     alive = false;
                     break;
                 }

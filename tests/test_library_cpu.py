@@ -76,6 +76,30 @@ def test_gemm_kernels_with_too_few_registers_are_refused():
         assert "prepare_gemm_kernel(" in body and "allow_dynamic_smem(" not in body, launch
 
 
+def test_waits_of_whole_warps_end_alike_for_every_lane():
+    """A bounded wait may give up, and each lane sees that for itself.  What a whole warp does behind a wait (tensor-memory
+    reads, shuffles, warp barriers) needs all lanes, so only code of a single lane (or of lanes that feed a group of slots each) calls the per-lane form."""
+    csrc = os.path.join(ROOT, "paper_2605_26632_b200", "csrc")
+    found = 0
+    for name in sorted(os.listdir(csrc)):
+        if name == "ptx.cuh":  # where both forms are defined
+            continue
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        headers, start = [], 0  # for every open brace the text in front of it
+        for i, ch in enumerate(text):
+            if ch == "{":
+                headers.append(text[start:i])
+            elif ch == "}":
+                headers.pop()
+            if ch in "{};":
+                start = i + 1
+            if text.startswith("mbar_wait(", i) and not text[i - 1].isalnum() and text[i - 1] != "_":
+                found += 1
+                one_lane = any(re.search(r"if \([^)]*\b(lane|threadIdx\.x) (== 0|< NG\b)", h) for h in headers)
+                assert one_lane, (name, text.count("\n", 0, i) + 1)
+    assert found >= 5
+
+
 def test_two_row_tile_schedule_covers_every_tile_exactly_once():
     """Host logic of the GEMM's work distribution: for any number of row tiles, column tiles,
     CTA pairs and 512-row items, every 256 x 240 tile is computed exactly once, doubles pair the
