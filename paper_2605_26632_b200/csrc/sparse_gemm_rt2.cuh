@@ -150,6 +150,18 @@ struct Gemm2Cfg {
     static constexpr int C_BYTES = EPI_WARPS * C_BOX_BYTES;
     static constexpr int BIAS_BYTES = BN * 4;          // the item's bias values (fp32), two items' worth
     static constexpr int SMEM_BYTES = 1024 /*align slack*/ + STAGES * STAGE_BYTES + C_BYTES + 2 * BIAS_BYTES + 256;
+    // Cycles from one chunk store of a CTA to the next.  The stores compete with the operand stream of the next main
+    // loop, whose ring is too short to ride out 122 KB leaving at once: a double's 40 chunks go one after the other,
+    // spread over 500 cycles per K block (a K block of a double takes 960, of a single 530-650), at most 16000 in
+    // all: 4096 x 3072 x 12288 122.1 -> 120.0 us, 4352 x 3072 x 9216 100.2 -> 98.7 (over 100 cycles per K block: 122.5
+    // and 99.7); without a limit the last stores at K = 12288 delay what follows (layer + 1 %).
+    // With a residual they go at once: a warp fetches the next item's only behind its last store, and fetched late
+    // it holds up that item's epilogue: 4352 x 3072 x 9216 115.1 -> 112.1 us, 4352 x 3072 x 3072 40.6 -> 39.7.
+    __host__ __device__ static constexpr int store_pace(int kblocks, bool residual) {
+        return residual ? 0 : (kblocks < 32 ? kblocks : 32) * 100 / EPI_WARPS;
+    }
+    static_assert(store_pace(24, false) * NCH * EPI_WARPS == 500 * 24 && store_pace(96, false) * NCH * EPI_WARPS == 16000 &&
+                      store_pace(24, true) == 0, "spread of a double's chunk stores");
     static_assert(NCH == 5 && BN % CH == 0 && BN_CTA % 8 == 0, "tile N: the epilogue deals five chunks per accumulator");
     static_assert(EPI_WARPS * 5 * C_BOX_BYTES <= STAGES * STAGE_BYTES, "last item: a staging box per chunk in the ring");
     static_assert(B_HALF_BYTES % 1024 == 0, "swizzle atoms need 1024-byte aligned tiles");
@@ -505,18 +517,14 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
             if (p.residual != nullptr) convert(std::true_type{});
             else convert(std::false_type{});
             if (!alive) continue;
-            // The stores compete with the operand stream of the next main loop, whose ring is too short to ride out
-            // 122 KB leaving at once: the 40 chunks of a CTA go one after the other, spread over 100 cycles per K
-            // block (a K block of a double takes 960), at most 3200.  4096 x 3072 x 12288 124.2 -> 122.2 us, 4352 x
-            // 3072 x 9216 101.4 -> 100.0; unlimited at K = 12288 the last stores delay what follows (layer + 1 %).
             const long long t_store = clock64();
-            const int pace = (kblocks < 32 ? kblocks : 32) * 100 / Cfg::EPI_WARPS;
+            const int pace = Cfg::store_pace(kblocks, p.residual != nullptr);
 #pragma unroll
             for (int slot = 0; slot < NCH; ++slot) {
                 if (slot >= slots) break;
                 int r, c;
                 chunk_of(slot, r, c);
-                if (!last) {
+                if (pace > 0 && !last) {
                     const long long at = t_store + (long long)(slot * Cfg::EPI_WARPS + warp - GEMM_EPI_WARP0) * pace;
                     for (int i = 0; i < 1000 && clock64() < at; ++i) __nanosleep(100);
                 }
