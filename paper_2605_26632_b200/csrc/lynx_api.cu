@@ -570,23 +570,33 @@ lynx_status launch_gemm_rt2(lynx_ctx* ctx, const Rt2Plan& plan, const void* valu
 // measured B200 launches of each tile (us): 1024 x 3072 x 3072 14.5 with 192 against 16.1 with 240,
 // 4352 x 3072 x 3072 37.4 against 36.2, 1024 x 3072 x 9216 28.6 with 256 (two rounds) against 30.0 with
 // 192 (three).  The 256-wide tile has one accumulator buffer, so its epilogue is not hidden.
-int pick_gemm_cfg_model(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, double* t_us = nullptr) {
+struct TileCost {
+    int id, bn;
+    double t_kb, epi;
+};
+// (the 192-wide tile runs with five stages of 42 KB, id 8)
+constexpr TileCost BF16_TILES[4] = {{7, 240, 0.41, 0.3}, {5, 256, 0.425, 2.0}, {8, 192, 0.325, 0.7}, {6, 128, 0.27, 0.6}};
+template <int NT>
+const TileCost& pick_tile(const TileCost (&tiles)[NT], int num_sms, int64_t M, int64_t N, double kb, double* t_us = nullptr) {
     const int pairs = num_sms / 2;
-    const double kb = (double)(K / 128) + lora_steps;
-    // (the 192-wide tile runs with five stages of 42 KB, id 8)
-    struct { int id, bn; double t_kb, epi; } cand[4] = {
-        {7, 240, 0.41, 0.3}, {5, 256, 0.425, 2.0}, {8, 192, 0.325, 0.7}, {6, 128, 0.27, 0.6}};
     double best = 1e30;
-    int cfg = 7;
-    for (auto& c : cand) {
-        const int64_t tiles = ((M + 255) / 256) * ((N + c.bn - 1) / c.bn);
-        const double rounds = (double)((tiles + pairs - 1) / pairs);
-        const double t = rounds * (kb * c.t_kb + c.epi);
-        if (t < best) { best = t; cfg = c.id; }
+    const TileCost* pick = &tiles[0];
+    for (const TileCost& c : tiles) {
+        const int64_t n = ((M + 255) / 256) * ((N + c.bn - 1) / c.bn);
+        const double t = (double)((n + pairs - 1) / pairs) * (kb * c.t_kb + c.epi);
+        if (t < best) { best = t; pick = &c; }
     }
     if (t_us) *t_us = best;
-    return cfg;
+    return *pick;
 }
+int pick_gemm_cfg_model(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, double* t_us = nullptr) {
+    return pick_tile(BF16_TILES, num_sms, M, N, (double)(K / 128) + lora_steps, t_us).id;
+}
+// The FP8 kernel's tiles (256 K per block; the 256-wide tile leaves no tensor memory for the metadata, the 192-wide
+// one has four stages): fits to launches of 57 products (64 ... 16138 rows); the choice is within 1 % of the fastest
+// tile on all of them.  With the bf16 times, and 240 in place of a 256, it was up to 26 % slower.
+// 1024 x 3072 x 4608 runs in two rounds of any of them: 12.8 us with 128, 14.8 with 192, 16.3 with 240.
+constexpr TileCost FP8_TILES[3] = {{7, 240, 0.412, 1.29}, {4, 192, 0.397, 0.50}, {6, 128, 0.296, 0.53}};
 double gemm_model_time(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps) {
     double t = 0.0;
     pick_gemm_cfg_model(num_sms, M, N, K, lora_steps, &t);
@@ -681,17 +691,12 @@ lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void*
     return LYNX_OK;
 }
 
-// FP8 tile choice: the development override if it names a CTA-pair tile, else the cost model's
-// choice among the same pair tiles (a stage is 256 K here; relative times as for bf16).
+// FP8 tile choice: the development override if it names a CTA-pair tile, else the cost model's.
 lynx_status launch_gemm_fp8(lynx_ctx* ctx, const void* values_q, const void* meta, int64_t M, int64_t K,
                             const void* Wq, int64_t N, int64_t ldwq, const float* wscale, const void* bias,
                             const lynx_comp* comp, void* Y, int64_t ldy, cudaStream_t st, bool layer_call = false) {
     int cfg = ctx->gemm_cfg;
-    if (cfg != 4 && cfg != 6 && cfg != 7) {
-        cfg = pick_gemm_cfg_model(ctx->num_sms, M, N, K / 2, 0);
-        if (cfg == 8) cfg = 4;  // (FP8 stages are larger: four of them)
-        if (cfg == 5) cfg = 7;  // the 256-wide tile has no FP8 instantiation (no tensor memory left for metadata)
-    }
+    if (cfg != 4 && cfg != 6 && cfg != 7) cfg = pick_tile(FP8_TILES, ctx->num_sms, M, N, (double)(K / 256)).id;
 #define LYNX_FP8_ARGS ctx, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, Y, ldy, st, layer_call
     switch (cfg) {
         case 4: return launch_gemm_fp8_cfg<GemmCfg<192, 2, 4, 32, true>>(LYNX_FP8_ARGS);
@@ -1757,6 +1762,11 @@ int lynx_gemm_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps,
     if (doubles) *doubles = plan.doubles;
     if (clusters) *clusters = plan.clusters;
     return (M > 256 && plan.t_us < gemm_model_time(num_sms, M, N, K, lora_steps)) ? 1 : 0;
+}
+
+int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K) {
+    if (num_sms < 2 || M < 1 || N < 8 || K < 256) return -1;
+    return pick_tile(FP8_TILES, num_sms, M, N, (double)(K / 256)).bn;
 }
 
 int lynx_gemm_register_shares_fit(int regs_per_thread) { return gemm_register_shares_fit(regs_per_thread) ? 1 : 0; }

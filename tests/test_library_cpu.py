@@ -100,6 +100,28 @@ def test_waits_of_whole_warps_end_alike_for_every_lane():
     assert found >= 5
 
 
+def test_fp8_tile_is_never_wider_than_its_rounds_call_for():
+    """A narrower tile does less per round: where it needs no more rounds over the CTA pairs it is the one to take."""
+    import random
+
+    from paper_2605_26632_b200 import binding
+
+    tile = binding.load_library().lynx_gemm_fp8_tile
+    rng = random.Random(2)
+    cases = [(1024, 4608, 3072), (700, 6144, 2048), (4096, 3072, 12288), (64, 256, 512), (16384, 21504, 3072)]
+    cases += [(rng.randint(1, 8192), 8 * rng.randint(1, 2688), 256 * rng.randint(1, 60)) for _ in range(400)]
+    seen = set()
+    for M, N, K in cases:
+        for pairs in (74, 66):
+            rounds = {w: -(-(-(-M // 256) * -(-N // w)) // pairs) for w in (128, 192, 240)}
+            w = tile(2 * pairs, M, N, K)
+            seen.add(w)
+            assert all(rounds[v] > rounds[w] for v in rounds if v < w), (M, N, K, pairs, w)
+    assert seen == {128, 192, 240}
+    assert tile(148, 4096, 3072, 12288) == 240 and tile(148, 1024, 4608, 3072) == 128
+    assert tile(148, 0, 8, 256) == -1
+
+
 def test_two_row_tile_schedule_covers_every_tile_exactly_once():
     """Host logic of the GEMM's work distribution: for any number of row tiles, column tiles,
     CTA pairs and 512-row items, every 256 x 240 tile is computed exactly once, doubles pair the
