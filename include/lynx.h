@@ -349,6 +349,9 @@ LYNX_API lynx_status lynx_selftest_wait_timeout(lynx_ctx* ctx, int64_t limit_us,
  * tiles of 256 x 240 over `clusters` pairs with `doubles` 512-row items: items[4i..4i+3] = first
  * row tile, column tile, row tiles (1 or 2), ordinal among the pair's single-tile items; returns
  * the item count (only the first `capacity` are written) or -1.
+ * lynx_gemm_phase0_plan: the tile width with which a rank-64 layer call in TENSOR or GROUP mode computes
+ * T = (X L_B^T) / s inside its GEMM launch (0: in a launch of its own), in *splits the K splits of a 256-row block and
+ * in *fill the items that each CTA pair with a tile less than the others takes (0: dealt to all pairs).
  * lynx_gemm_accumulator_waits: the parities with which the MMA issuer waits for hand-backs when its items
  * use the accumulator buffers order[0..n-1] (of `buffers`, 1 or 2): parities[i] before item i, then
  * parities[n + a] for buffer a before the kernel ends; returns n + buffers or -1.
@@ -359,6 +362,7 @@ LYNX_API int lynx_gemm_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lo
 LYNX_API int lynx_gemm_schedule_items(int tiles_m, int tiles_n, int clusters, int doubles, int cluster,
                                       int* items, int capacity);
 LYNX_API int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K);
+LYNX_API int lynx_gemm_phase0_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* splits, int* fill);
 LYNX_API int lynx_gemm_register_shares_fit(int regs_per_thread);
 LYNX_API int lynx_gemm_accumulator_waits(int buffers, const int* order, int n, int* parities);
 

@@ -200,18 +200,47 @@ struct LoraArgs {
     uint32_t* l0_ready = nullptr;
 };
 
+// What the CTA-pair tiles 256 x {256, 240, 192, 128} cost.
+// Model: rounds of tiles over the CTA pairs x (K blocks x time per K block + what a tile adds), fits to
+// measured B200 launches of each tile (us): 1024 x 3072 x 3072 14.5 with 192 against 16.1 with 240,
+// 4352 x 3072 x 3072 37.4 against 36.2, 1024 x 3072 x 9216 28.6 with 256 (two rounds) against 30.0 with
+// 192 (three).  The 256-wide tile has one accumulator buffer, so its epilogue is not hidden.
+struct TileCost {
+    int id, bn;
+    double t_kb, epi;
+};
+// (the 192-wide tile runs with five stages of 42 KB, id 8)
+constexpr TileCost BF16_TILES[4] = {{7, 240, 0.41, 0.3}, {5, 256, 0.425, 2.0}, {8, 192, 0.325, 0.7}, {6, 128, 0.27, 0.6}};
+template <int NT>
+const TileCost& pick_tile(const TileCost (&tiles)[NT], int num_sms, int64_t M, int64_t N, double kb, double* t_us = nullptr) {
+    const int pairs = num_sms / 2;
+    double best = 1e30;
+    const TileCost* pick = &tiles[0];
+    for (const TileCost& c : tiles) {
+        const int64_t n = ((M + 255) / 256) * ((N + c.bn - 1) / c.bn);
+        const double t = (double)((n + pairs - 1) / pairs) * (kb * c.t_kb + c.epi);
+        if (t < best) { best = t; pick = &c; }
+    }
+    if (t_us) *t_us = best;
+    return *pick;
+}
+
 // Plan of the in-GEMM down projection: items = 256-row blocks x K splits.  Clusters with one tile
 // fewer than the busiest ("light": index >= tiles % clusters) have a tile time of slack.  If ALL
 // items fit into that slack (at most `fill` per light cluster) they go there and the busiest
 // clusters carry none; otherwise every cluster takes its share round-robin, which finishes T
 // soonest -- a T that is late stalls the first tile of every cluster at its low-rank stage
 // (measured: a partial placement on few light clusters cost more than it saved).
-// t_tile_us: one tile's main loop; an item streams its K blocks at about 0.75 us per 128-element
-// block while most clusters stream too (HBM bound), plus ~1 us of pipeline fill.
+// bn: the launched tile's width; its time comes from the table above.  The other times are fits to whole layers with
+// splits and fill forced, 11 shapes: an item streams its K blocks at about 0.4 us per 128-element block; the
+// plans chosen are within 1.4 % of the best forced one on average, 5 % at worst (2048 x 12288 x 3072: 95.6 us).
 struct L0Plan {
     int splits, kb_per_split, light0, fill;
 };
-L0Plan l0_plan(int clusters, int tiles, int tiles_m, int kblocks, double t_tile_us, int force_splits, int force_fill) {
+L0Plan l0_plan(int clusters, int tiles, int tiles_m, int kblocks, int bn, int force_splits, int force_fill) {
+    double t_tile_us = 0.0;
+    for (const TileCost& c : BF16_TILES)
+        if (c.bn == bn) t_tile_us = kblocks * c.t_kb + c.epi;
     L0Plan best{1, kblocks, clusters, 0};
     double best_t = 1e30;
     const int rem = tiles % clusters, light = rem ? clusters - rem : 0;
@@ -221,8 +250,8 @@ L0Plan l0_plan(int clusters, int tiles, int tiles_m, int kblocks, double t_tile_
         const int real = (kblocks + per - 1) / per;
         const int items = tiles_m * real;
         // finalize: one L2 round trip per split under load, plus fences and the ticket
-        const double t_fin = real > 1 ? 1.5 + 1.3 * real : 0.5;
-        // inside the slack of the light clusters: few clusters stream, ~0.42 us per K block
+        const double t_fin = real > 1 ? 2.5 + 1.0 * real : 0.5;
+        // inside the slack of the light clusters
         const double t_item_s = per * 0.42 + 2.0;
         int fill = light ? (int)((t_tile_us - t_fin) / t_item_s) : 0;
         if (fill > 8) fill = 8;
@@ -233,8 +262,8 @@ L0Plan l0_plan(int clusters, int tiles, int tiles_m, int kblocks, double t_tile_
             if (t < best_t) { best_t = t; best = L0Plan{real, per, rem, fill}; }
         }
         if (force_fill > 0) continue;
-        // round-robin over all clusters: everybody streams, ~0.75 us per K block
-        const double t_item_r = per * 0.75 + 1.0;
+        // round-robin over all clusters
+        const double t_item_r = per * 0.4 + 1.0;
         const double late = t_fin - 0.5 * t_tile_us;
         const double t = (double)((items + clusters - 1) / clusters) * t_item_r + (late > 0 ? late : 0) + 0.02 * real;
         if (t < best_t) { best_t = t; best = L0Plan{real, per, clusters, 0}; }
@@ -411,9 +440,7 @@ lynx_status launch_gemm_cfg(lynx_ctx* ctx, const void* values, const void* meta,
         }
     }
     if (l0) {
-        // slack of a light cluster = one tile's main loop (measured ~0.465 us per K block of the 240-wide tile)
-        const L0Plan plan = l0_plan(clusters, tiles, p.tiles_m, (int)(K / 128), (double)(K / 128) * 0.465 + 0.6,
-                                    ctx->l0_force_splits, ctx->l0_force_fill);
+        const L0Plan plan = l0_plan(clusters, tiles, p.tiles_m, (int)(K / 128), Cfg::BN, ctx->l0_force_splits, ctx->l0_force_fill);
         p.l0_splits = plan.splits;
         p.l0_kb_per_split = plan.kb_per_split;
         p.l0_light0 = plan.light0;
@@ -565,30 +592,6 @@ lynx_status launch_gemm_rt2(lynx_ctx* ctx, const Rt2Plan& plan, const void* valu
 }
 
 // Tile configuration for (M, N, K): the development override, else the smallest modelled time.
-// CTA-pair tiles 256 x {256, 240, 192, 128}.
-// Model: rounds of tiles over the CTA pairs x (K blocks x time per K block + what a tile adds), fits to
-// measured B200 launches of each tile (us): 1024 x 3072 x 3072 14.5 with 192 against 16.1 with 240,
-// 4352 x 3072 x 3072 37.4 against 36.2, 1024 x 3072 x 9216 28.6 with 256 (two rounds) against 30.0 with
-// 192 (three).  The 256-wide tile has one accumulator buffer, so its epilogue is not hidden.
-struct TileCost {
-    int id, bn;
-    double t_kb, epi;
-};
-// (the 192-wide tile runs with five stages of 42 KB, id 8)
-constexpr TileCost BF16_TILES[4] = {{7, 240, 0.41, 0.3}, {5, 256, 0.425, 2.0}, {8, 192, 0.325, 0.7}, {6, 128, 0.27, 0.6}};
-template <int NT>
-const TileCost& pick_tile(const TileCost (&tiles)[NT], int num_sms, int64_t M, int64_t N, double kb, double* t_us = nullptr) {
-    const int pairs = num_sms / 2;
-    double best = 1e30;
-    const TileCost* pick = &tiles[0];
-    for (const TileCost& c : tiles) {
-        const int64_t n = ((M + 255) / 256) * ((N + c.bn - 1) / c.bn);
-        const double t = (double)((n + pairs - 1) / pairs) * (kb * c.t_kb + c.epi);
-        if (t < best) { best = t; pick = &c; }
-    }
-    if (t_us) *t_us = best;
-    return *pick;
-}
 int pick_gemm_cfg_model(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, double* t_us = nullptr) {
     return pick_tile(BF16_TILES, num_sms, M, N, (double)(K / 128) + lora_steps, t_us).id;
 }
@@ -1762,6 +1765,21 @@ int lynx_gemm_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps,
     if (doubles) *doubles = plan.doubles;
     if (clusters) *clusters = plan.clusters;
     return (M > 256 && plan.t_us < gemm_model_time(num_sms, M, N, K, lora_steps)) ? 1 : 0;
+}
+
+int lynx_gemm_phase0_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* splits, int* fill) {
+    if (num_sms < 2 || M < 1 || N < 8 || K < 128) return -1;
+    double t_us = 0.0;
+    const int cfg = pick_gemm_cfg_model(num_sms, M, N, K, 1, &t_us);
+    if (!cfg_supports_l0(cfg)) return 0;
+    int bn = 0;
+    for (const TileCost& c : BF16_TILES)
+        if (c.id == cfg) bn = c.bn;
+    const int tiles_m = (int)((M + 255) / 256), tiles = tiles_m * (int)((N + bn - 1) / bn), pairs = num_sms / 2;
+    const L0Plan plan = l0_plan(tiles < pairs ? tiles : pairs, tiles, tiles_m, (int)(K / 128), bn, 0, -1);
+    if (splits) *splits = plan.splits;
+    if (fill) *fill = plan.fill;
+    return bn;
 }
 
 int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K) {

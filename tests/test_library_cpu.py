@@ -122,6 +122,35 @@ def test_fp8_tile_is_never_wider_than_its_rounds_call_for():
     assert tile(148, 0, 8, 256) == -1
 
 
+def test_phase0_plan_fits_the_slack_it_counts_on():
+    """The down projection inside the GEMM launch: work that goes to the CTA pairs with a tile less than the others fits there
+    as a whole, and the tile's time is the launched tile's.  2048 x 12288 x 3072 runs 192-wide tiles on 74 pairs: 20 pairs
+    have a tile less, 8 row blocks in two K splits take 26 us of the 31 that a tile lasts, whole rows of K do not fit."""
+    import random
+
+    from paper_2605_26632_b200 import binding
+
+    lib = binding.load_library()
+
+    def plan(M, N, K, sms=148):
+        s, f = ctypes.c_int(-1), ctypes.c_int(-1)
+        return lib.lynx_gemm_phase0_plan(sms, M, N, K, ctypes.byref(s), ctypes.byref(f)), s.value, f.value
+
+    assert plan(2048, 3072, 12288) == (192, 2, 1)
+    rng = random.Random(3)
+    for _ in range(300):
+        M, N, K = rng.randint(1, 16384), 8 * rng.randint(1, 2688), 128 * rng.randint(1, 120)
+        width, splits, fill = plan(M, N, K)
+        if width == 0:
+            continue
+        assert width in (192, 240, 256) and 1 <= splits <= max(1, K // 256) and 0 <= fill <= 8
+        rows, tiles = -(-M // 256), -(-M // 256) * -(-N // width)
+        pairs = min(74, tiles)
+        light = pairs - tiles % pairs if tiles % pairs else 0
+        assert fill == 0 or light * fill >= rows * splits, (M, N, K)
+    assert plan(0, 8, 128)[0] == -1
+
+
 def test_two_row_tile_schedule_covers_every_tile_exactly_once():
     """Host logic of the GEMM's work distribution: for any number of row tiles, column tiles,
     CTA pairs and 512-row items, every 256 x 240 tile is computed exactly once, doubles pair the
