@@ -354,7 +354,8 @@ LYNX_API lynx_status lynx_selftest_wait_timeout(lynx_ctx* ctx, int64_t limit_us,
  * in *fill the items that each CTA pair with a tile less than the others takes (0: dealt to all pairs).
  * lynx_gemm_accumulator_waits: the parities with which the MMA issuer waits for hand-backs when its items
  * use the accumulator buffers order[0..n-1] (of `buffers`, 1 or 2): parities[i] before item i, then
- * parities[n + a] for buffer a before the kernel ends; returns n + buffers or -1.
+ * parities[n + a] for buffer a before the kernel ends; returns n + buffers or -1.  order NULL: the single-tile
+ * kernel, whose item i uses buffer i % buffers; parities[n ...] then go on in that order.
  * lynx_gemm_register_shares_fit: 1 when a GEMM kernel that was built to launch with `regs_per_thread` registers
  * can give its warps their shares, 0 when it would wait for them (the library then refuses to launch it). */
 LYNX_API int lynx_gemm_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, int* doubles,

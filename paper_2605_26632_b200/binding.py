@@ -147,9 +147,11 @@ def gemm_schedule_items(tiles_m: int, tiles_n: int, clusters: int, doubles: int,
 
 
 def gemm_accumulator_waits(buffers: int, order):
-    """-> parities of the MMA issuer's waits for hand-backs: one per item, then one per buffer (host only)."""
-    n = len(order)
-    src, out = (ctypes.c_int * max(n, 1))(*order), (ctypes.c_int * (n + buffers))()
+    """-> parities of the MMA issuer's waits for hand-backs: one per item, then one per buffer (host only).
+    order: the items' buffers, or the number of items that use the buffers in turn."""
+    n = order if isinstance(order, int) else len(order)
+    src = None if isinstance(order, int) else (ctypes.c_int * max(n, 1))(*order)
+    out = (ctypes.c_int * (n + buffers))()
     if load_library().lynx_gemm_accumulator_waits(buffers, src, n, out) < 0:
         raise ValueError("lynx_gemm_accumulator_waits: bad arguments")
     return list(out)

@@ -1790,7 +1790,11 @@ int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K) {
 int lynx_gemm_register_shares_fit(int regs_per_thread) { return gemm_register_shares_fit(regs_per_thread) ? 1 : 0; }
 
 int lynx_gemm_accumulator_waits(int buffers, const int* order, int n, int* parities) {
-    if (buffers < 1 || buffers > 2 || !order || n < 0 || !parities) return -1;
+    if (buffers < 1 || buffers > 2 || n < 0 || !parities) return -1;
+    if (!order) {
+        for (int i = 0; i < n + buffers; ++i) parities[i] = (int)(buffers == 2 ? CyclicTurn<2>(i).fill() : CyclicTurn<1>(i).fill());
+        return n + buffers;
+    }
     AccTurns turns;
     for (int i = 0; i < n; ++i) {
         if (order[i] < 0 || order[i] >= buffers) return -1;

@@ -483,7 +483,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     }
                 }
             }
-            for (int s = 0; s < STAGES && ok; ++s) {  // the last releases of the stages (see AccTurns)
+            for (int s = 0; s < STAGES && ok; ++s) {  // the last releases of the stages (see epilogue.cuh)
                 ok = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error);
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
@@ -501,7 +501,6 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
             constexpr uint32_t BH = Cfg::B_HALF_BYTES >> 4;
             uint32_t stage = 0, phase = 0;
             bool ok = true;
-            AccTurns turns;
             if constexpr (L0) {
                 // phase 0: eight dense K = 16 steps per stage into the first 64 accumulator columns
                 constexpr uint32_t idesc_l0 = make_idesc_sp_bf16(Cfg::BM * CG, Cfg::L0_R) & ~(1u << 2);
@@ -510,8 +509,9 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     const int split = item / p.tiles_m;
                     const int k0 = split * p.l0_kb_per_split;
                     const int k1 = (k0 + p.l0_kb_per_split < kblocks) ? k0 + p.l0_kb_per_split : kblocks;
-                    const int acc = (Cfg::ACC_STAGES == 2) ? (li & 1) : 0;
-                    if (!mbar_wait_warp(bar_tempty + 8 * acc, turns.fill(acc), cta_abort, p.dev_error)) {
+                    const CyclicTurn<Cfg::ACC_STAGES> turn(li);
+                    const int acc = turn.buffer;
+                    if (!mbar_wait_warp(bar_tempty + 8 * acc, turn.fill(), cta_abort, p.dev_error)) {
                         ok = false;
                         break;
                     }
@@ -550,9 +550,9 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
             }
             for (int it = 0; it < num_items && ok; ++it) {
                 const WorkItem w = sched.get(cluster_id, it);
-                const int gi = l0_n + it;  // accumulator buffers alternate over phase 0 items and tiles alike
-                const int acc = (Cfg::ACC_STAGES == 2) ? (gi & 1) : 0;
-                ok = mbar_wait_warp(bar_tempty + 8 * acc, turns.fill(acc), cta_abort, p.dev_error);
+                const CyclicTurn<Cfg::ACC_STAGES> turn(l0_n + it);  // buffers alternate over phase 0 items and tiles alike
+                const int acc = turn.buffer;
+                ok = mbar_wait_warp(bar_tempty + 8 * acc, turn.fill(), cta_abort, p.dev_error);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN;
@@ -620,8 +620,10 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     else tc_commit_pair(bar_tfull + 8 * acc, 0x3);
                 }
             }
-            for (int a = 0; a < Cfg::ACC_STAGES && ok; ++a)  // the last hand-backs (see AccTurns)
-                ok = mbar_wait_warp(bar_tempty + 8 * a, turns.fill(a), cta_abort, p.dev_error);
+            for (int a = 0; a < Cfg::ACC_STAGES && ok; ++a) {  // the last hand-backs (see epilogue.cuh)
+                const CyclicTurn<Cfg::ACC_STAGES> turn(l0_n + num_items + a);
+                ok = mbar_wait_warp(bar_tempty + 8 * turn.buffer, turn.fill(), cta_abort, p.dev_error);
+            }
         }
     }
     } else {
@@ -632,7 +634,6 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
         const uint32_t own_box = sC + (warp - GEMM_EPI_WARP0) * Cfg::BOX_BYTES;
         const uint32_t tempty0 = (CG == 2) ? mapa(bar_tempty, 0) : bar_tempty;
         bool alive = true;
-        AccTurns turns;
         if constexpr (L0) {
             // ---- phase 0: drain the 64-column accumulator of each (row block, K split) item (the first
             //      four warps; the others only hand the accumulator back) ----
@@ -641,7 +642,8 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
             for (int li = 0; li < l0_n && alive; ++li) {
                 const int item = l0s.item(cluster_id, li);
                 const int tmb = item % p.tiles_m, split = item / p.tiles_m;
-                const int acc = (Cfg::ACC_STAGES == 2) ? (li & 1) : 0;
+                const CyclicTurn<Cfg::ACC_STAGES> turn(li);
+                const int acc = turn.buffer;
                 const int row_in_block = (int)rank * Cfg::BM + q * 32 + lane;
                 const int64_t row = (int64_t)tmb * BLOCK_ROWS + row_in_block;
                 // the row's scale is fetched while the item's K loop runs (a global load costs over a
@@ -652,7 +654,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                                                                   : __ldg(p.row_scale + row);
                     inv_s = (sc == 0.0f) ? 0.0f : __frcp_rn(sc);
                 }
-                if (!mbar_wait_warp(bar_tfull + 8 * acc, turns.drain(acc), cta_abort, p.dev_error)) {
+                if (!mbar_wait_warp(bar_tfull + 8 * acc, turn.drain(), cta_abort, p.dev_error)) {
                     alive = false;
                     break;
                 }
@@ -752,8 +754,8 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
             int tm, tn;
             tile_coords(w.tile, p.tiles_m, p.tiles_n, p.group_m, tm, tn);
             const bool last = it == num_items - 1;
-            const int gi = l0_n + it;
-            const int acc = (Cfg::ACC_STAGES == 2) ? (gi & 1) : 0;
+            const CyclicTurn<Cfg::ACC_STAGES> turn(l0_n + it);
+            const int acc = turn.buffer;
             // the tile's per-column terms as fp32, for all epilogue warps (the other parity's may still be read)
             const uint32_t sb = sStrip + (it & 1) * Cfg::STRIP_BYTES, sc = sb + BN * 4;
             if (const int c = (int)threadIdx.x - 32 * GEMM_EPI_WARP0; c < BN) {
@@ -794,7 +796,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                                 epi_load_residual<CH>(p.residual, p.ldr, m0, p.M, tn * BN + (c0 + slot) * CH, p.N, lane, packed[slot]);
                     }
                 }
-                alive = mbar_wait_warp(bar_tfull + 8 * acc, turns.drain(acc), cta_abort, p.dev_error);
+                alive = mbar_wait_warp(bar_tfull + 8 * acc, turn.drain(), cta_abort, p.dev_error);
                 if (!alive) return;
                 tc_fence_after();
                 if (w.kind == 2) {

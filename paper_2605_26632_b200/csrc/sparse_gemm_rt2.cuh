@@ -322,7 +322,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     if (++stage == nst) { stage = 0; phase ^= 1; }
                 }
             }
-            // the last releases of the stages (see AccTurns; a switch of the rings has waited for the other one's)
+            // the last releases of the stages (see epilogue.cuh; a switch of the rings has waited for the other one's)
             const uint32_t nst = ring1 ? (uint32_t)Cfg::STAGES1 : (uint32_t)STAGES, bempty = ring1 ? bar_empty1 : bar_empty;
             for (uint32_t s = 0; s < nst && ok; ++s) {
                 ok = mbar_wait_warp(bempty + 8 * stage, phase ^ 1, cta_abort, p.dev_error);
@@ -423,7 +423,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     if (++stage == nst) { stage = 0; phase ^= 1; }
                 }
             }
-            for (int a = 0; a < 2 && ok; ++a)  // the last hand-backs (see AccTurns)
+            for (int a = 0; a < 2 && ok; ++a)  // the last hand-backs (see epilogue.cuh)
                 ok = mbar_wait_warp(bar_tempty + 8 * a, turns.fill(a), cta_abort, p.dev_error);
         }
     }

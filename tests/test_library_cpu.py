@@ -44,20 +44,23 @@ def test_no_accumulator_hand_back_is_outstanding_when_the_gemm_ends():
     from paper_2605_26632_b200 import binding
 
     rng = random.Random(1)
-    orders = [(b, [i % b for i in range(n)]) for b in (1, 2) for n in range(6)]  # one after the other, as single tiles are
+    orders = [(b, n) for b in (1, 2) for n in range(8)]  # single-tile kernel: the buffers in turn
     orders += [(2, [0, 1] * d + [i % 2 for i in range(s)]) for d in range(4) for s in range(4)]  # doubles, then singles
     orders += [(2, [rng.randint(0, 1) for _ in range(rng.randint(1, 9))]) for _ in range(40)]
     for buffers, order in orders:
         waits = binding.gemm_accumulator_waits(buffers, order)
-        assert len(waits) == len(order) + buffers
+        if isinstance(order, int):
+            n, uses = order, [i % buffers for i in range(order + buffers)]
+        else:
+            n, uses = len(order), order + list(range(buffers))
+        assert len(waits) == len(uses)
         filled, back = [0] * buffers, [0] * buffers
-        for i, parity in enumerate(waits):
-            a = order[i] if i < len(order) else i - len(order)
+        for i, (parity, a) in enumerate(zip(waits, uses)):
             while (back[a] & 1) == parity:  # the phase with this parity is not complete: the issuer waits
                 assert back[a] < filled[a], ("waits for ever", buffers, order, i)
                 back[a] += 1
             assert back[a] == filled[a], ("not handed back yet", buffers, order, i)
-            if i < len(order):
+            if i < n:
                 filled[a] += 1
         assert back == filled, (buffers, order)
 
