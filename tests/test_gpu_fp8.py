@@ -259,6 +259,33 @@ def test_every_fp8_tile_configuration(cfg, monkeypatch):
         ctx.close()
 
 
+@pytest.mark.parametrize("cfg", [4, 6, 7])
+@pytest.mark.parametrize("with_res", [False, True])
+def test_fp8_tiles_in_a_row(cfg, with_res, monkeypatch):
+    """Several tiles per CTA pair in every FP8 tile configuration: staging boxes (16- and 32-row ones) that are used again,
+    row and column scales of the tile at hand.  The last column tile holds 16 columns, or 160 of the 240-wide tile's."""
+    from paper_2605_26632_b200 import binding
+
+    monkeypatch.setenv("LYNX_GEMM_CFG", str(cfg))
+    M, K, N = 2570, 512, 6160
+    d = inputs.make_workload(inputs.Workload("t", M, K, N, "outlier", 810), with_bias=True, with_residual=with_res)
+    res = None if d["residual"] is None else d["residual"].cuda()
+    oq, ows = oracle.quantize_weights_fp8(u16(d["W"]), True)
+    ref = oracle.act_sparse_linear_fp8(u16(d["X"]), oq, ows, bias=u16(d["bias"]), comp_mode=1,
+                                       Yr=None if res is None else u16(res))["Y"]
+    ctx = binding.Lynx(0)
+    try:
+        Wq, ws = ctx.quantize_weights_fp8(d["W"].cuda(), True)
+        out = torch.full((M, N + 8), float("nan"), dtype=torch.bfloat16, device="cuda")  # pitch wider than N
+        Y = ctx.act_sparse_linear_fp8(d["X"].cuda(), Wq, ws, d["bias"].cuda(), 1, res, out=out[:, :N])
+        check_y(Y, ref)
+        assert bool(out[:, N:].isnan().all()), "columns past N were written"
+        torch.cuda.synchronize()
+        assert ctx.last_error() == 0
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("name", ["mlp_down", "attn_qkv", "mlp_up"])
 def test_dit_workloads_full_size_fp8(lx, name):
     """Weight codes bit-exact.  Y against the oracle on every row and column for mlp_down (the

@@ -291,8 +291,9 @@ def test_two_row_tile_gemm_kernel_with_lora(R, doubles, monkeypatch):
         ctx.close()
 
 
+@pytest.mark.parametrize("with_res", [False, True])
 @pytest.mark.parametrize("cfg", [4, 7])
-def test_stream_k_with_lora(cfg, monkeypatch):
+def test_stream_k_with_lora(cfg, with_res, monkeypatch):
     from paper_2605_26632_b200 import binding
 
     monkeypatch.setenv("LYNX_GEMM_CFG", str(cfg))
@@ -300,10 +301,11 @@ def test_stream_k_with_lora(cfg, monkeypatch):
     ctx = binding.Lynx(0)
     try:
         M, K, N = 2304, 2048, 2880  # leaves a tail of tiles, long enough in K for the stream-K split
-        X, W, b, _, LA, LB = make_case(M, K, N, 64, 600 + cfg)
+        X, W, b, res, LA, LB = make_case(M, K, N, 64, 600 + cfg, with_res=with_res)
         rows = np.arange(0, M, 37, dtype=np.int64)
-        ref = oracle.act_sparse_linear_lora(u16(X), u16(W), u16(LA), u16(LB), bias=u16(b), comp_mode=1, rows=rows)
-        Y = ctx.act_sparse_linear_lora(X.cuda(), W.cuda(), LA.cuda(), LB.cuda(), b.cuda(), 1)
+        ref = oracle.act_sparse_linear_lora(u16(X), u16(W), u16(LA), u16(LB), bias=u16(b), comp_mode=1, rows=rows,
+                                            Yr=None if res is None else u16(res))
+        Y = ctx.act_sparse_linear_lora(X.cuda(), W.cuda(), LA.cuda(), LB.cuda(), b.cuda(), 1, None if res is None else res.cuda())
         check_y(Y[torch.from_numpy(rows).cuda()], ref["Y"])
         torch.cuda.synchronize()
         assert ctx.last_error() == 0
