@@ -98,7 +98,7 @@ typedef struct {
  * caches the tensor maps (TMA descriptors) it encodes, keyed by pointer, shape, leading dimension
  * and tile, so a layer called again on the same buffers re-encodes nothing.  Reads no environment
  * variable except LYNX_DEV: with LYNX_DEV=1 (tests, measurement scripts) it also reads the
- * development overrides (LYNX_GEMM_CFG, LYNX_SPLITK, LYNX_PRUNE_TPU, ...). */
+ * development overrides (LYNX_GEMM_CFG, LYNX_RT2, LYNX_PRUNE_TPU, ...). */
 LYNX_API lynx_status lynx_create(lynx_ctx** out, int device);
 /* Frees the context's scratch.  The caller must have synchronised every stream it used. */
 LYNX_API lynx_status lynx_destroy(lynx_ctx* ctx);

@@ -56,7 +56,6 @@ struct lynx_ctx {
     int fp8_ring_forced = 0;
     int gemm_group_m = 16;    // row tiles per group of the GEMM's tile order (LYNX_GEMM_GROUP_M; 0 = one group)
     int pl_force_splits = 0;  // development override: cluster size of the prune + down-projection kernel
-    int splitk_force = 1;     // in-cluster split-K of the GEMM for launches with few tiles: 1 = cost model, 0 = off, 2..4 forced
     int rt2 = -1;             // two-row-tile GEMM kernel: -1 = cost model, 0 = never, 1 = whenever it applies
     int rt2_doubles = -1;     // development override: number of 512-row items of its schedule
     int prune_finalize = 0;   // row-scale finalize of the stand-alone prune call: 0 = per shape, 1 = in-kernel ticket, 2 = own launch
@@ -1027,7 +1026,6 @@ lynx_status lynx_create(lynx_ctx** out, int device) {
         if (geti("LYNX_FP8_RING", &ctx->fp8_ring)) ctx->fp8_ring_forced = 1;  // 0 = one CTA per 16 rows, n = ring with n warps per row
         geti("LYNX_RT2", &ctx->rt2);                      // two-row-tile GEMM kernel: 0 never, 1 whenever it applies
         geti("LYNX_RT2_D", &ctx->rt2_doubles);            // and the number of 512-row items of its schedule
-        geti("LYNX_SPLITK", &ctx->splitk_force);          // in-cluster split-K of the GEMM: 0 off, 1 model (default), 2..4 forced
         geti("LYNX_PRUNE_FINALIZE", &ctx->prune_finalize);  // row-scale finalize: 0 model, 1 in-kernel ticket, 2 own launch
     }
     if (ctx->streamk) {

@@ -421,7 +421,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                     // (the W tiles and the byte count of the first npre stages were issued before the wait)
                     const bool pre = wi == 0 && kb - w.kb0 < npre;
                     if (!elect_one()) {
-                        } else if constexpr (CG == 1) {
+                    } else if constexpr (CG == 1) {
                         const uint32_t bar = bar_full + 8 * stage;
                         if (!pre) mbar_arrive_expect_tx(bar, Cfg::STAGE_BYTES);
                         tma_load_2d(a_dst, &tmap_a, kb * Cfg::A_BOX_X, m0, bar);
