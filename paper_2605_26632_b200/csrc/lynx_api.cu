@@ -939,6 +939,7 @@ lynx_status launch_prune_lora(lynx_ctx* ctx, const void* X, int64_t M, int64_t K
             p.kb_per_split = per;
         }
     }
+    p.zero = 0;
     p.values = static_cast<uint16_t*>(values);
     p.meta = static_cast<uint8_t*>(meta);
     p.scale_partial = scale_partial;

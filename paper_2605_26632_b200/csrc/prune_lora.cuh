@@ -42,6 +42,7 @@ struct PruneLoraParams {
     uint16_t* T;           // [M x R] bf16, leading dimension ldt
     int64_t ldt;
     uint32_t* dev_error;
+    uint32_t zero;  // 0
 };
 
 template <int R_>
@@ -194,9 +195,13 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             lds128(base + 1024 + (((c0 + 1) ^ sw) << 4), b0[4], b0[5], b0[6], b0[7]);
             lds128(base + 1024 + (((c0 + 2) ^ sw) << 4), b1[0], b1[1], b1[2], b1[3]);
             lds128(base + 1024 + (((c0 + 3) ^ sw) << 4), b1[4], b1[5], b1[6], b1[7]);
-            // the tile is in registers: hand the stage back before the arithmetic and the stores
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_empty + 8 * stage);
+            // The tile is in registers: hand the stage back before the arithmetic and the stores.  In registers means that
+            // every lane's loads have returned: a load that is only issued may read the stage after the next block of K
+            // has landed in it (rank 128, whose three stages turn fastest: most launches had such a 16-byte piece).
+            // The vote waits for all eight loads, and the arrive for the vote (`zero` is 0, which the compiler cannot know).
+            const uint32_t last = a0[0] ^ a0[4] ^ a1[0] ^ a1[4] ^ b0[0] ^ b0[4] ^ b1[0] ^ b1[4];
+            const bool any = __any_sync(0xffffffffu, (last & p.zero) != 0);
+            if (lane == 0) mbar_arrive(bar_empty + 8 * stage + (any ? 8u : 0u));
             TileOut out;
             prune_tile_core<SUMS>(a0, a1, b0, b1, lut, out, numA, denA, numB, denB);
             prune_tile_store(out, va, vb, slab, okA, okB);
