@@ -25,7 +25,7 @@ EXPORTS = [
     "lynx_reserve_lora", "lynx_lora_down", "lynx_prune_compress_lora", "lynx_sparse_linear_lora", "lynx_act_sparse_linear_lora",
     "lynx_quantize_weights_fp8", "lynx_prune_compress_fp8", "lynx_sparse_linear_fp8",
     "lynx_act_sparse_linear_fp8", "lynx_gemm_plan", "lynx_gemm_schedule_items", "lynx_gemm_accumulator_waits",
-    "lynx_gemm_register_shares_fit", "lynx_gemm_fp8_tile", "lynx_gemm_phase0_plan",
+    "lynx_gemm_register_shares_fit", "lynx_gemm_split_plan", "lynx_gemm_fp8_tile", "lynx_gemm_phase0_plan",
     "lynx_selftest_wait_timeout",
 ]
 
@@ -106,6 +106,7 @@ def load_library() -> ctypes.CDLL:
     lib.lynx_gemm_schedule_items.argtypes = [i32, i32, i32, i32, i32, ctypes.POINTER(i32), i32]
     lib.lynx_gemm_accumulator_waits.argtypes = [i32, ctypes.POINTER(i32), i32, ctypes.POINTER(i32)]
     lib.lynx_gemm_register_shares_fit.argtypes = [i32]
+    lib.lynx_gemm_split_plan.argtypes = [i32, i64, i64, i64, i32, ctypes.POINTER(i32)]
     lib.lynx_gemm_fp8_tile.argtypes = [i32, i64, i64, i64]
     lib.lynx_gemm_phase0_plan.argtypes = [i32, i64, i64, i64, ctypes.POINTER(i32), ctypes.POINTER(i32)]
     lib.lynx_selftest_wait_timeout.argtypes = [vp, i64, vp]
@@ -134,6 +135,15 @@ def gemm_plan(num_sms: int, M: int, N: int, K: int, lora_steps: int = 0):
     if r < 0:
         raise ValueError("lynx_gemm_plan: bad arguments")
     return bool(r), d.value, c.value
+
+
+def gemm_split_plan(fp8: bool, M: int, N: int, K: int, lora_steps: int = 0):
+    """-> (tile, splits) of the kernel that splits K over a cluster, (0, 1) where it is not used (host only)."""
+    s = ctypes.c_int(1)
+    r = load_library().lynx_gemm_split_plan(1 if fp8 else 0, M, N, K, lora_steps, ctypes.byref(s))
+    if r < 0:
+        raise ValueError("lynx_gemm_split_plan: bad arguments")
+    return r, s.value
 
 
 def gemm_schedule_items(tiles_m: int, tiles_n: int, clusters: int, doubles: int, cluster: int):

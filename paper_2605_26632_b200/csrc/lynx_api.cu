@@ -13,6 +13,7 @@
 #include "prune_compress.cuh"
 #include "sparse_gemm.cuh"
 #include "sparse_gemm_rt2.cuh"
+#include "sparse_gemm_split.cuh"
 #include "fused_linear.cuh"
 #include "lora_down.cuh"
 #include "fp8_path.cuh"
@@ -58,6 +59,8 @@ struct lynx_ctx {
     int pl_force_splits = 0;  // development override: cluster size of the prune + down-projection kernel
     int rt2 = -1;             // two-row-tile GEMM kernel: -1 = cost model, 0 = never, 1 = whenever it applies
     int rt2_doubles = -1;     // development override: number of 512-row items of its schedule
+    int split = -1;           // K split over a cluster's members: -1 = cost model, 0 = never, 10 * tile id + splits
+    int cluster_cap[9] = {};  // CTAs, one per SM, of clusters of 1..8 that the GPU holds at once
     int prune_finalize = 0;   // row-scale finalize of the stand-alone prune call: 0 = per shape, 1 = in-kernel ticket, 2 = own launch
     // encoded tensor maps of recent launches, keyed by everything that went into the encoding
     // (a layer called again on the same buffers skips cuTensorMapEncodeTiled)
@@ -608,13 +611,169 @@ int pick_gemm_cfg(const lynx_ctx* ctx, int64_t M, int64_t N, int64_t K, int lora
     if (ctx->gemm_cfg != 0) return ctx->gemm_cfg;
     return pick_gemm_cfg_model(ctx->num_sms, M, N, K, lora_steps);
 }
+// ------------------------------------------------------- K split over a cluster (sparse_gemm_split) -----
+
+template <class Cfg, bool LORA>
+lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, const void* values, const void* meta, int64_t M, int64_t K, const void* W,
+                              int64_t N, int64_t ldw, const float* wscale, const void* bias, const lynx_comp* comp,
+                              const LoraArgs* lora, void* Y, int64_t ldy, cudaStream_t st, const ScaleSrc* ss, bool layer_call) {
+    constexpr CUtensorMapDataType op_type = Cfg::FP8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    constexpr int op_bytes = Cfg::FP8 ? 1 : 2;
+    CUtensorMap ta, tb, te, ty, tt, tla;
+    const uint64_t rb = (uint64_t)((M + 127) / 128), kb128 = (uint64_t)(K / 128);
+    if (!make_tmap_2d(ctx, &ta, op_type, op_bytes, values, (uint64_t)M, (uint64_t)(K / 2), (uint64_t)(K / 2) * op_bytes, Cfg::BOX_X,
+                      Cfg::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_tmap_2d(ctx, &tb, op_type, op_bytes, W, (uint64_t)N, (uint64_t)K, (uint64_t)ldw * op_bytes, Cfg::BOX_X, Cfg::BN_CTA,
+                      CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_tmap_2d(ctx, &te, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, meta, rb * kb128 * 2, 256, 1024, 256, Cfg::E_BYTES / 1024,
+                      CU_TENSOR_MAP_SWIZZLE_NONE) ||
+        !make_tmap_2d(ctx, &ty, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, (uint64_t)M, (uint64_t)N, (uint64_t)ldy * 2, Cfg::CH, 32,
+                      Cfg::CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE))
+        return LYNX_ERR_CUDA;
+    if (LORA) {
+        if (!make_tmap_2d(ctx, &tt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->T, (uint64_t)M, (uint64_t)lora->R,
+                          (uint64_t)lora->ldt * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
+            !make_tmap_2d(ctx, &tla, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->LA, (uint64_t)N, (uint64_t)lora->R,
+                          (uint64_t)lora->ldla * 2, 64, Cfg::BN_CTA, CU_TENSOR_MAP_SWIZZLE_128B))
+            return LYNX_ERR_CUDA;
+    } else {
+        tt = ta;  // never read: lora_steps = 0
+        tla = tb;
+    }
+    SplitGemmParams p;
+    p.M = M; p.N = N; p.K = K;
+    p.row_scale = comp ? comp->row_scale : nullptr;
+    p.scale_partial = ss ? ss->partial : nullptr;
+    p.scale_ks = ss ? ss->ks : 0;
+    p.col_scale = wscale;
+    p.bias = static_cast<const uint16_t*>(bias);
+    p.residual = comp ? static_cast<const uint16_t*>(comp->residual) : nullptr;
+    p.ldr = comp ? comp->ldr : 0;
+    p.dev_error = ctx->err_dev;
+    constexpr int rows = Cfg::R * Cfg::CG * Cfg::BM;
+    p.tiles_m = (int)((M + rows - 1) / rows);
+    p.splits = splits;
+    p.lora_steps = LORA ? lora->R / 64 : 0;
+    p.w_prefetch = layer_call ? 1 : 0;
+    const int tiles_n = (int)((N + Cfg::BN - 1) / Cfg::BN);
+    auto kern = sparse_gemm_split_kernel<Cfg, LORA>;
+    static bool attr_set[MAX_CTX_DEVICES] = {};  // per instantiation
+    if (lynx_status as = prepare_gemm_kernel(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
+    cudaLaunchConfig_t cfg = {};
+    const int grid = p.tiles_m * tiles_n * splits * Cfg::CG;
+    // With a quarter of the SMs free the next kernel's CTAs (a prune launch's are small) start there and run their
+    // prologue: 256 x 3072 x 3072 layer 10.1 -> 9.8 us.  With fewer they pile up on the few that are: 128 x 3072 x 9216
+    // (144 SMs) 16.2 -> 17.6.
+    p.trigger = grid * 4 <= ctx->num_sms * 3 ? 1 : 0;
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(Cfg::THREADS);
+    cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)(Cfg::CG * splits);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = ctx->pdl ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, te, ty, tt, tla, p) != cudaSuccess) return LYNX_ERR_CUDA;
+    ctx->launches++;
+    return LYNX_OK;
+}
+
+// Plan of the split: tile and number of splits, modelled with the same kind of figures as the tiles above
+// (K blocks per split x time per K block + what the exchange adds), so that the two can be compared.  Only
+// plans of one round over the GPU are considered: there is nothing to split where the tiles fill it.  Fits to layers of
+// 28 shapes with every tile and number of splits forced; whole layers with the plans chosen here against the other
+// kernels: 256 x 12288 x 3072 33.1 -> 23.9 us, 65 x 15360 x 3072 38.1 -> 23.5, 338 x 15360 x 3072 42.6 -> 38, 381 x 13824 x 632
+// 31.8 -> 16.5, 182 x 3072 x 3072 10.2 -> 9.7.  Below about 14 K blocks the exchange costs more than the shorter main loop
+// gives (397 x 1792 x 1992 with a low-rank branch 14.0 -> 15.2), which is where the constants `fix` draw the line;
+// higher for FP8, whose prune launch holds an SM per row up to 148 (71 x 3840 x 3840 10.3 -> 11.3 in four splits).
+struct SplitTile {
+    int id, rows, bn, cg;
+    double t_kb, fix;
+};
+constexpr SplitTile SPLIT_BF16[] = {{1, 256, 128, 2, 0.20, 3.4}, {2, 256, 192, 2, 0.31, 4.6}, {5, 128, 128, 1, 0.29, 3.0}};
+constexpr SplitTile SPLIT_FP8[] = {{1, 256, 128, 2, 0.25, 3.6}, {2, 256, 192, 2, 0.39, 4.5}, {5, 128, 128, 1, 0.30, 3.7}};
+// CTAs, one per SM, of clusters of 1..8 that a GPU of 148 SMs holds at once, as cudaOccupancyMaxActiveClusters says
+constexpr int CLUSTER_CAP_148[9] = {0, 148, 148, 135, 132, 130, 132, 105, 120};
+// Products of at least this many rows are never split: lynx_act_sparse_linear_host works on them in chunks of rows, and a
+// chunk's result is bit for bit the whole product's.
+constexpr int64_t SPLIT_MAX_ROWS = 2048;
+struct SplitPlan {
+    int id = 0, splits = 1;
+    double t_us = 1e30;
+};
+template <bool FP8>
+SplitPlan split_plan(const int (&cap)[9], int64_t M, int64_t N, int64_t K, int lora_steps) {
+    SplitPlan best;
+    if (M >= SPLIT_MAX_ROWS) return best;
+    const int64_t kb = K / (FP8 ? 256 : 128);
+    for (const SplitTile& c : FP8 ? SPLIT_FP8 : SPLIT_BF16) {
+        const int64_t tiles = ((M + c.rows - 1) / c.rows) * ((N + c.bn - 1) / c.bn);
+        for (int s = 2; s * c.cg <= 8 && s <= kb; ++s) {
+            if (tiles * s * c.cg > cap[s * c.cg]) continue;
+            const double t = (double)((kb + s - 1) / s + lora_steps) * c.t_kb + c.fix + 0.3 * c.cg * (s - 2);
+            if (t < best.t_us) best = SplitPlan{c.id, s, t};
+        }
+    }
+    return best;
+}
+
+template <bool FP8>
+lynx_status launch_gemm_split_id(lynx_ctx* ctx, const SplitPlan& plan, const void* values, const void* meta, int64_t M, int64_t K,
+                                 const void* W, int64_t N, int64_t ldw, const float* wscale, const void* bias, const lynx_comp* comp,
+                                 const LoraArgs* lora, void* Y, int64_t ldy, cudaStream_t st, const ScaleSrc* ss, bool layer_call) {
+    auto go = [&](auto cfg) {
+        using Cfg = decltype(cfg);
+        const int splits = plan.splits;
+        if (!Cfg::splits_fit(splits) || splits > K / Cfg::BK) return LYNX_ERR_INVALID_ARG;
+#define LYNX_SPLIT_ARGS ctx, splits, values, meta, M, K, W, N, ldw, wscale, bias, comp, lora, Y, ldy, st, ss, layer_call
+        if constexpr (!FP8) {
+            if (lora) return launch_gemm_split<Cfg, true>(LYNX_SPLIT_ARGS);
+        }
+        return launch_gemm_split<Cfg, false>(LYNX_SPLIT_ARGS);
+#undef LYNX_SPLIT_ARGS
+    };
+    switch (plan.id) {
+        case 1: return go(SplitCfg<1, 128, 2, 5, FP8>{});
+        case 2: return go(SplitCfg<1, 192, 2, FP8 ? 4 : 5, FP8>{});
+        case 5: return go(SplitCfg<1, 128, 1, 4, FP8>{});
+        default: return LYNX_ERR_INVALID_ARG;
+    }
+}
+
+// The split plan of a product if it is modelled faster than the other kernels, id 0 if not.
+template <bool FP8>
+SplitPlan split_plan_if_faster(const int (&cap)[9], int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps) {
+    const SplitPlan plan = split_plan<FP8>(cap, M, N, K, lora_steps);
+    double t = 0.0;
+    if (FP8) pick_tile(FP8_TILES, num_sms, M, N, (double)(K / 256), &t);
+    else t = gemm_model_time(num_sms, M, N, K, lora_steps);
+    return plan.t_us < t ? plan : SplitPlan{};
+}
+template <bool FP8>
+SplitPlan choose_split(const lynx_ctx* ctx, int64_t M, int64_t N, int64_t K, int lora_steps) {
+    if (ctx->split == 0) return SplitPlan{};
+    if (ctx->split > 0) return SplitPlan{ctx->split / 10, ctx->split % 10, 0.0};
+    return split_plan_if_faster<FP8>(ctx->cluster_cap, ctx->num_sms, M, N, K, lora_steps);
+}
+
 // every tile but the 2-CTA 256 x 128 one has room in its W slot for a phase-0 stage
 bool cfg_supports_l0(int cfg) { return cfg >= 1 && cfg <= 8 && cfg != 6; }
 
 lynx_status launch_gemm(lynx_ctx* ctx, const void* values, const void* meta, int64_t M, int64_t K, const void* W,
                         int64_t N, int64_t ldw, const void* bias, const lynx_comp* comp, const LoraArgs* lora, void* Y,
-                        int64_t ldy, cudaStream_t st, int cfg = 0, const ScaleSrc* ss = nullptr, bool layer_call = false) {
+                        int64_t ldy, cudaStream_t st, int cfg = 0, const ScaleSrc* ss = nullptr, bool layer_call = false,
+                        bool split_ok = true) {
     const int lora_steps = lora ? lora->R / 64 : 0;
+    if (split_ok && cfg == 0 && ctx->gemm_cfg == 0 && ctx->rt2 != 1 && !ctx->streamk && !(lora && lora->X)) {
+        const SplitPlan plan = choose_split<false>(ctx, M, N, K, lora_steps);
+        if (plan.id)
+            return launch_gemm_split_id<false>(ctx, plan, values, meta, M, K, W, N, ldw, nullptr, bias, comp, lora, Y, ldy, st, ss, layer_call);
+    }
     if (cfg == 0 && ctx->gemm_cfg == 0 && ctx->rt2 != 0 && !ctx->streamk && !(lora && lora->X) && M > 256) {
         // the two-row-tile kernel where its schedule is modelled faster than the best plain tile
         const Rt2Plan plan = rt2_plan(ctx->num_sms, M, N, K, lora_steps, ctx->rt2_doubles);
@@ -697,6 +856,12 @@ lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void*
 lynx_status launch_gemm_fp8(lynx_ctx* ctx, const void* values_q, const void* meta, int64_t M, int64_t K,
                             const void* Wq, int64_t N, int64_t ldwq, const float* wscale, const void* bias,
                             const lynx_comp* comp, void* Y, int64_t ldy, cudaStream_t st, bool layer_call = false) {
+    if (ctx->gemm_cfg == 0) {
+        const SplitPlan plan = choose_split<true>(ctx, M, N, K, 0);
+        if (plan.id)
+            return launch_gemm_split_id<true>(ctx, plan, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, nullptr, Y, ldy, st, nullptr,
+                                              layer_call);
+    }
     int cfg = ctx->gemm_cfg;
     if (cfg != 4 && cfg != 6 && cfg != 7) cfg = pick_tile(FP8_TILES, ctx->num_sms, M, N, (double)(K / 256)).id;
 #define LYNX_FP8_ARGS ctx, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, Y, ldy, st, layer_call
@@ -1005,6 +1170,28 @@ lynx_status lynx_create(lynx_ctx** out, int device) {
         delete ctx;
         return LYNX_ERR_WORKSPACE;
     }
+    {
+        // how many CTAs, one per SM, of clusters of 1..8 the GPU holds at once
+        auto kern = sparse_gemm_split_kernel<SplitCfg<1, 128, 2, 5>, false>;
+        constexpr int smem = SplitCfg<1, 128, 2, 5>::SMEM_BYTES;
+        const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+        for (int i = 1; i <= 8 && ok; ++i) {
+            cudaLaunchConfig_t qc = {};
+            qc.gridDim = dim3((unsigned)(ctx->num_sms / i * i));
+            qc.blockDim = dim3(GEMM_THREADS);
+            qc.dynamicSmemBytes = smem;
+            cudaLaunchAttribute qa[1];
+            qa[0].id = cudaLaunchAttributeClusterDimension;
+            qa[0].val.clusterDim.x = (unsigned)i;
+            qa[0].val.clusterDim.y = 1;
+            qa[0].val.clusterDim.z = 1;
+            qc.attrs = qa;
+            qc.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kern, &qc) == cudaSuccess) ctx->cluster_cap[i] = n * i;
+        }
+        (void)cudaGetLastError();  // (a size that does not fit leaves its count at zero: no such plan)
+    }
     // Development overrides (tile configuration, schedules, kernel forms) are read only when
     // LYNX_DEV=1 is set: tests and measurement scripts set it, a production process reads nothing else.
     const char* dev = getenv("LYNX_DEV");
@@ -1027,6 +1214,7 @@ lynx_status lynx_create(lynx_ctx** out, int device) {
         if (geti("LYNX_FP8_RING", &ctx->fp8_ring)) ctx->fp8_ring_forced = 1;  // 0 = one CTA per 16 rows, n = ring with n warps per row
         geti("LYNX_RT2", &ctx->rt2);                      // two-row-tile GEMM kernel: 0 never, 1 whenever it applies
         geti("LYNX_RT2_D", &ctx->rt2_doubles);            // and the number of 512-row items of its schedule
+        geti("LYNX_SPLIT", &ctx->split);                  // K split over a cluster: 0 never, 10 * tile id + splits
         geti("LYNX_PRUNE_FINALIZE", &ctx->prune_finalize);  // row-scale finalize: 0 model, 1 in-kernel ticket, 2 own launch
     }
     if (ctx->streamk) {
@@ -1241,10 +1429,11 @@ lynx_status lynx_sparse_linear(lynx_ctx* ctx, const void* values, const void* me
                        static_cast<cudaStream_t>(stream));
 }
 
-lynx_status lynx_act_sparse_linear(lynx_ctx* ctx, const void* X, int64_t M, int64_t K, int64_t ldx, const void* W,
-                                   int64_t N, int64_t ldw, const void* bias, lynx_comp_mode mode,
-                                   const void* residual, int64_t ldr, void* Y, int64_t ldy, lynx_fuse_mode fuse,
-                                   void* stream) {
+// split_ok: the GEMM may split K over a cluster (an element's order of additions then depends on M).
+static lynx_status act_sparse_linear_impl(lynx_ctx* ctx, const void* X, int64_t M, int64_t K, int64_t ldx, const void* W,
+                                          int64_t N, int64_t ldw, const void* bias, lynx_comp_mode mode,
+                                          const void* residual, int64_t ldr, void* Y, int64_t ldy, lynx_fuse_mode fuse,
+                                          void* stream, bool split_ok) {
     lynx_status s = check_common(ctx, M, K);
     if (s != LYNX_OK) return s;
     if (fuse != LYNX_FUSE_AUTO && fuse != LYNX_FUSE_SEPARATE && fuse != LYNX_FUSE_FUSED) return LYNX_ERR_INVALID_ARG;
@@ -1292,9 +1481,16 @@ lynx_status lynx_act_sparse_linear(lynx_ctx* ctx, const void* X, int64_t M, int6
     comp.ldr = ldr;
     if ((s = check_device_error(ctx)) == LYNX_OK)
         s = launch_gemm(ctx, values, meta, M, K, W, N, ldw, bias, &comp, nullptr, Y, ldy,
-                        static_cast<cudaStream_t>(stream), 0, &ss, true);
+                        static_cast<cudaStream_t>(stream), 0, &ss, true, split_ok);
     clear_deferred(ctx);  // the sums in the scratch belonged to this call
     return s;
+}
+
+lynx_status lynx_act_sparse_linear(lynx_ctx* ctx, const void* X, int64_t M, int64_t K, int64_t ldx, const void* W,
+                                   int64_t N, int64_t ldw, const void* bias, lynx_comp_mode mode,
+                                   const void* residual, int64_t ldr, void* Y, int64_t ldy, lynx_fuse_mode fuse,
+                                   void* stream) {
+    return act_sparse_linear_impl(ctx, X, M, K, ldx, W, N, ldw, bias, mode, residual, ldr, Y, ldy, fuse, stream, true);
 }
 
 lynx_status lynx_act_sparse_linear_host(lynx_ctx* ctx, const void* X_host, int64_t M, int64_t K, const void* W,
@@ -1314,8 +1510,9 @@ lynx_status lynx_act_sparse_linear_host(lynx_ctx* ctx, const void* X_host, int64
     char* yd = xd + x_bytes;
     // Token rows are independent (except under the whole-tensor scale), so the call is pipelined over
     // row chunks: the copy-in of chunk c + 1 and the copy-out of chunk c - 1 overlap the kernels of
-    // chunk c on two copy streams (PCIe is full duplex); the result is the unchunked one bit for bit.
-    int chunks = (M >= 2048 && mode != LYNX_COMP_TENSOR) ? 4 : 1;
+    // chunk c on two copy streams (PCIe is full duplex); the result is the unchunked one bit for bit
+    // (products of as many rows are not split over K, so the chunks must not be either).
+    int chunks = (M >= SPLIT_MAX_ROWS && mode != LYNX_COMP_TENSOR) ? 4 : 1;
     const int64_t rows_per = ((M + chunks - 1) / chunks + 255) / 256 * 256;
     chunks = (int)((M + rows_per - 1) / rows_per);
     if (chunks == 1) {
@@ -1353,8 +1550,8 @@ lynx_status lynx_act_sparse_linear_host(lynx_ctx* ctx, const void* X_host, int64
     for (int c = 0; c < chunks; ++c) {
         const int64_t r0 = c * rows_per, rows = (r0 + rows_per <= M) ? rows_per : M - r0;
         if (cudaStreamWaitEvent(st, ctx->ev_h2d[c], 0) != cudaSuccess) return LYNX_ERR_CUDA;
-        s = lynx_act_sparse_linear(ctx, xd + (size_t)r0 * K * 2, rows, K, K, W, N, ldw, bias, mode, nullptr, 0,
-                                   yd + (size_t)r0 * N * 2, N, fuse, stream);
+        s = act_sparse_linear_impl(ctx, xd + (size_t)r0 * K * 2, rows, K, K, W, N, ldw, bias, mode, nullptr, 0,
+                                   yd + (size_t)r0 * N * 2, N, fuse, stream, false);
         if (s != LYNX_OK) return s;
         if (cudaEventRecord(ctx->ev_done[c], st) != cudaSuccess ||
             cudaStreamWaitEvent(ctx->d2h_stream, ctx->ev_done[c], 0) != cudaSuccess ||
@@ -1779,6 +1976,14 @@ int lynx_gemm_phase0_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* spl
     if (splits) *splits = plan.splits;
     if (fill) *fill = plan.fill;
     return bn;
+}
+
+int lynx_gemm_split_plan(int fp8, int64_t M, int64_t N, int64_t K, int lora_steps, int* splits) {
+    if (M < 1 || N < 8 || K < (fp8 ? 256 : 128) || (fp8 && lora_steps)) return -1;
+    const SplitPlan plan = fp8 ? split_plan_if_faster<true>(CLUSTER_CAP_148, 148, M, N, K, 0)
+                               : split_plan_if_faster<false>(CLUSTER_CAP_148, 148, M, N, K, lora_steps);
+    if (splits) *splits = plan.splits;
+    return plan.id;
 }
 
 int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K) {

@@ -262,6 +262,12 @@ __device__ __forceinline__ uint32_t mapa(uint32_t smem_addr, uint32_t rank) {
     return r;
 }
 
+// 16-byte store to the shared memory of any CTA of the cluster (address from mapa)
+__device__ __forceinline__ void sts128_cluster(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d)
+                 : "memory");
+}
+
 // 16-byte load from the shared memory of any CTA of the cluster (address from mapa)
 __device__ __forceinline__ float4 lds128_cluster_f32(uint32_t cluster_addr) {
     float4 v;

@@ -278,3 +278,25 @@ def test_bench_launches_its_own_ranks_when_started_plainly():
     d = json.loads(line)
     assert d["launch_check"] and d["n_gpus"] == 2 and d["slowest_rank_ms"] == 15.0
     assert abs(d["aggregate_tflops"] - 1e12 * 10 * 2 / 15e-3 / 1e12) < 1e-6
+
+
+def test_split_plan_is_one_round_and_has_a_k_block_for_every_member():
+    import random
+
+    from paper_2605_26632_b200 import binding
+
+    rows, width, ctas = {1: 256, 2: 256, 5: 128}, {1: 128, 2: 192, 5: 128}, {1: 2, 2: 2, 5: 1}
+    held = {2: 148, 3: 135, 4: 132, 5: 130, 6: 132, 7: 105, 8: 120}
+    rng, seen = random.Random(4), set()
+    cases = [(2047, 256, 16384, 0, 0), (2048, 256, 16384, 0, 0), (1, 8, 128, 0, 0), (256, 3072, 12288, 0, 1)]
+    cases += [(rng.randint(1, 2300), 8 * rng.randint(1, 1300), 256 * rng.randint(1, 64), rng.random() < 0.3, 0) for _ in range(2000)]
+    for M, N, K, fp8, lora in cases:
+        tile, s = binding.gemm_split_plan(fp8, M, N, K, lora)
+        if tile == 0:
+            continue
+        seen.add((tile, bool(fp8)))
+        members = ctas[tile] * s
+        assert 2 <= members <= 8 and s >= 2 and s <= K // (256 if fp8 else 128) and M < 2048
+        assert -(-M // rows[tile]) * -(-N // width[tile]) * members <= held[members], (M, N, K)
+    assert seen == {(t, f) for t in (1, 2, 5) for f in (False, True)}
+    assert binding.gemm_split_plan(False, 256, 3072, 12288) == (1, 2) and binding.gemm_split_plan(False, 4096, 3072, 12288)[0] == 0
