@@ -347,7 +347,7 @@ LYNX_API lynx_status lynx_selftest_wait_timeout(lynx_ctx* ctx, int64_t limit_us,
  * lynx_gemm_split_plan goes before both: for a product of few tiles on a GPU of 148 SMs it returns the tile of the
  * kernel that splits K over the members of a cluster (1: 256 x 128 per CTA pair, 2: 256 x 192, 5: 128 x 128 per CTA;
  * the number of members in *splits), 0 when K is not split, -1 on bad arguments.
- * lynx_gemm_fp8_tile returns the width of the tiles (256 x 128, 192 or 240) of an FP8 product, or -1.
+ * lynx_gemm_fp8_tile returns the width of the tiles (256 x 128, 192 or 240) of an FP8 product in the single-tile kernel, or -1.
  * lynx_gemm_schedule_items lists the work items of CTA pair `cluster` for `tiles_m` x `tiles_n`
  * tiles of 256 x 240 over `clusters` pairs with `doubles` 512-row items: items[4i..4i+3] = first
  * row tile, column tile, row tiles (1 or 2), ordinal among the pair's single-tile items; returns

@@ -481,6 +481,7 @@ lynx_status launch_gemm_cfg(lynx_ctx* ctx, const void* values, const void* meta,
 // ------------------------------------------------------- two-row-tile GEMM kernel (sparse_gemm_rt2) -----
 
 using Rt2Cfg = Gemm2Cfg<240, 3>;
+using Rt2CfgFp8 = Gemm2Cfg<240, 3, true>;
 
 // Modelled time (us) of the slowest cluster for a schedule with D doubles.  The figures are fits to
 // measured B200 launches (back to back, clocks as they settle): 0.41 us per K block of a 256 x 240 single
@@ -489,14 +490,21 @@ using Rt2Cfg = Gemm2Cfg<240, 3>;
 // stores of 122 KB per CTA slow the next item's first loads).  4352 x 3072 x 3072: one double + one single per
 // cluster 34.9 us, three singles 36.2; 4096 x 3072 x 12288: doubles 121.7, singles 127.1.  Within each class of
 // clusters the one at the first position carries the most singles, so two clusters decide the maximum.
-constexpr double RT2_T1 = 0.41, RT2_T2 = 0.63, RT2_E1 = 0.3, RT2_E2 = 4.5;
-double rt2_makespan(const PairSchedule& sc, double kb) {
+// FP8 (256-element K blocks): fits to whole layers of 19 shapes at the clocks that calls back to back settle at, single-tile
+// kernel -> two row tiles: 16384 x 12288 x 3072 410 -> 390 us, 4352 x 3072 x 9216 81.5 -> 78.5, 1337 x 3840 x 10240 42.0 -> 40.2,
+// 4096 x 12288 x 3072 104.1 -> 103.7; up to K = 2048 the exposed epilogues cost more than the bytes saved give
+// (8192 x 2048 x 8192 98.5 against 102.4).
+struct Rt2Cost {
+    double t1, t2, e1, e2;
+};
+constexpr Rt2Cost RT2_BF16 = {0.41, 0.63, 0.3, 4.5}, RT2_FP8 = {0.41, 0.617, 1.6, 4.0};
+double rt2_makespan(const PairSchedule& sc, const Rt2Cost& c2, double kb) {
     double worst = 0.0;
     const int probe[2] = {sc.b % sc.C, 0};  // position 0 (first light cluster), position L (first heavy one)
     for (int i = 0; i < 2; ++i) {
         const int c = probe[i];
         const int nd = sc.num_doubles(c), ns = sc.num_singles(c);
-        const double t = nd * (kb * RT2_T2 + RT2_E2) + ns * (kb * RT2_T1 + RT2_E1);
+        const double t = nd * (kb * c2.t2 + c2.e2) + ns * (kb * c2.t1 + c2.e1);
         if (t > worst) worst = t;
     }
     return worst;
@@ -506,10 +514,10 @@ struct Rt2Plan {
     int doubles, clusters;
     double t_us;
 };
-Rt2Plan rt2_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, int force_doubles) {
+// kb: K blocks of an item, low-rank stages included
+Rt2Plan rt2_plan(const Rt2Cost& cost, int num_sms, int64_t M, int64_t N, double kb, int force_doubles) {
     const int tiles_m = (int)((M + 255) / 256), tiles_n = (int)((N + Rt2Cfg::BN - 1) / Rt2Cfg::BN);
     const int pairs = num_sms / 2;
-    const double kb = (double)(K / 128) + lora_steps;
     const int dmax = (tiles_m / 2) * tiles_n;
     Rt2Plan best{0, 1, 1e30};
     auto consider = [&](int D) {
@@ -518,7 +526,7 @@ Rt2Plan rt2_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, i
         const int C = items < pairs ? items : pairs;
         PairSchedule sc;
         sc.init(tiles_m, tiles_n, C, D, 8);
-        const double t = rt2_makespan(sc, kb);
+        const double t = rt2_makespan(sc, cost, kb);
         if (t < best.t_us) best = Rt2Plan{D, C, t};
     };
     if (force_doubles >= 0) {
@@ -532,22 +540,23 @@ Rt2Plan rt2_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, i
     return best;
 }
 
-template <bool LORA>
+template <class Cfg, bool LORA>
 lynx_status launch_gemm_rt2(lynx_ctx* ctx, const Rt2Plan& plan, const void* values, const void* meta, int64_t M,
-                            int64_t K, const void* W, int64_t N, int64_t ldw, const void* bias, const lynx_comp* comp,
-                            const LoraArgs* lora, void* Y, int64_t ldy, cudaStream_t st, const ScaleSrc* ss,
-                            bool layer_call) {
-    using Cfg = Rt2Cfg;
+                            int64_t K, const void* W, int64_t N, int64_t ldw, const float* wscale, const void* bias,
+                            const lynx_comp* comp, const LoraArgs* lora, void* Y, int64_t ldy, cudaStream_t st,
+                            const ScaleSrc* ss, bool layer_call) {
+    constexpr CUtensorMapDataType op_type = Cfg::FP8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    constexpr int op_bytes = Cfg::FP8 ? 1 : 2;
     CUtensorMap ta, tb, te, ty, tt, tla;
-    const uint64_t rb = (uint64_t)((M + 127) / 128), kblocks = (uint64_t)(K / 128);
-    if (!make_tmap_2d(ctx, &ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, values, (uint64_t)M, (uint64_t)(K / 2),
-                      (uint64_t)K, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_tmap_2d(ctx, &tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W, (uint64_t)N, (uint64_t)K, (uint64_t)ldw * 2, 64,
-                      Cfg::BN_CTA, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_tmap_2d(ctx, &te, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, meta, rb * kblocks * 2, 256, 1024, 256, 2,
+    const uint64_t rb = (uint64_t)((M + 127) / 128), kb128 = (uint64_t)(K / 128);
+    if (!make_tmap_2d(ctx, &ta, op_type, op_bytes, values, (uint64_t)M, (uint64_t)(K / 2), (uint64_t)(K / 2) * op_bytes, Cfg::BOX_X,
+                      Cfg::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_tmap_2d(ctx, &tb, op_type, op_bytes, W, (uint64_t)N, (uint64_t)K, (uint64_t)ldw * op_bytes, Cfg::BOX_X, Cfg::BN_CTA,
+                      CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_tmap_2d(ctx, &te, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, meta, rb * kb128 * 2, 256, 1024, 256, Cfg::E_BYTES / 1024,
                       CU_TENSOR_MAP_SWIZZLE_NONE) ||
         !make_tmap_2d(ctx, &ty, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, (uint64_t)M, (uint64_t)N, (uint64_t)ldy * 2, Cfg::CH,
-                      32, CU_TENSOR_MAP_SWIZZLE_NONE))
+                      Cfg::BOX_ROWS, CU_TENSOR_MAP_SWIZZLE_NONE))
         return LYNX_ERR_CUDA;
     if (LORA) {
         if (!make_tmap_2d(ctx, &tt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->T, (uint64_t)M, (uint64_t)lora->R,
@@ -564,6 +573,7 @@ lynx_status launch_gemm_rt2(lynx_ctx* ctx, const Rt2Plan& plan, const void* valu
     p.row_scale = comp ? comp->row_scale : nullptr;
     p.scale_partial = ss ? ss->partial : nullptr;
     p.scale_ks = ss ? ss->ks : 0;
+    p.col_scale = wscale;
     p.bias = static_cast<const uint16_t*>(bias);
     p.residual = comp ? static_cast<const uint16_t*>(comp->residual) : nullptr;
     p.ldr = comp ? comp->ldr : 0;
@@ -776,10 +786,12 @@ lynx_status launch_gemm(lynx_ctx* ctx, const void* values, const void* meta, int
     }
     if (cfg == 0 && ctx->gemm_cfg == 0 && ctx->rt2 != 0 && !ctx->streamk && !(lora && lora->X) && M > 256) {
         // the two-row-tile kernel where its schedule is modelled faster than the best plain tile
-        const Rt2Plan plan = rt2_plan(ctx->num_sms, M, N, K, lora_steps, ctx->rt2_doubles);
+        const Rt2Plan plan = rt2_plan(RT2_BF16, ctx->num_sms, M, N, (double)(K / 128) + lora_steps, ctx->rt2_doubles);
         if (ctx->rt2 == 1 || plan.t_us < gemm_model_time(ctx->num_sms, M, N, K, lora_steps))
-            return lora ? launch_gemm_rt2<true>(ctx, plan, values, meta, M, K, W, N, ldw, bias, comp, lora, Y, ldy, st, ss, layer_call)
-                        : launch_gemm_rt2<false>(ctx, plan, values, meta, M, K, W, N, ldw, bias, comp, lora, Y, ldy, st, ss, layer_call);
+            return lora ? launch_gemm_rt2<Rt2Cfg, true>(ctx, plan, values, meta, M, K, W, N, ldw, nullptr, bias, comp, lora, Y, ldy, st, ss,
+                                                        layer_call)
+                        : launch_gemm_rt2<Rt2Cfg, false>(ctx, plan, values, meta, M, K, W, N, ldw, nullptr, bias, comp, lora, Y, ldy, st,
+                                                         ss, layer_call);
     }
     if (cfg == 0) cfg = pick_gemm_cfg(ctx, M, N, K, lora_steps);
 #define LYNX_GEMM_ARGS ctx, values, meta, M, K, W, N, ldw, bias, comp, lora, Y, ldy, st, ss, layer_call
@@ -856,11 +868,20 @@ lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void*
 lynx_status launch_gemm_fp8(lynx_ctx* ctx, const void* values_q, const void* meta, int64_t M, int64_t K,
                             const void* Wq, int64_t N, int64_t ldwq, const float* wscale, const void* bias,
                             const lynx_comp* comp, void* Y, int64_t ldy, cudaStream_t st, bool layer_call = false) {
-    if (ctx->gemm_cfg == 0) {
+    if (ctx->gemm_cfg == 0 && ctx->rt2 != 1) {
         const SplitPlan plan = choose_split<true>(ctx, M, N, K, 0);
         if (plan.id)
             return launch_gemm_split_id<true>(ctx, plan, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, nullptr, Y, ldy, st, nullptr,
                                               layer_call);
+    }
+    if (ctx->gemm_cfg == 0 && ctx->rt2 != 0 && M > 256) {
+        // the two-row-tile kernel where its schedule is modelled faster than the best plain tile
+        const Rt2Plan plan = rt2_plan(RT2_FP8, ctx->num_sms, M, N, (double)(K / 256), ctx->rt2_doubles);
+        double t = 0.0;
+        pick_tile(FP8_TILES, ctx->num_sms, M, N, (double)(K / 256), &t);
+        if (ctx->rt2 == 1 || plan.t_us < t)
+            return launch_gemm_rt2<Rt2CfgFp8, false>(ctx, plan, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, nullptr, Y, ldy, st,
+                                                     nullptr, layer_call);
     }
     int cfg = ctx->gemm_cfg;
     if (cfg != 4 && cfg != 6 && cfg != 7) cfg = pick_tile(FP8_TILES, ctx->num_sms, M, N, (double)(K / 256)).id;
@@ -1957,7 +1978,7 @@ lynx_status lynx_selftest_wait_timeout(lynx_ctx* ctx, int64_t limit_us, void* st
 // Host-only inspection of the two-row-tile GEMM's plan and schedule (no device is touched).
 int lynx_gemm_plan(int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps, int* doubles, int* clusters) {
     if (num_sms < 2 || M < 1 || N < 8 || K < 128) return -1;
-    const Rt2Plan plan = rt2_plan(num_sms, M, N, K, lora_steps, -1);
+    const Rt2Plan plan = rt2_plan(RT2_BF16, num_sms, M, N, (double)(K / 128) + lora_steps, -1);
     if (doubles) *doubles = plan.doubles;
     if (clusters) *clusters = plan.clusters;
     return (M > 256 && plan.t_us < gemm_model_time(num_sms, M, N, K, lora_steps)) ? 1 : 0;

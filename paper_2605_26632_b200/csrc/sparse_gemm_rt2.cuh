@@ -20,6 +20,10 @@
 // choice (PairSchedule, a cost model): doubles cost less per unit, singles fill the clusters that
 // would otherwise idle in the last round.
 //
+// FP8 operands (Gemm2Cfg<.., true>): the same with 256 logical K per stage, 70 KB and twice the metadata columns, for which
+// tensor memory has two slots (E_SLOTS).  The board's power cap bounds these launches, too (994 W, 1180 MHz): what counts is
+// the bytes not moved.  16384 x 12288 x 3072 307 -> 288 us in blocks of seconds, 4096 x 3072 x 12288 78.0 -> 72.7 in short ones.
+//
 // Roles per CTA (384 threads): warp 0 TMA producer, warp 1 MMA issuer (leader CTA), both converged with
 // one elected lane issuing (see sparse_gemm.cuh), warps 2 and 3 idle, warps 4-11 epilogue.  Every wait is
 // bounded (mbar_wait): on expiry the kernel raises the error word and all roles leave.
@@ -114,6 +118,7 @@ struct Gemm2Params {
     const float* row_scale;      // [M] or nullptr
     const float* scale_partial;  // or: per-K-split row sums of a deferred prune launch
     int scale_ks;
+    const float* col_scale;    // [N] FP8 weight scales or nullptr
     const uint16_t* bias;      // [N] bf16 or nullptr
     const uint16_t* residual;  // [M x N] bf16 (ld = ldr) or nullptr
     int64_t ldr;
@@ -123,13 +128,16 @@ struct Gemm2Params {
     int w_prefetch;  // layer calls: W tiles of the first stages are fetched before the wait for the prune launch
 };
 
-template <int BN_, int STAGES_>
+// FP8_ = true: E4M3 operands, in the byte geometry of a stage as in GemmCfg (256 logical K, twice the metadata).
+template <int BN_, int STAGES_, bool FP8_ = false>
 struct Gemm2Cfg {
     static constexpr int BN = BN_, STAGES = STAGES_, CG = 2;
-    static constexpr int BM = 128, BK = 128;
+    static constexpr bool FP8 = FP8_;
+    static constexpr int BM = 128, BK = FP8 ? 256 : 128;
+    static constexpr int BOX_X = FP8 ? 128 : 64;       // elements of a 128-byte row of A or W
     static constexpr int BN_CTA = BN / CG;
     static constexpr int A_BYTES = BM * 128;           // one row tile of compressed A: 16 KB
-    static constexpr int E_BYTES = 2048;               // its metadata block
+    static constexpr int E_BYTES = FP8 ? 4096 : 2048;  // its metadata
     static constexpr int B_HALF_BYTES = BN_CTA * 128;  // one 128-byte K slice of this CTA's W rows
     static constexpr int B_BYTES = 2 * B_HALF_BYTES;
     static constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * E_BYTES + B_BYTES;
@@ -137,7 +145,11 @@ struct Gemm2Cfg {
     static constexpr int CH = 48;                      // epilogue column chunk
     static constexpr int NCH = BN / CH;
     static constexpr int E_COL0 = 2 * BN;              // metadata columns behind the two accumulators
-    static constexpr int E_COLS = 8;                   // per stage: 4 per row tile
+    static constexpr int E_COLS = 2 * E_BYTES / 512;   // per stage: half of them per row tile
+    // Slots of a stage's metadata in tensor memory.  FP8 stages have 16 columns, and beside two 240-column accumulators
+    // there is room for two of them: the issuer waits for the MMAs of the stage before the last, whose columns it
+    // overwrites.  (The last stage's eight MMAs run meanwhile: nothing stalls.)
+    static constexpr int E_SLOTS = FP8 ? 2 : STAGES;
     static constexpr int TMEM_COLS = 512;
     static constexpr int EPI_WARPS = GEMM_EPI_WARPS;
     static constexpr int THREADS = GEMM_THREADS;
@@ -146,9 +158,10 @@ struct Gemm2Cfg {
     static constexpr int STAGES1 = 4;
     static constexpr int RING1_A = 0, RING1_B = STAGES1 * A_BYTES, RING1_E = RING1_B + STAGES1 * B_BYTES;
     static constexpr int NUM_BARS = 2 * STAGES + 2 * STAGES1 + 4;
-    static constexpr int C_BOX_BYTES = 32 * CH * 2;    // one epilogue warp's staging box: 32 rows x 48 columns
-    static constexpr int C_BYTES = EPI_WARPS * C_BOX_BYTES;
-    static constexpr int BIAS_BYTES = BN * 4;          // the item's bias values (fp32), two items' worth
+    static constexpr int C_BOX_BYTES = 32 * CH * 2;    // a chunk of 32 rows x 48 columns
+    static constexpr int BOX_ROWS = FP8 ? 16 : 32;     // rows of an epilogue warp's own staging box
+    static constexpr int C_BYTES = EPI_WARPS * BOX_ROWS * CH * 2;
+    static constexpr int BIAS_BYTES = BN * 4 * (FP8 ? 2 : 1);  // the item's bias values (and weight scales, fp32), two items' worth
     static constexpr int SMEM_BYTES = 1024 /*align slack*/ + STAGES * STAGE_BYTES + C_BYTES + 2 * BIAS_BYTES + 256;
     // Cycles from one chunk store of a CTA to the next.  The stores compete with the operand stream of the next main
     // loop, whose ring is too short to ride out 122 KB leaving at once: a double's 40 chunks go one after the other,
@@ -165,7 +178,8 @@ struct Gemm2Cfg {
     static_assert(NCH == 5 && BN % CH == 0 && BN_CTA % 8 == 0, "tile N: the epilogue deals five chunks per accumulator");
     static_assert(EPI_WARPS * 5 * C_BOX_BYTES <= STAGES * STAGE_BYTES, "last item: a staging box per chunk in the ring");
     static_assert(B_HALF_BYTES % 1024 == 0, "swizzle atoms need 1024-byte aligned tiles");
-    static_assert(E_COL0 + E_COLS * STAGES <= TMEM_COLS && 4 * STAGES1 <= E_COLS * STAGES, "tensor memory budget");
+    static_assert(E_COL0 + E_COLS * E_SLOTS <= TMEM_COLS && E_COLS / 2 * STAGES1 <= E_COLS * E_SLOTS, "tensor memory budget");
+    static_assert(E_SLOTS == STAGES || (E_SLOTS == 2 && STAGES == 3), "the issuer looks two stages back");
     static_assert(RING1_E + STAGES1 * E_BYTES <= STAGES * STAGE_BYTES, "the single-tile ring fits into the double ring's memory");
     static_assert(8 * NUM_BARS + 16 <= 256, "barrier area");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
@@ -252,7 +266,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
             const uint32_t b_dst = r1 ? sA + Cfg::RING1_B + s * Cfg::B_BYTES : sB + s * Cfg::B_BYTES;
             if (leader) mbar_arrive_expect_tx(bfull + 8 * s, 2 * tx);
             tma_load_2d_pair(b_dst, &tmap_b, s * Cfg::BK, n0, full0 + 8 * s);
-            tma_load_2d_pair(b_dst + Cfg::B_HALF_BYTES, &tmap_b, s * Cfg::BK + 64, n0, full0 + 8 * s);
+            tma_load_2d_pair(b_dst + Cfg::B_HALF_BYTES, &tmap_b, s * Cfg::BK + Cfg::BOX_X, n0, full0 + 8 * s);
         }
     }
     // everything above overlapped the previous kernel's tail; its results are needed from here on
@@ -263,6 +277,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     if (warp == 0) {
         // ------------------------------------------------------------------ producer ----------
         {
+            constexpr int E_ROWS = Cfg::E_BYTES / 1024;  // 1024-byte rows of the metadata tensor map per stage and row tile
             uint32_t stage = 0, phase = 0, issued = 0;
             bool ok = true;
             bool ring1 = false;  // false: the 3 x 66 KB ring of the doubles, true: the 4 x 48 KB ring of the singles
@@ -300,15 +315,15 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                         const bool pre = it == 0 && kb < npre;  // W tile and byte count went out before the wait
                         // the leader announces the bytes of both CTAs; the peer's bytes may land first
                         if (leader && !pre) mbar_arrive_expect_tx(bfull + 8 * stage, 2 * tx);
-                        tma_load_2d_pair(a_dst, &tmap_a, kb * 64, rb0 * Cfg::BM, bar);
-                        tma_load_2d_pair(e_dst, &tmap_e, 0, 2 * (rb0 * kblocks + kb), bar);
+                        tma_load_2d_pair(a_dst, &tmap_a, kb * Cfg::BOX_X, rb0 * Cfg::BM, bar);
+                        tma_load_2d_pair(e_dst, &tmap_e, 0, E_ROWS * (rb0 * kblocks + kb), bar);
                         if (!pre) {
                             tma_load_2d_pair(b_dst, &tmap_b, kb * Cfg::BK, n0, bar);
-                            tma_load_2d_pair(b_dst + Cfg::B_HALF_BYTES, &tmap_b, kb * Cfg::BK + 64, n0, bar);
+                            tma_load_2d_pair(b_dst + Cfg::B_HALF_BYTES, &tmap_b, kb * Cfg::BK + Cfg::BOX_X, n0, bar);
                         }
                         if (rows == 2) {
-                            tma_load_2d_pair(a_dst + Cfg::A_BYTES, &tmap_a, kb * 64, (rb0 + 2) * Cfg::BM, bar);
-                            tma_load_2d_pair(e_dst + Cfg::E_BYTES, &tmap_e, 0, 2 * ((rb0 + 2) * kblocks + kb), bar);
+                            tma_load_2d_pair(a_dst + Cfg::A_BYTES, &tmap_a, kb * Cfg::BOX_X, (rb0 + 2) * Cfg::BM, bar);
+                            tma_load_2d_pair(e_dst + Cfg::E_BYTES, &tmap_e, 0, E_ROWS * ((rb0 + 2) * kblocks + kb), bar);
                         }
                     } else {
                         // low-rank stages: T boxes in the A slots, L_A box in the first half of the W slot
@@ -341,7 +356,10 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
             const uint32_t b_lo0 = (uint32_t)make_desc_sw128(sB);
             const uint64_t e_d0 = make_desc_rows16(sE), e1_d0 = make_desc_rows16(sA + Cfg::RING1_E);
             constexpr uint32_t BH = Cfg::B_HALF_BYTES >> 4;
+            constexpr uint32_t idesc8 = make_idesc_sp_e4m3(Cfg::BM * 2, BN);
+            constexpr int E_HALF = Cfg::E_COLS / 2;  // metadata columns of one row tile
             uint32_t stage = 0, phase = 0;
+            uint32_t e_slot = 0;  // FP8 doubles: the stage's metadata slot
             bool ring1 = false;
             AccTurns turns;
             bool ok = true;
@@ -375,14 +393,34 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                                                 : ring_lo0 + stage * (2 * Cfg::A_BYTES >> 4);
                     const uint32_t b_lo = ring1 ? ring_lo0 + ((Cfg::RING1_B + stage * Cfg::B_BYTES) >> 4)
                                                 : b_lo0 + stage * (Cfg::B_BYTES >> 4);
-                    const uint32_t e_tmem = tmem_base + Cfg::E_COL0 + (ring1 ? 4 * stage : Cfg::E_COLS * stage);
+                    if constexpr (Cfg::E_SLOTS < STAGES) {
+                        if (!ring1) {
+                            // the stage before the last one: with three stages the next one of the ring, a round back
+                            // (a fresh barrier passes)
+                            const uint32_t older = stage == STAGES - 1 ? 0u : stage + 1;
+                            if (!mbar_wait_warp(bempty + 8 * older, older ? phase ^ 1u : phase, cta_abort, p.dev_error)) {
+                                ok = false;
+                                break;
+                            }
+                            tc_fence_after();
+                            e_slot ^= 1u;
+                        }
+                    }
+                    const uint32_t e_tmem = tmem_base + Cfg::E_COL0 +
+                                            (ring1 ? E_HALF * stage : Cfg::E_COLS * (Cfg::E_SLOTS < STAGES ? e_slot : stage));
                     const uint64_t e_desc = ring1 ? e1_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4))
                                                   : e_d0 + (uint64_t)(stage * (2 * Cfg::E_BYTES >> 4));
                     const bool sparse = kb < kblocks;
                     // one row tile's MMAs of this stage
                     auto issue = [&](int r) {
-                        const uint32_t dt = d_tmem + r * BN, al = a_lo + r * (Cfg::A_BYTES >> 4), et = e_tmem + 4 * r;
-                        if (sparse) {
+                        const uint32_t dt = d_tmem + r * BN, al = a_lo + r * (Cfg::A_BYTES >> 4), et = e_tmem + E_HALF * r;
+                        if constexpr (Cfg::FP8) {
+                            // four K steps of 64 logical elements: A advances 32 bytes, W 64 bytes, metadata two columns
+                            mma_sp_f8_lh<2>(dt, al, b_lo, desc_hi, et, idesc8, accumulate);
+                            mma_sp_f8_lh<2>(dt, al + 2, b_lo + 4, desc_hi, et + 2, idesc8, 1u);
+                            mma_sp_f8_lh<2>(dt, al + 4, b_lo + BH, desc_hi, et + 4, idesc8, 1u);
+                            mma_sp_f8_lh<2>(dt, al + 6, b_lo + BH + 4, desc_hi, et + 6, idesc8, 1u);
+                        } else if (sparse) {
                             // four K steps of 32 logical elements: A advances 32 bytes, W 64 bytes (steps 2, 3 in
                             // the second 64-element slice); metadata column pair + step parity
                             mma_sp_bf16_lh<2>(dt, al, b_lo, desc_hi, et, idesc0, accumulate);
@@ -399,8 +437,14 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     };
                     if (elect_one()) {
                         if (sparse) {
-                            tmem_cp_128x128b<2>(e_tmem, e_desc);
-                            if (rows == 2) tmem_cp_128x128b<2>(e_tmem + 4, e_desc + (uint64_t)(Cfg::E_BYTES >> 4));
+                            // (a row tile's 128 x 128 metadata blocks, one or two: four columns each)
+#pragma unroll
+                            for (int j = 0; j < E_HALF / 4; ++j) tmem_cp_128x128b<2>(e_tmem + 4 * j, e_desc + (uint64_t)(j * (2048 >> 4)));
+                            if (rows == 2) {
+#pragma unroll
+                                for (int j = 0; j < E_HALF / 4; ++j)
+                                    tmem_cp_128x128b<2>(e_tmem + E_HALF + 4 * j, e_desc + (uint64_t)((Cfg::E_BYTES + j * 2048) >> 4));
+                            }
                         }
                         issue(0);
                         if (kb == ksteps - 1) tc_commit_pair(bar_tfull + 8 * acc0, 0x3);
@@ -435,7 +479,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         const int h = (warp - GEMM_EPI_WARP0) >> 2;  // which of the quarter's two warps
         const int q = warp & 3;         // tensor-memory lane quarter this warp may read
         const uint32_t tempty0 = mapa(bar_tempty, 0);
-        const uint32_t own_box = sC + (warp - GEMM_EPI_WARP0) * Cfg::C_BOX_BYTES;
+        const uint32_t own_box = sC + (warp - GEMM_EPI_WARP0) * (Cfg::C_BYTES / Cfg::EPI_WARPS);
         constexpr int CH = Cfg::CH, NCH = Cfg::NCH;
         const int n_first = h == 0 ? 3 : 2;  // chunks of the item's first accumulator
         AccTurns turns;
@@ -446,10 +490,11 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
             const bool last = it == num_items - 1;
             const int acc0 = (rows == 2) ? 0 : (ordinal & 1);
             // the item's bias values as fp32, for all epilogue warps (the other parity's may still be read)
-            const uint32_t sb = sBias + (it & 1) * Cfg::BIAS_BYTES;
+            const uint32_t sb = sBias + (it & 1) * Cfg::BIAS_BYTES, sc = sb + BN * 4;
             if (const int c = (int)threadIdx.x - 32 * GEMM_EPI_WARP0; c < BN) {
                 const int n = tn * BN + c;
                 sts32f(sb + c * 4, (p.bias != nullptr && n < p.N) ? __uint_as_float((uint32_t)__ldg(p.bias + n) << 16) : 0.0f);
+                if constexpr (Cfg::FP8) sts32f(sc + c * 4, (p.col_scale != nullptr && n < p.N) ? __ldg(p.col_scale + n) : 1.0f);
             }
             bar_sync_named(GEMM_EPI_BARRIER, 32 * Cfg::EPI_WARPS);  // every warp passes it once per item, whatever became of its waits
             if (!alive) continue;
@@ -511,7 +556,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     float sr[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) sr[i] = r ? s[1][i] : s[0][i];
-                    epi_convert<CH, false, RES>(v, sr, sb + c * (CH * 4), 0u, lane, packed[slot]);
+                    epi_convert<CH, Cfg::FP8, RES>(v, sr, sb + c * (CH * 4), sc + c * (CH * 4), lane, packed[slot]);
                 }
             };
             if (p.residual != nullptr) convert(std::true_type{});
@@ -532,7 +577,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                 // rows past M and columns past N are clipped by the store.  The last item stages in the ring:
                 // its MMAs are done (the wait above) and nothing is loaded any more.
                 if (n0 < p.N)
-                    epi_store<CH, 32>(&tmap_y, packed[slot], n0, m0 + r * 256,
+                    epi_store<CH, Cfg::BOX_ROWS>(&tmap_y, packed[slot], n0, m0 + r * 256,
                                       last ? smem_base + ((warp - GEMM_EPI_WARP0) * NCH + slot) * Cfg::C_BOX_BYTES : own_box, last, lane);
             }
         }

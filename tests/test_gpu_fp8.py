@@ -316,3 +316,31 @@ def test_fp8_argument_errors(lx):
         lx.prune_compress_fp8(X, 2)  # whole-tensor scale is not available in FP8
     assert e.value.status == 1
     assert lx.launch_count() == n0
+
+
+@pytest.mark.parametrize("doubles", [0, 20, 100000])
+@pytest.mark.parametrize("M,K,N", [(512, 256, 240), (700, 1024, 1000), (1537, 2304, 3000), (2570, 768, 6160)])
+def test_two_row_tile_gemm_equals_the_single_tile_kernel(M, K, N, doubles, monkeypatch):
+    """Same MMAs in the same order per element, whatever the schedule: bit for bit, with stages that reuse the two metadata
+    slots (1, 4, 9 and 3 K blocks), switches from doubles to singles, ragged rows and columns, with and without residual."""
+    from paper_2605_26632_b200 import binding
+
+    X, W = inputs.make_x(M, K, "outlier", 88).cuda(), inputs.make_w(N, K, 88).cuda()
+    b, res = inputs.make_bias(N, 88).cuda(), inputs.make_residual(M, N, 88).cuda()
+    monkeypatch.setenv("LYNX_GEMM_CFG", "7")
+    single = binding.Lynx(0)
+    monkeypatch.setenv("LYNX_GEMM_CFG", "0")
+    monkeypatch.setenv("LYNX_RT2", "1")
+    monkeypatch.setenv("LYNX_RT2_D", str(doubles))
+    ctx = binding.Lynx(0)
+    try:
+        Wq, ws = single.quantize_weights_fp8(W, True)
+        for r in (None, res):
+            Y = single.act_sparse_linear_fp8(X, Wq, ws, b, 1, r)
+            for _ in range(2):
+                assert torch.equal(ctx.act_sparse_linear_fp8(X, Wq, ws, b, 1, r), Y)
+        torch.cuda.synchronize()
+        assert ctx.last_error() == 0
+    finally:
+        single.close()
+        ctx.close()
