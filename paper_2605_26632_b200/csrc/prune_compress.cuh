@@ -11,7 +11,7 @@
 //
 // Selection runs on pairs of groups with 16-bit lanes packed in 32-bit registers: the six
 // "magnitude_i >= magnitude_j" comparisons (i < j) are borrow-free packed subtractions with a guard
-// bit, the keep flags are bitwise majorities, and the kept positions come from a 16-entry table.
+// bit, the keep flags are bitwise majorities, and the kept positions come from a table of eight entries.
 #pragma once
 
 #include "ptx.cuh"
@@ -25,37 +25,44 @@ __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
     return (a & b) | (a & c) | (b & c);
 }
 
+// bit by bit: a where the mask is set, b elsewhere
+__device__ __forceinline__ uint32_t bit_select(uint32_t mask, uint32_t a, uint32_t b) { return (a & mask) | (b & ~mask); }
+
 // Keep patterns of two groups A = (a01, a23) and B = (b01, b23) (each register holds two bf16,
 // lower index in the lower half).  Returns 4*pattern(A) in bits 0..15 and 4*pattern(B) in bits
-// 16..31, where bit i of a pattern says element i is kept.
+// 16..31, where bit i of a pattern says that element i is kept, i < 3 (two of four are: the fourth follows).
 //
 // Element i outranks element j (i < j) iff mag_i >= mag_j (ties go to the lower index); an
 // element is kept iff fewer than two others outrank it.
-__device__ __forceinline__ uint32_t keep_patterns_x2(uint32_t a01, uint32_t a23, uint32_t b01,
-                                                     uint32_t b23) {
+//
+// Its instructions are most of a prune kernel's (25 of the ALU pipe per two groups).  With a fourth flag, gathered by a shift and
+// a mask each, it was 28: prune of 4096 x 12288 25.2 -> 24.6 us, prune + down projection of 4352 x 3072 12.9 -> 12.5.  The
+// differences as multiply-adds (19 + 6 on the other pipe) gain 1 % there and lose 6 % with the down projection: not used.
+__device__ __forceinline__ uint32_t keep_patterns_x2(uint32_t a01, uint32_t a23, uint32_t b01, uint32_t b23) {
     const uint32_t MAG = 0x7FFF7FFFu, GUARD = 0x80008000u;
     // x_i = (A's element i, B's element i)
     const uint32_t x0 = prmt(a01, b01, 0x5410), x1 = prmt(a01, b01, 0x7632);
     const uint32_t x2 = prmt(a23, b23, 0x5410), x3 = prmt(a23, b23, 0x7632);
-    const uint32_t g0 = (x0 & MAG) | GUARD, g1 = (x1 & MAG) | GUARD, g2 = (x2 & MAG) | GUARD;
+    const uint32_t g0 = x0 | GUARD, g1 = x1 | GUARD, g2 = x2 | GUARD;
     const uint32_t m1 = x1 & MAG, m2 = x2 & MAG, m3 = x3 & MAG;
     // bit 15 / bit 31 of (guard|mag_i) - mag_j is set iff mag_i >= mag_j; the guard bit keeps
     // every 16-bit lane positive so no borrow crosses lanes
     const uint32_t c01 = g0 - m1, c02 = g0 - m2, c03 = g0 - m3;
     const uint32_t c12 = g1 - m2, c13 = g1 - m3, c23 = g2 - m3;
-    const uint32_t k0 = maj3(c01, c02, c03);     // not outranked by 1, 2, 3 (at least two of)
-    const uint32_t k1 = maj3(~c01, c12, c13);    // not outranked by 0, 2, 3
-    const uint32_t k2 = maj3(~c02, ~c12, c23);   // not outranked by 0, 1, 3
-    const uint32_t k3 = maj3(~c03, ~c13, ~c23);  // not outranked by 0, 1, 2
-    return ((k0 >> 13) & 0x00040004u) | ((k1 >> 12) & 0x00080008u) | ((k2 >> 11) & 0x00100010u) |
-           ((k3 >> 10) & 0x00200020u);
+    const uint32_t k0 = maj3(c01, c02, c03);    // not outranked by 1, 2, 3 (at least two of)
+    const uint32_t k1 = maj3(~c01, c12, c13);   // not outranked by 0, 2, 3
+    const uint32_t k2 = maj3(~c02, ~c12, c23);  // not outranked by 0, 1, 3
+    // flags side by side below bit 15 / bit 31, then down to bits 2..4 / 18..20
+    const uint32_t k01 = bit_select(GUARD, k1, k0 >> 1);
+    return (bit_select(GUARD, k2, k01 >> 1) >> 11) & 0x001C001Cu;
 }
 
-// Table entry for a keep pattern with bits i0 < i1 set, copy j (j = position of the group's
-// nibble in its 16-bit metadata word):  low 16 bits = byte-permute selector that packs elements
-// i0, i1 into one register;  bits 16+4j.. = nibble i0 | i1 << 2.
-__device__ __forceinline__ uint32_t prune_lut_entry(uint32_t pattern, int j) {
-    if (__popc(pattern) != 2) return 0;
+// Table entry for the flags of elements 0..2 (bit i: element i is kept; the fourth is if they are one too few), copy j (j =
+// position of the group's nibble in its 16-bit metadata word):  low 16 bits = byte-permute selector that packs the kept
+// elements i0 < i1 into one register;  bits 16+4j.. = nibble i0 | i1 << 2.
+__device__ __forceinline__ uint32_t prune_lut_entry(uint32_t flags, int j) {
+    const uint32_t pattern = __popc(flags) == 1 ? flags | 8u : flags;
+    if (flags > 7 || __popc(pattern) != 2) return 0;
     const uint32_t i0 = __ffs(pattern) - 1, i1 = 31 - __clz(pattern);
     const uint32_t sel = (2 * i0) | ((2 * i0 + 1) << 4) | ((2 * i1) << 8) | ((2 * i1 + 1) << 12);
     return sel | ((i0 | (i1 << 2)) << (16 + 4 * j));
