@@ -1394,7 +1394,17 @@ static lynx_status prune_impl(lynx_ctx* ctx, const void* X, int64_t M, int64_t K
     }
     ctx->launches++;
     if (mode == LYNX_COMP_TENSOR) {
-        tensor_scale_kernel<<<1, 1024, 0, st>>>(sums, M, row_scale);
+        cudaLaunchConfig_t tc = {};
+        tc.gridDim = dim3(1);
+        tc.blockDim = dim3(1024);
+        tc.stream = st;
+        cudaLaunchAttribute tattr[1];
+        tattr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        tattr[0].val.programmaticStreamSerializationAllowed = ctx->pdl ? 1 : 0;
+        tc.attrs = tattr;
+        tc.numAttrs = 1;
+        const float* row_sums = sums;
+        if (cudaLaunchKernelEx(&tc, tensor_scale_kernel, row_sums, M, row_scale) != cudaSuccess) return LYNX_ERR_CUDA;
         ctx->launches++;
     }
     if (src) {

@@ -411,28 +411,48 @@ row_scale_finalize_kernel(const float* __restrict__ partial, int64_t M, int KS, 
 }
 
 // Whole-tensor scale: s = sqrt(sum_m num_m / (sum_m den_m + eps)), written to every row_scale[m].
-// One CTA; fp64 partial sums in a fixed order.
+// One CTA; fp64 partial sums in a fixed order.  Its time is latency: the loads, the tree, and the two launches around
+// it, which overlap with their neighbours (programmatic dependents).  With one load at a time, a barrier per level and a plain
+// launch the layer 1359 x 3072 x 3072 took 24.5 us, now 20.6; 256 x 3072 x 3072 15.5 -> 13.3.
 __global__ void __launch_bounds__(1024)
 tensor_scale_kernel(const float* __restrict__ sums, int64_t M, float* __restrict__ row_scale) {
     __shared__ double sn[1024], sd[1024];
+    __shared__ float scale;
     const int tid = threadIdx.x;
+    griddep_wait();
+    griddep_launch_dependents();  // the GEMM behind it runs its prologue meanwhile
     double num = 0.0, den = 0.0;
-    for (int64_t m = tid; m < M; m += 1024) {
-        num += (double)sums[2 * m];
-        den += (double)sums[2 * m + 1];
+    const float2* pairs = reinterpret_cast<const float2*>(sums);
+    for (int64_t m0 = tid; m0 < M; m0 += 8 * 1024) {  // eight loads in flight
+        float2 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = m0 + u * 1024 < M ? __ldcg(pairs + m0 + u * 1024) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            num += (double)v[u].x;
+            den += (double)v[u].y;
+        }
     }
     sn[tid] = num;
     sd[tid] = den;
     __syncthreads();
-    for (int s = 512; s > 0; s >>= 1) {
+    for (int s = 512; s >= 32; s >>= 1) {
         if (tid < s) {
-            sn[tid] += sn[tid + s];
-            sd[tid] += sd[tid + s];
+            sn[tid] = num += sn[tid + s];
+            sd[tid] = den += sd[tid + s];
         }
         __syncthreads();
     }
-    const float sc = (float)sqrt(sn[0] / (sd[0] + 1e-8));
-    for (int64_t m = tid; m < M; m += 1024) row_scale[m] = sc;
+    if (tid < 32) {  // the same tree within a warp
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) {
+            num += __shfl_down_sync(0xffffffffu, num, s);
+            den += __shfl_down_sync(0xffffffffu, den, s);
+        }
+        if (tid == 0) scale = (float)sqrt(num / (den + 1e-8));
+    }
+    __syncthreads();
+    for (int64_t m = tid; m < M; m += 1024) row_scale[m] = scale;
 }
 
 // ---- inspection helpers -------------------------------------------------------------------------
