@@ -1060,30 +1060,40 @@ lynx_status launch_lora_down(lynx_ctx* ctx, const void* X, int64_t M, int64_t K,
     return LYNX_OK;
 }
 
-// K splits of the prune + down-projection kernel (128-element K blocks) = CTAs per cluster, 1..8.
-// Every CTA holds a whole SM; `cap[i]` = CTAs of clusters of i + 1 that the GPU holds at once.
-void prune_lora_plan(const int cap[8], int64_t M, int64_t K, int* splits, int* kb_per_split) {
-    const int tiles_m = (int)((M + 127) / 128), kblocks = (int)(K / 128);
-    int best_s = 1, best_per = kblocks;
-    double best = 1e30;
-    for (int i = 0; i < 8; ++i) {
-        const int sp = i + 1;
-        if (sp > kblocks) break;
-        if (cap[i] < sp) continue;
-        const int per = (kblocks + sp - 1) / sp;
-        if ((kblocks + per - 1) / per != sp) continue;  // every CTA of the cluster needs a K block
-        const double rounds = (double)(((int64_t)tiles_m * sp + cap[i] - 1) / cap[i]);
-        const double t = rounds * (per + 4.0);
-        if (t < best) { best = t; best_s = sp; best_per = per; }
+// Plan of the prune + down-projection kernel: rows per block and K splits (128-element K blocks) = CTAs per cluster.
+// Every CTA holds a whole SM; `cap[i]` = CTAs of clusters of i that the GPU holds at once.  Figures (us) fitted to 13 shapes with
+// every plan forced: a K block of 128 rows 1.04, of 64 rows 0.6, and what a CTA adds (first loads, drain, the cluster's
+// exchange).  64-row blocks where they fill more of the GPU: 4352 x 3072 13.2 -> 11.7 (136 CTAs of 12 half blocks instead of 102
+// of 8; four splits of 128 rows are one cluster too many), 1024 x 3072 10.0 -> 8.0, 1621 x 1024 7.0 -> 5.9; not 4096 x 12288
+// (31.4 against 33.1) and 12271 x 3072 (30.5 against 37.3), where 128-row blocks fill it as well.
+struct PruneLoraPlan {
+    int rows, splits, kb_per_split;
+};
+PruneLoraPlan prune_lora_plan(const int (&cap)[9], int64_t M, int64_t K, int force_rows = 0, int force_splits = 0) {
+    const int kblocks = (int)(K / 128);
+    PruneLoraPlan best{128, 1, kblocks};
+    double best_t = 1e30;
+    for (int rows = 128; rows >= 64; rows /= 2) {
+        if (force_rows && rows != force_rows) continue;
+        const int64_t blocks = (M + 127) / 128 * (128 / rows);  // whole 128-row blocks of metadata
+        // (64-row blocks leave two partial sums per split and row, up to eight of which are added in ascending order)
+        for (int sp = 1; sp <= (rows == 128 ? 8 : 4) && sp <= kblocks; ++sp) {
+            if (cap[sp] < sp || (force_splits && sp != force_splits)) continue;
+            const int per = (kblocks + sp - 1) / sp;
+            if ((kblocks + per - 1) / per != sp) continue;  // every CTA of the cluster needs a K block,
+            if (rows == 64 && kblocks - (sp - 1) * per < 2) continue;  // every group of its prune warps one, too
+            const double rounds = (double)((blocks * sp + cap[sp] - 1) / cap[sp]);
+            const double t = rounds * (rows == 128 ? per * 1.04 + 5.2 + 0.15 * sp : per * 0.6 + 4.3 + 0.15 * sp);
+            if (t < best_t) { best_t = t; best = PruneLoraPlan{rows, sp, per}; }
+        }
     }
-    *splits = best_s;
-    *kb_per_split = best_per;
+    return best;
 }
 
 template <class Cfg, bool SUMS>
 lynx_status launch_prune_lora(lynx_ctx* ctx, const void* X, int64_t M, int64_t K, int64_t ldx, const void* LB,
                               int64_t ldlb, void* values, void* meta, float* scale_partial, void* T, int64_t ldt,
-                              cudaStream_t st, int* splits_out) {
+                              cudaStream_t st, const PruneLoraPlan& plan) {
     CUtensorMap tx, tlb;
     if (!make_tmap_2d(ctx, &tx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)K, (uint64_t)ldx * 2, 64,
                       Cfg::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
@@ -1093,38 +1103,10 @@ lynx_status launch_prune_lora(lynx_ctx* ctx, const void* X, int64_t M, int64_t K
     auto kern = prune_lora_kernel<Cfg, SUMS>;
     static bool attr_set[MAX_CTX_DEVICES] = {};  // per instantiation
     if (lynx_status as = allow_dynamic_smem(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
-    // how many CTAs of clusters of 1..8 fit on the GPU at once (asked once per device)
-    static int caps[MAX_CTX_DEVICES][8] = {};
-    int* cap = caps[ctx->device];
-    if (cap[0] == 0) {
-        for (int i = 0; i < 8; ++i) {
-            cudaLaunchConfig_t qc = {};
-            qc.gridDim = dim3((unsigned)(ctx->num_sms / (i + 1) * (i + 1)));
-            qc.blockDim = dim3(Cfg::THREADS);
-            qc.dynamicSmemBytes = Cfg::SMEM_BYTES;
-            cudaLaunchAttribute qa[1];
-            qa[0].id = cudaLaunchAttributeClusterDimension;
-            qa[0].val.clusterDim.x = (unsigned)(i + 1);
-            qa[0].val.clusterDim.y = 1;
-            qa[0].val.clusterDim.z = 1;
-            qc.attrs = qa;
-            qc.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, kern, &qc) != cudaSuccess) n = 0;
-            cap[i] = n * (i + 1);
-        }
-        if (cap[0] <= 0) cap[0] = ctx->num_sms;
-    }
     PruneLoraParams p;
     p.M = M; p.K = K;
-    prune_lora_plan(cap, M, K, &p.splits, &p.kb_per_split);
-    if (const int f = ctx->pl_force_splits; f >= 1 && f <= 8 && cap[f - 1] >= f) {
-        const int kblocks = (int)(K / 128), per = (kblocks + f - 1) / f;
-        if (f <= kblocks && (kblocks + per - 1) / per == f) {  // every CTA of the cluster gets a K block
-            p.splits = f;
-            p.kb_per_split = per;
-        }
-    }
+    p.splits = plan.splits;
+    p.kb_per_split = plan.kb_per_split;
     p.zero = 0;
     p.values = static_cast<uint16_t*>(values);
     p.meta = static_cast<uint8_t*>(meta);
@@ -1132,7 +1114,7 @@ lynx_status launch_prune_lora(lynx_ctx* ctx, const void* X, int64_t M, int64_t K
     p.T = static_cast<uint16_t*>(T);
     p.ldt = ldt;
     p.dev_error = ctx->err_dev;
-    const int tiles_m = (int)((M + Cfg::BM - 1) / Cfg::BM);
+    const int tiles_m = (int)((M + 127) / 128) * (128 / Cfg::BM);  // whole 128-row blocks of metadata
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles_m * p.splits));
     cfg.blockDim = dim3(Cfg::THREADS);
@@ -1149,7 +1131,6 @@ lynx_status launch_prune_lora(lynx_ctx* ctx, const void* X, int64_t M, int64_t K
     cfg.numAttrs = 2;
     if (cudaLaunchKernelEx(&cfg, kern, tx, tlb, p) != cudaSuccess) return LYNX_ERR_CUDA;
     ctx->launches++;
-    *splits_out = p.splits;
     return LYNX_OK;
 }
 
@@ -1212,6 +1193,7 @@ lynx_status lynx_create(lynx_ctx** out, int device) {
             if (cudaOccupancyMaxActiveClusters(&n, kern, &qc) == cudaSuccess) ctx->cluster_cap[i] = n * i;
         }
         (void)cudaGetLastError();  // (a size that does not fit leaves its count at zero: no such plan)
+        if (ctx->cluster_cap[1] <= 0) ctx->cluster_cap[1] = ctx->num_sms;
     }
     // Development overrides (tile configuration, schedules, kernel forms) are read only when
     // LYNX_DEV=1 is set: tests and measurement scripts set it, a production process reads nothing else.
@@ -1231,7 +1213,7 @@ lynx_status lynx_create(lynx_ctx** out, int device) {
         geti("LYNX_DEFER_SCALE", &ctx->defer_scale);
         geti("LYNX_PRUNE_TPU", &ctx->prune_tpu);          // 128-element K blocks per warp
         geti("LYNX_GEMM_GROUP_M", &ctx->gemm_group_m);    // row tiles per group of the GEMM's tile order
-        geti("LYNX_PL_SPLITS", &ctx->pl_force_splits);    // K splits (= cluster size) of the prune + down-projection kernel
+        geti("LYNX_PL_SPLITS", &ctx->pl_force_splits);    // K splits (= cluster size) of the prune + down-projection kernel, + 10: 64-row blocks
         if (geti("LYNX_FP8_RING", &ctx->fp8_ring)) ctx->fp8_ring_forced = 1;  // 0 = one CTA per 16 rows, n = ring with n warps per row
         geti("LYNX_RT2", &ctx->rt2);                      // two-row-tile GEMM kernel: 0 never, 1 whenever it applies
         geti("LYNX_RT2_D", &ctx->rt2_doubles);            // and the number of 512-row items of its schedule
@@ -1648,14 +1630,21 @@ static lynx_status prune_lora_impl(lynx_ctx* ctx, const void* X, int64_t M, int6
     if ((s = check_device_error(ctx)) != LYNX_OK) return s;
     float* spart = reinterpret_cast<float*>(static_cast<char*>(ctx->scratch) + L.partial);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int splits = 0;
     const bool sums = mode == LYNX_COMP_ROW;
-    if (R == 64)
-        s = sums ? launch_prune_lora<PruneLoraCfg<64>, true>(ctx, X, M, K, ldx, LB, ldlb, values, meta, spart, T, ldt, st, &splits)
-                 : launch_prune_lora<PruneLoraCfg<64>, false>(ctx, X, M, K, ldx, LB, ldlb, values, meta, nullptr, T, ldt, st, &splits);
-    else
-        s = sums ? launch_prune_lora<PruneLoraCfg<128>, true>(ctx, X, M, K, ldx, LB, ldlb, values, meta, spart, T, ldt, st, &splits)
-                 : launch_prune_lora<PruneLoraCfg<128>, false>(ctx, X, M, K, ldx, LB, ldlb, values, meta, nullptr, T, ldt, st, &splits);
+    PruneLoraPlan plan = prune_lora_plan(ctx->cluster_cap, M, K);
+    if (ctx->pl_force_splits) {  // development override: cluster size, + 10 for 64-row blocks, where it applies
+        const int rows = ctx->pl_force_splits >= 10 ? 64 : 128;
+        const PruneLoraPlan forced = prune_lora_plan(ctx->cluster_cap, M, K, rows, ctx->pl_force_splits % 10);
+        if (forced.rows == rows && forced.splits == ctx->pl_force_splits % 10) plan = forced;
+    }
+    const int splits = plan.splits * (128 / plan.rows);  // partial sums per row
+    auto go = [&](auto cfg) {
+        using Cfg = decltype(cfg);
+        return sums ? launch_prune_lora<Cfg, true>(ctx, X, M, K, ldx, LB, ldlb, values, meta, spart, T, ldt, st, plan)
+                    : launch_prune_lora<Cfg, false>(ctx, X, M, K, ldx, LB, ldlb, values, meta, nullptr, T, ldt, st, plan);
+    };
+    if (R == 64) s = plan.rows == 128 ? go(PruneLoraCfg<64, 128>{}) : go(PruneLoraCfg<64, 64>{});
+    else s = plan.rows == 128 ? go(PruneLoraCfg<128, 128>{}) : go(PruneLoraCfg<128, 64>{});
     if (s != LYNX_OK) return s;
     // the scratch's sums now belong to this call, in this kernel's split count
     ctx->deferred_partial = sums ? spart : nullptr;

@@ -5,8 +5,8 @@
 //     T[m, r] = bf16( (sum_k X[m,k] L_B[r,k]) / s_m )
 // Both consumers want every element of X exactly once, so X crosses HBM once instead of twice.
 //
-// One CTA per (128-row block, K split); the splits of a row block form a thread-block cluster
-// (1 to 8 CTAs).  Warp 0: TMA producer -- a stage is 128 rows x 128 K of X
+// One CTA per (row block of 128 or 64 rows, K split); the splits of a row block form a thread-block cluster
+// (1 to 8 CTAs).  Warp 0: TMA producer -- a stage is (128-row blocks) 128 rows x 128 K of X
 // (two 128-byte-swizzled boxes of 64 elements) plus the matching R x 128 slice of L_B.  Warp 1
 // issues eight dense tcgen05.mma (K = 16) per stage into a 128 x R fp32 accumulator in tensor
 // memory.  Warps 6..13 each read one 16 x 128 tile of the stage out of shared memory (undoing the
@@ -45,17 +45,21 @@ struct PruneLoraParams {
     uint32_t zero;  // 0
 };
 
-template <int R_>
+// BM: rows of a row block, 128 or 64.  The MMAs are 128 rows high either way: of 64-row blocks the other half of the A operand
+// is whatever lies behind the box in the ring (rows of the result that nobody reads).
+template <int R_, int BM_>
 struct PruneLoraCfg {
     static constexpr int R = R_;
-    static constexpr int BM = 128, BK = 128;
-    static constexpr int STAGES = (R == 64) ? 4 : 3;
-    static constexpr int X_BOX_BYTES = BM * 128;      // 128 rows x 64 elements: 16 KB
+    static constexpr int BM = BM_, BK = 128;
+    static constexpr int STAGES = BM == 128 ? ((R == 64) ? 4 : 3) : ((R == 64) ? 6 : 4);
+    static constexpr int X_BOX_BYTES = BM * 128;      // BM rows x 64 elements
     static constexpr int X_BYTES = 2 * X_BOX_BYTES;
     static constexpr int B_BOX_BYTES = R * 128;       // R rows x 64 elements
     static constexpr int B_BYTES = 2 * B_BOX_BYTES;
     static constexpr int STAGE_BYTES = X_BYTES + B_BYTES;
     static constexpr int PRUNERS = 8;                 // warps, one 16 x 128 tile each per stage
+    static constexpr int TILES = BM / 16;             // tiles of a stage: TURNS groups of prune warps take the stages in turn
+    static constexpr int TURNS = PRUNERS / TILES;
     static constexpr int THREADS = 64 + 128 + 32 * PRUNERS;
     static constexpr int TAIL_THREADS = 128 + 32 * PRUNERS;  // drain + prune warps meet once at the end
     static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 1536;
@@ -63,6 +67,8 @@ struct PruneLoraCfg {
     static constexpr int PARTIAL_BYTES = BM * R * 4;  // the drained accumulator, kept in the L_B ring
     static_assert(PARTIAL_BYTES <= STAGES * B_BYTES, "the partial fits where the L_B stages were");
     static_assert(R == 64 || R == 128, "rank");
+    static_assert((BM == 128 || BM == 64) && STAGES % TURNS == 0, "row block");
+    static_assert(X_BOX_BYTES + 128 * 128 <= X_BYTES + STAGES * B_BYTES, "the last stage's MMAs read inside the ring");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 };
 
@@ -82,12 +88,10 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     uint8_t* tail = smem_gen + (sBar - smem_base);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 128);
     volatile uint32_t* cta_abort = tmem_slot + 1;
-    const uint32_t s_sums = sBar + 256;  // [128] (sum x^2, sum kept^2) of this split's rows
+    const uint32_t s_sums = sBar + 256;  // [turn][row] (sum x^2, sum kept^2) of this split's rows
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles_m = (int)((p.M + Cfg::BM - 1) / Cfg::BM);
     const int split = (int)cluster_ctarank(), tm = blockIdx.x / p.splits;  // cluster = the splits of a row block
-    (void)tiles_m;
     const int kblocks = (int)(p.K / Cfg::BK);
     const int kb0 = split * p.kb_per_split;
     const int kb1 = (kb0 + p.kb_per_split < kblocks) ? kb0 + p.kb_per_split : kblocks;
@@ -97,7 +101,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         *cta_abort = 0;
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full + 8 * s, 1);
-            mbar_init(bar_empty + 8 * s, 1 + Cfg::PRUNERS);  // the MMAs' commit + one arrive per prune warp
+            mbar_init(bar_empty + 8 * s, 1 + Cfg::TILES);  // the MMAs' commit + one arrive per tile's prune warp
         }
         mbar_init(bar_done, 1);
         fence_mbar_init();
@@ -141,7 +145,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer --------
         if (lane == 0) {
-            constexpr uint32_t idesc = make_idesc_bf16(Cfg::BM, R);
+            constexpr uint32_t idesc = make_idesc_bf16(128, R);
             const uint64_t d0 = make_desc_sw128(sX);
             const uint32_t desc_hi = (uint32_t)(d0 >> 32);
             const uint32_t a_lo0 = (uint32_t)d0, b_lo0 = (uint32_t)make_desc_sw128(sB);
@@ -171,19 +175,21 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         }
     } else if (warp >= 6) {
         // ------------------------------------------------------------------ prune warps -------
-        const int pw = warp - 6, r = lane >> 2, q = lane & 3;
+        const int pw = (warp - 6) % Cfg::TILES, turn = (warp - 6) / Cfg::TILES, r = lane >> 2, q = lane & 3;
         const int rowA_in = 16 * pw + r;                      // row inside the 128-row block; row B = + 8
         const int64_t rowA = (int64_t)tm * Cfg::BM + rowA_in, rowB = rowA + 8;
         const bool okA = rowA < p.M, okB = rowB < p.M;        // rows past M arrive as zeros (TMA fill)
         // this lane's 32 elements: box q / 2, chunks (q % 2) * 4 + 0..3 of the row's 128-byte line
         const uint32_t offA = (uint32_t)(q >> 1) * Cfg::X_BOX_BYTES + (uint32_t)rowA_in * 128;
         const uint32_t sw = (uint32_t)(r & 7), c0 = (uint32_t)(q & 1) * 4;
-        uint16_t* va = p.values + rowA * (p.K / 2) + (int64_t)kb0 * 64 + q * 16;
+        uint16_t* va = p.values + rowA * (p.K / 2) + (int64_t)(kb0 + turn) * 64 + q * 16;
         uint16_t* vb = va + 8 * (p.K / 2);
-        uint32_t* slab = reinterpret_cast<uint32_t*>(p.meta + ((int64_t)tm * kblocks + kb0) * 2048 + pw * 256 + lane * 4);
+        const int64_t row_block = (int64_t)tm * Cfg::BM / 128;  // metadata blocks have 128 rows
+        uint32_t* slab = reinterpret_cast<uint32_t*>(p.meta + (row_block * kblocks + kb0 + turn) * 2048 +
+                                                     (tm * Cfg::TILES % 8 + pw) * 256 + lane * 4);
         float numA = 0.f, denA = 0.f, numB = 0.f, denB = 0.f;
-        uint32_t stage = 0, phase = 0;
-        for (int kb = kb0; kb < kb1; ++kb) {
+        uint32_t stage = turn, phase = 0;
+        for (int kb = kb0 + turn; kb < kb1; kb += Cfg::TURNS) {
             if (!mbar_wait_warp(bar_full + 8 * stage, phase, cta_abort, p.dev_error)) break;
             const uint32_t base = sX + stage * Cfg::X_BYTES + offA;
             uint32_t a0[8], a1[8], b0[8], b1[8];
@@ -205,8 +211,9 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             TileOut out;
             prune_tile_core<SUMS>(a0, a1, b0, b1, lut, out, numA, denA, numB, denB);
             prune_tile_store(out, va, vb, slab, okA, okB);
-            va += 64; vb += 64; slab += 512;
-            if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            va += 64 * Cfg::TURNS; vb += 64 * Cfg::TURNS; slab += 512 * Cfg::TURNS;
+            stage += Cfg::TURNS;
+            if (stage >= STAGES) { stage -= STAGES; phase ^= 1; }
         }
         if constexpr (SUMS) {
 #pragma unroll
@@ -217,11 +224,11 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 denB += __shfl_xor_sync(0xffffffffu, denB, off);
             }
             if (q == 0) {
-                float* mine = p.scale_partial + (((int64_t)tm * 8 + pw) * p.splits + split) * 32;
+                float* mine = p.scale_partial + ((((int64_t)tm * Cfg::TILES + pw) * p.splits + split) * Cfg::TURNS + turn) * 32;
                 *reinterpret_cast<float2*>(mine + 2 * r) = make_float2(numA, denA);
                 *reinterpret_cast<float2*>(mine + 2 * (r + 8)) = make_float2(numB, denB);
-                sts64f(s_sums + rowA_in * 8, numA, denA);
-                sts64f(s_sums + (rowA_in + 8) * 8, numB, denB);
+                sts64f(s_sums + (turn * Cfg::BM + rowA_in) * 8, numA, denA);
+                sts64f(s_sums + (turn * Cfg::BM + rowA_in + 8) * 8, numB, denB);
             }
             __syncwarp();
         }
@@ -233,7 +240,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         const int q = warp & 3;  // tensor-memory lane quarter this warp may read
         const int r_in_tile = q * 32 + lane;
         const bool alive = mbar_wait_warp(bar_done, 0, cta_abort, p.dev_error);  // every MMA has retired: sB is free
-        if (alive) {
+        if (alive && q * 32 < Cfg::BM) {
             tc_fence_after();
             const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
@@ -243,7 +250,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                    sts128(sB + (uint32_t)(((c * 8 + j) * 128 + r_in_tile) * 16), v[4 * j], v[4 * j + 1], v[4 * j + 2],
+                    sts128(sB + (uint32_t)(((c * 8 + j) * Cfg::BM + r_in_tile) * 16), v[4 * j], v[4 * j + 1], v[4 * j + 2],
                            v[4 * j + 3]);
             }
         }
@@ -271,16 +278,19 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             const int r_t = row_first + r_l;
             const int64_t grow = (int64_t)tm * Cfg::BM + r_t;
             if (grow >= p.M) continue;
-            const uint32_t a0 = sB + (uint32_t)(((2 * piece) * 128 + r_t) * 16);
-            const uint32_t a1 = sB + (uint32_t)(((2 * piece + 1) * 128 + r_t) * 16);
+            const uint32_t a0 = sB + (uint32_t)(((2 * piece) * Cfg::BM + r_t) * 16);
+            const uint32_t a1 = sB + (uint32_t)(((2 * piece + 1) * Cfg::BM + r_t) * 16);
             float4 a[8], b[8];
-            float2 q[8];
+            float2 q[8][Cfg::TURNS];
 #pragma unroll
             for (int sp = 0; sp < 8; ++sp)  // every split's loads in flight together
                 if (sp < p.splits) {
                     a[sp] = lds128_cluster_f32(mapa(a0, (uint32_t)sp));
                     b[sp] = lds128_cluster_f32(mapa(a1, (uint32_t)sp));
-                    if constexpr (SUMS) q[sp] = lds64_cluster_f32(mapa(s_sums + r_t * 8, (uint32_t)sp));
+                    if constexpr (SUMS) {
+#pragma unroll
+                        for (int u = 0; u < Cfg::TURNS; ++u) q[sp][u] = lds64_cluster_f32(mapa(s_sums + (u * Cfg::BM + r_t) * 8, (uint32_t)sp));
+                    }
                 }
             float acc[8], num = 0.0f, den = 0.0f;
 #pragma unroll
@@ -291,7 +301,10 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                     acc[0] += a[sp].x; acc[1] += a[sp].y; acc[2] += a[sp].z; acc[3] += a[sp].w;
                     acc[4] += b[sp].x; acc[5] += b[sp].y; acc[6] += b[sp].z; acc[7] += b[sp].w;
                     // (up to eight partial sums in ascending order: the additions of row_scale_from_partials)
-                    if constexpr (SUMS) { num += q[sp].x; den += q[sp].y; }
+                    if constexpr (SUMS) {
+#pragma unroll
+                        for (int u = 0; u < Cfg::TURNS; ++u) { num += q[sp][u].x; den += q[sp][u].y; }
+                    }
                 }
             const float s = SUMS ? sqrtf(num / (den + 1e-8f)) : 1.0f;
             uint32_t o[4];

@@ -161,6 +161,35 @@ def test_prune_compress_lora_every_cluster_size(splits, K, monkeypatch):
         ctx.close()
 
 
+@pytest.mark.parametrize("R", [64, 128])
+@pytest.mark.parametrize("splits", [1, 2, 3, 4])
+@pytest.mark.parametrize("M", [390, 40])
+def test_prune_compress_lora_64_row_blocks(splits, R, M, lx, monkeypatch):
+    """Two groups of prune warps take the stages in turn (uneven splits of 14 K blocks: one group has a block more), the last
+    64-row block holds no row, and the layer's GEMM adds two partial sums per split and row."""
+    from paper_2605_26632_b200 import binding
+
+    monkeypatch.setenv("LYNX_PL_SPLITS", str(10 + splits))
+    ctx = binding.Lynx(0)
+    try:
+        K, N = 1792, 264
+        X, W, b, res, LA, LB = make_case(M, K, N, R, 92 + splits, with_res=True)
+        want_v, want_m, _ = lx.prune_compress(X.cuda(), 1)
+        for _ in range(3):
+            values, meta, T = ctx.prune_compress_lora(X.cuda(), LB.cuda(), 1)
+            assert torch.equal(values.view(torch.int16), want_v.view(torch.int16)) and torch.equal(meta, want_m)
+        ref = oracle_t(X, LB, 1)
+        got = T.float().cpu().numpy()
+        tol = 2.0 ** -8 * np.abs(ref) + 1e-5 * np.abs(ref).max()
+        assert (np.abs(got - ref) <= tol).all(), float(np.abs(got - ref).max())
+        ref = oracle.act_sparse_linear_lora(u16(X), u16(W), u16(LA), u16(LB), bias=u16(b), comp_mode=1, Yr=u16(res))
+        check_y(ctx.act_sparse_linear_lora(X.cuda(), W.cuda(), LA.cuda(), LB.cuda(), b.cuda(), 1, res.cuda()), ref["Y"])
+        torch.cuda.synchronize()
+        assert ctx.last_error() == 0
+    finally:
+        ctx.close()
+
+
 def test_prune_compress_lora_zero_rows_leading_dimensions_and_errors(lx):
     from paper_2605_26632_b200 import binding
 
