@@ -16,6 +16,13 @@
 // for its four rows; in the row-per-lane shape every lane needs every column's value, and those broadcast
 // loads alone occupied the shared memory for 1900 cycles per 512 x 240 item.  The blocks go to the
 // staging box with stmatrix.
+//
+// The next launch.  In low-rank and FP8 layer calls the single-tile kernel lets it begin (griddepcontrol.launch_dependents)
+// when its last tile's MMAs are done: what follows such a layer, in a chain of them, is a prune kernel with one block per SM,
+// whose prologue then runs as the SMs become free, under the last epilogues.  FP8 299 x 3840 x 3840 12.3 -> 11.8 us, 936 x 3072 x
+// 3072 13.4 -> 12.9; rank 64 299 x 3840 x 3840 21.6 -> 21.1, 936 x 3072 x 3072 22.2 -> 21.5.  Not in the two-row-tile kernel
+// (low-rank: no difference; FP8 4096 x 12288 x 3072 105.0 -> 106.2), and not in the plain layer: the small blocks of its prune kernel
+// pile up on the SMs that leave first (936 x 3072 x 3072 16.1 -> 17.0).
 #pragma once
 
 #include "ptx.cuh"

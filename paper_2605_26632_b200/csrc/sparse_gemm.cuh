@@ -799,6 +799,9 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 alive = mbar_wait_warp(bar_tfull + 8 * acc, turn.drain(), cta_abort, p.dev_error);
                 if (!alive) return;
                 tc_fence_after();
+                if constexpr (LORA || Cfg::FP8) {
+                    if (last && p.w_prefetch) griddep_launch_dependents();  // see epilogue.cuh
+                }
                 if (w.kind == 2) {
                     // wait until every contributing cluster's matching warp has published its rows
                     for (int cc = w.first_contrib; cc < cluster_id && alive; ++cc)
