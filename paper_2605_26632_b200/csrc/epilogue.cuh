@@ -110,7 +110,7 @@ __device__ __forceinline__ void epi_load_residual(const uint16_t* residual, int6
             const uint16_t* src = residual + row * ldr + n0 + 2 * (lane & 3);
 #pragma unroll
             for (int g = 0; g < CH / 8; ++g)
-                out[half][2 * g + k] = (row < M && n0 + 8 * g < N) ? __ldg(reinterpret_cast<const uint32_t*>(src + 8 * g)) : 0u;
+                out[half][2 * g + k] = (row < M && n0 + 8 * g < N) ? *reinterpret_cast<const uint32_t*>(src + 8 * g) : 0u;
         }
 }
 

@@ -138,8 +138,8 @@ prune_compress_fp8_kernel(const uint16_t* __restrict__ X, int64_t M, int64_t K, 
     }
     float amaxA = __uint_as_float(topA << 16), amaxB = __uint_as_float(topB << 16);
     if constexpr (GIVEN) {
-        amaxA = okA ? __ldg(row_amax + rowA) : 0.0f;
-        amaxB = okB ? __ldg(row_amax + rowB) : 0.0f;
+        amaxA = okA ? __ldcg(row_amax + rowA) : 0.0f;
+        amaxB = okB ? __ldcg(row_amax + rowB) : 0.0f;
     }
     const float invA = amaxA > 0.0f ? __fdiv_rn(448.0f, amaxA) : 0.0f;
     const float invB = amaxB > 0.0f ? __fdiv_rn(448.0f, amaxB) : 0.0f;
@@ -185,7 +185,7 @@ prune_compress_fp8_kernel(const uint16_t* __restrict__ X, int64_t M, int64_t K, 
         uint32_t top = 0;
 #pragma unroll
         for (int w = 0; w < FP8_PRUNE_WARPS; ++w) top = max(top, s_top[w][tid]);
-        float sc = __fdiv_rn(GIVEN ? __ldg(row_amax + row0 + tid) : __uint_as_float(top << 16), 448.0f);
+        float sc = __fdiv_rn(GIVEN ? __ldcg(row_amax + row0 + tid) : __uint_as_float(top << 16), 448.0f);
         if constexpr (SUMS) {
             float num = 0.f, den = 0.f;
 #pragma unroll
@@ -317,10 +317,10 @@ prune_compress_fp8_ring_kernel(const uint16_t* __restrict__ X, int64_t M, int64_
         uint32_t use = 0;
         // a supplied row maximum is fetched one row ahead: its latency hides behind the row's work
         float amax_next = 0.0f;
-        if (GIVEN && g < NG && g < count) amax_next = __ldg(row_amax + start + g);
+        if (GIVEN && g < NG && g < count) amax_next = __ldcg(row_amax + start + g);
         for (int i = g; g < NG && i < count; i += NG, ++it) {
             const float amax_given = amax_next;
-            if (GIVEN && i + NG < count) amax_next = __ldg(row_amax + start + i + NG);
+            if (GIVEN && i + NG < count) amax_next = __ldcg(row_amax + start + i + NG);
             const int slot = first + ls;
             bool ok = mbar_wait_warp(bar_full + 8 * slot, use & 1, cta_abort, dev_error);
             const uint32_t sbase = data + (uint32_t)slot * row_bytes;

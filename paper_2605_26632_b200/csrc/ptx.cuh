@@ -482,15 +482,18 @@ __device__ __forceinline__ uint64_t make_desc_rows16(uint32_t smem_addr) {
 
 // ---------------------------------------------------------------------------- memory ---------
 
+// Global loads of the kernels that may start while their predecessor still runs (griddep_wait) are plain ones, not ld.global.nc
+// or __ldg: those ask that the data be read-only for as long as the kernel lives, and here the kernel before may still be writing
+// it -- a layer's Y is the next layer's X, residual or bias -- when this one's CTAs are placed.
 __device__ __forceinline__ void ldg256_stream(const void* p, uint32_t (&r)[8]) {
-    asm volatile("ld.global.nc.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+    asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
                    "=r"(r[7])
                  : "l"(p));
 }
 // same 32-byte load with the default cache policy (the data is read again shortly)
 __device__ __forceinline__ void ldg256_keep(const void* p, uint32_t (&r)[8]) {
-    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
                    "=r"(r[7])
                  : "l"(p));

@@ -493,8 +493,8 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
             const uint32_t sb = sBias + (it & 1) * Cfg::BIAS_BYTES, sc = sb + BN * 4;
             if (const int c = (int)threadIdx.x - 32 * GEMM_EPI_WARP0; c < BN) {
                 const int n = tn * BN + c;
-                sts32f(sb + c * 4, (p.bias != nullptr && n < p.N) ? __uint_as_float((uint32_t)__ldg(p.bias + n) << 16) : 0.0f);
-                if constexpr (Cfg::FP8) sts32f(sc + c * 4, (p.col_scale != nullptr && n < p.N) ? __ldg(p.col_scale + n) : 1.0f);
+                sts32f(sb + c * 4, (p.bias != nullptr && n < p.N) ? __uint_as_float((uint32_t)p.bias[n] << 16) : 0.0f);
+                if constexpr (Cfg::FP8) sts32f(sc + c * 4, (p.col_scale != nullptr && n < p.N) ? p.col_scale[n] : 1.0f);
             }
             bar_sync_named(GEMM_EPI_BARRIER, 32 * Cfg::EPI_WARPS);  // every warp passes it once per item, whatever became of its waits
             if (!alive) continue;
@@ -508,7 +508,7 @@ sparse_gemm_rt2_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                 float sl = 1.0f;
                 if (r < rows && row < p.M) {
                     if (p.scale_partial != nullptr) sl = row_scale_from_partials(p.scale_partial, row, p.scale_ks);
-                    else if (p.row_scale != nullptr) sl = __ldg(p.row_scale + row);
+                    else if (p.row_scale != nullptr) sl = p.row_scale[row];
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) s[r][i] = __shfl_sync(0xffffffffu, sl, 8 * i + (lane >> 2));

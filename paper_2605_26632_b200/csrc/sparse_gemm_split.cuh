@@ -285,8 +285,8 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
         const uint32_t sc = sStrip + BN * 4;
         if (const int c = (int)threadIdx.x - 32 * GEMM_EPI_WARP0; c < BN) {
             const int n = tn * BN + c;
-            sts32f(sStrip + c * 4, (p.bias != nullptr && n < p.N) ? __uint_as_float((uint32_t)__ldg(p.bias + n) << 16) : 0.0f);
-            if constexpr (Cfg::FP8) sts32f(sc + c * 4, (p.col_scale != nullptr && n < p.N) ? __ldg(p.col_scale + n) : 1.0f);
+            sts32f(sStrip + c * 4, (p.bias != nullptr && n < p.N) ? __uint_as_float((uint32_t)p.bias[n] << 16) : 0.0f);
+            if constexpr (Cfg::FP8) sts32f(sc + c * 4, (p.col_scale != nullptr && n < p.N) ? p.col_scale[n] : 1.0f);
         }
         bar_sync_named(GEMM_EPI_BARRIER, 32 * GEMM_EPI_WARPS);
         // unit of row tile r: chunks [c0, c0 + n) of the accumulator; the odd chunk goes to the first warp of the quarter in the
@@ -310,7 +310,7 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
             float sl = 1.0f;
             if (row < p.M) {
                 if (p.scale_partial != nullptr) sl = row_scale_from_partials(p.scale_partial, row, p.scale_ks);
-                else if (p.row_scale != nullptr) sl = __ldg(p.row_scale + row);
+                else if (p.row_scale != nullptr) sl = p.row_scale[row];
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) s[i] = __shfl_sync(0xffffffffu, sl, 8 * i + (lane >> 2));
