@@ -120,30 +120,31 @@ def load_library() -> ctypes.CDLL:
 
 
 _calls = None
+_calls_failure = None
 
 
 def load_calls():
-    """The CPython extension that makes the per-layer calls (csrc/binding_calls.cpp), built first if its sources are newer.
-    Raises if it can be neither built nor loaded."""
-    global _calls
+    """The CPython extension that makes the per-layer calls (csrc/binding_calls.cpp), built first if there is none for these
+    sources, this interpreter and this torch.  Raises if it can be neither built nor loaded, then and whenever it is asked again."""
+    global _calls, _calls_failure
     if _calls is None:
-        load_library()
-        if _build.calls_are_stale():
-            try:
-                _build.build_calls()
-            except Exception:  # no compiler on this host
-                if not os.path.exists(_build.CALLS):
-                    raise
-        spec = importlib.util.spec_from_file_location(
-            "_lynx_calls", _build.CALLS, loader=importlib.machinery.ExtensionFileLoader("_lynx_calls", _build.CALLS))
-        module = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(module)
+        if _calls_failure is not None:
+            raise RuntimeError("_lynx_calls could not be loaded before") from _calls_failure
+        try:
+            load_library()
+            spec = importlib.util.spec_from_file_location(
+                "_lynx_calls", loader=importlib.machinery.ExtensionFileLoader("_lynx_calls", _build.build_calls()))
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
+        except Exception as e:
+            _calls_failure = e
+            raise
         _calls = module
     return _calls
 
 
 class _GeneralPathOnly:
-    """Stands in for the extension where it cannot be loaded (another torch than it was built for, no compiler): every call
+    """Stands in for the extension where it is not to be had (no compiler for a torch that it was not built for): every call
     takes the general path."""
 
     @staticmethod
@@ -151,6 +152,14 @@ class _GeneralPathOnly:
         return None
 
     layer_lora = layer_fp8 = prune = gemm = layer
+
+
+def _layer_calls():
+    try:
+        return load_calls()
+    except Exception as e:
+        warnings.warn(f"lynx: the binding's compiled calls are not available, layers cost more host time: {e}")
+        return _GeneralPathOnly
 
 
 def status_string(status: int) -> str:
@@ -273,11 +282,7 @@ class Lynx:
         _check(self._lib.lynx_create(ctypes.byref(h), device), "lynx_create")
         self._h = h
         self._address = h.value
-        try:
-            self._calls = load_calls()
-        except Exception as e:
-            warnings.warn(f"lynx: the binding's compiled calls are not available, layers cost more host time: {e}")
-            self._calls = _GeneralPathOnly
+        self._calls = _layer_calls()
 
     def close(self):
         if getattr(self, "_h", None):

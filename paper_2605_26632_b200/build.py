@@ -1,7 +1,9 @@
-"""Builds ``liblynx.so`` (the C-ABI CUDA library, nvcc for sm_100a) and ``_lynx_calls.so`` (the binding's per-layer calls,
-a CPython extension on top of it) in-tree."""
+"""Builds ``liblynx.so`` (the C-ABI CUDA library, nvcc for sm_100a) and ``_lynx_calls.<tag>.so`` (the binding's per-layer
+calls, a CPython extension on top of it) in-tree."""
 from __future__ import annotations
 
+import glob
+import hashlib
 import os
 import subprocess
 import sys
@@ -11,7 +13,6 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblynx.so")
-CALLS = os.path.join(HERE, "_lynx_calls.so")
 HEADER = os.path.join(ROOT, "include", "lynx.h")
 SOURCES = [os.path.join(CSRC, "lynx_api.cu")]
 CALLS_SOURCES = [os.path.join(CSRC, "binding_calls.cpp")]
@@ -30,8 +31,16 @@ def is_stale() -> bool:
     return _older(LIB, DEPS)
 
 
-def calls_are_stale() -> bool:
-    return _older(CALLS, CALLS_DEPS)
+def calls_path() -> str:
+    """The extension's file.  It inlines the layouts of CPython's and torch's objects and the library's C ABI, and a build for
+    others may load and read wrong fields: its name says what it was built for, and no other file is ever loaded."""
+    import torch
+
+    h = hashlib.sha256(f"{torch.version.git_version} {int(torch._C._GLIBCXX_USE_CXX11_ABI)}".encode())
+    for f in CALLS_DEPS:
+        with open(f, "rb") as src:
+            h.update(src.read())
+    return os.path.join(HERE, f"_lynx_calls.{sysconfig.get_config_var('SOABI')}.torch-{torch.__version__}.{h.hexdigest()[:12]}.so")
 
 
 def _nvcc() -> str:
@@ -61,23 +70,27 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 def build_calls(force: bool = False, verbose: bool = False) -> str:
-    """Needs liblynx.so, and torch's headers and libraries as installed."""
-    if not force and not calls_are_stale():
-        return CALLS
+    """Needs liblynx.so, and torch's headers and libraries as installed.  -> calls_path()"""
+    path = calls_path()
+    if not force and os.path.exists(path):
+        return path
     import torch
 
     torch_dir = os.path.dirname(os.path.abspath(torch.__file__))
     cuda_include = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")
-    tmp = CALLS + f".tmp{os.getpid()}"
+    tmp = path + f".tmp{os.getpid()}"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-shared",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            "-I" + sysconfig.get_paths()["include"], "-isystem", os.path.join(torch_dir, "include"),
            "-isystem", os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"), "-isystem", cuda_include]
     cmd += CALLS_SOURCES + ["-o", tmp, "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10",
                             "-lc10_cuda", "-L" + HERE, "-l:liblynx.so", "-Wl,-rpath,$ORIGIN"]
-    _run(cmd, CALLS, verbose)
-    os.replace(tmp, CALLS)
-    return CALLS
+    _run(cmd, path, verbose)
+    os.replace(tmp, path)
+    for old in glob.glob(glob.escape(path.rsplit(".", 2)[0]) + ".*.so"):  # of other sources
+        if old != path:
+            os.remove(old)
+    return path
 
 
 if __name__ == "__main__":

@@ -35,6 +35,37 @@ def test_size_helpers():
     assert lib.lynx_workspace_bytes(256, 512, 512) >= 256 * 256 * 2 + 2 * 4 * 2048 + 256 * 4
 
 
+def test_compiled_calls_for_another_torch_or_other_sources_are_not_loaded(monkeypatch, tmp_path):
+    """The extension reads tensors through inlined layouts: only a build for this interpreter, torch and header may be loaded.
+    Where it cannot be made the layers take the general path, and the compiler is not run again for every context."""
+    from paper_2605_26632_b200 import binding, build
+
+    assert binding.load_calls() is binding._layer_calls() and os.path.samefile(binding.load_calls().__file__, build.calls_path())
+    header = tmp_path / "lynx.h"
+    header.write_text(open(build.HEADER).read() + "\n")
+    for target, name, value in ((torch, "__version__", "0.0+other"), (torch.version, "git_version", "other"),
+                                (build, "CALLS_DEPS", build.CALLS_SOURCES + [str(header)])):
+        tried = []
+
+        def no_compiler(cmd, path, verbose):
+            tried.append(path)
+            raise RuntimeError("no compiler")
+
+        with monkeypatch.context() as mp:
+            here = build.calls_path()
+            mp.setattr(target, name, value)
+            mp.setattr(build, "_run", no_compiler)
+            mp.setattr(binding, "_calls", None)
+            mp.setattr(binding, "_calls_failure", None)
+            assert build.calls_path() != here
+            for _ in range(2):
+                with pytest.raises(RuntimeError):
+                    binding.load_calls()
+                with pytest.warns(UserWarning, match="compiled calls"):
+                    assert binding._layer_calls() is binding._GeneralPathOnly
+            assert tried == [build.calls_path()]
+
+
 def test_no_accumulator_hand_back_is_outstanding_when_the_gemm_ends():
     """The MMA issuer's waits, against barriers that complete a phase per hand-back and an epilogue that hands back as
     late as it can: no buffer is filled before its contents were handed back, and when the issuer is through
