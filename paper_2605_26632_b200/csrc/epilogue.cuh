@@ -17,12 +17,14 @@
 // loads alone occupied the shared memory for 1900 cycles per 512 x 240 item.  The blocks go to the
 // staging box with stmatrix.
 //
-// The next launch.  In low-rank and FP8 layer calls the single-tile kernel lets it begin (griddepcontrol.launch_dependents)
-// when its last tile's MMAs are done: what follows such a layer, in a chain of them, is a prune kernel with one block per SM,
-// whose prologue then runs as the SMs become free, under the last epilogues.  FP8 299 x 3840 x 3840 12.3 -> 11.8 us, 936 x 3072 x
-// 3072 13.4 -> 12.9; rank 64 299 x 3840 x 3840 21.6 -> 21.1, 936 x 3072 x 3072 22.2 -> 21.5.  Not in the two-row-tile kernel
-// (low-rank: no difference; FP8 4096 x 12288 x 3072 105.0 -> 106.2), and not in the plain layer: the small blocks of its prune kernel
-// pile up on the SMs that leave first (936 x 3072 x 3072 16.1 -> 17.0).
+// The next launch.  The single-tile kernel lets it begin (griddepcontrol.launch_dependents) when its last tile's MMAs are done, in
+// the layer calls whose own prune kernel has one block per SM: what follows, in a chain of them, is such a kernel, and its
+// prologue then runs as the SMs become free, under the last epilogues.  These are the low-rank layers (rank 64: 299 x 3840 x 3840
+// 21.6 -> 21.1 us, 936 x 3072 x 3072 22.2 -> 21.5) and FP8 layers of K >= 2048 (299 x 2048 x 3840 10.3 -> 9.8, 936 x 2816 x
+// 3072 13.2 -> 12.7, 936 x 2304 x 9216 19.4 -> 18.9).  Shorter FP8 rows are pruned in blocks of 16 rows, which, like the small
+// blocks of the plain layer's prune kernel, pile up on the SMs that leave first: 936 x 1792 x 3072 12.1 -> 14.2, 600 x 1024 x 3072
+// 9.1 -> 10.1, 4352 x 1536 x 3072 22.7 -> 23.7, plain 936 x 3072 x 3072 16.1 -> 17.0.  Nor is it used in the two-row-tile kernel
+// (low-rank: no difference; FP8 4096 x 12288 x 3072 105.0 -> 106.2).
 #pragma once
 
 #include "ptx.cuh"

@@ -420,6 +420,7 @@ lynx_status launch_gemm_cfg(lynx_ctx* ctx, const void* values, const void* meta,
     p.T = nullptr;
     p.ldt = 0;
     p.w_prefetch = (layer_call && !ctx->streamk) ? 1 : 0;
+    p.trigger = p.w_prefetch;  // read by the low-rank kernels: their layers' prune launch has a block per SM
 
     auto kern = lora ? sparse_gemm_kernel<Cfg, true> : sparse_gemm_kernel<Cfg, false>;
     static bool attr_set[2][MAX_CTX_DEVICES] = {};  // per instantiation (with / without the low-rank code)
@@ -809,6 +810,14 @@ lynx_status launch_gemm(lynx_ctx* ctx, const void* values, const void* meta, int
 #undef LYNX_GEMM_ARGS
 }
 
+// Rows of X that the persistent ring form of the FP8 prune kernel (a block per SM, X read once) keeps in shared memory; 0 where
+// the one with a block per 16 rows is launched: the ring wants at least two rows, and rows long enough to occupy a warp.
+int fp8_ring_slots(int64_t K) {
+    const int64_t slots = (FP8_RING_SMEM_MAX - FP8_RING_HEADER) / (K * 2);
+    if (slots < 2 || K < 2048) return 0;
+    return slots > FP8_RING_MAX_SLOTS ? FP8_RING_MAX_SLOTS : (int)slots;
+}
+
 // FP8 (E4M3) instantiation: byte tensor maps, K blocks of 256, optional per-channel weight scale.
 template <class Cfg>
 lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void* meta, int64_t M, int64_t K,
@@ -839,6 +848,7 @@ lynx_status launch_gemm_fp8_cfg(lynx_ctx* ctx, const void* values_q, const void*
     p.group_m = gemm_group_rows(ctx, p.tiles_m);
     p.l0_splits = 1;
     p.w_prefetch = layer_call ? 1 : 0;
+    p.trigger = layer_call && ctx->fp8_ring && fp8_ring_slots(K) ? 1 : 0;
     auto kern = sparse_gemm_kernel<Cfg, false>;
     static bool attr_set[MAX_CTX_DEVICES] = {};  // per instantiation
     if (lynx_status as = prepare_gemm_kernel(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
@@ -1835,11 +1845,7 @@ lynx_status lynx_prune_compress_fp8(lynx_ctx* ctx, const void* X, int64_t M, int
     uint8_t* vp = static_cast<uint8_t*>(values_q);
     uint8_t* mp = static_cast<uint8_t*>(meta);
     cudaError_t e;
-    // The persistent ring kernel reads X once (also when the maxima have to be found in the data).
-    // It wants at least two rows in shared memory and rows long enough to occupy a warp.
-    int slots = (int)((FP8_RING_SMEM_MAX - FP8_RING_HEADER) / (K * 2));
-    if (slots > FP8_RING_MAX_SLOTS) slots = FP8_RING_MAX_SLOTS;
-    if (ctx->fp8_ring && slots >= 2 && K >= 2048) {
+    if (const int slots = ctx->fp8_ring ? fp8_ring_slots(K) : 0) {
         // gw warps share a row; ng = CW / gw groups, each with at least one slot of its own
         int gw = fp8_ring_group_width(slots);
         if (ctx->fp8_ring_forced && (ctx->fp8_ring == 1 || ctx->fp8_ring == 2 || ctx->fp8_ring == 4 || ctx->fp8_ring == 8))
@@ -2005,6 +2011,8 @@ int lynx_gemm_split_plan(int fp8, int64_t M, int64_t N, int64_t K, int lora_step
     if (splits) *splits = plan.splits;
     return plan.id;
 }
+
+int lynx_gemm_fp8_begins_next(int64_t K) { return K < 256 || K % 256 ? -1 : fp8_ring_slots(K) ? 1 : 0; }
 
 int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K) {
     if (num_sms < 2 || M < 1 || N < 8 || K < 256) return -1;

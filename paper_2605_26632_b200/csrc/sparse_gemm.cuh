@@ -86,6 +86,7 @@ struct GemmParams {
     // launch), so the W tiles of the first ring stages may be fetched before the wait for that
     // kernel; the direct GEMM entry points leave this 0 (whatever precedes them might write W).
     int w_prefetch;
+    int trigger;  // the next kernel's CTAs may be placed when a CTA's last tile's MMAs are done (see epilogue.cuh)
 };
 
 // Work distribution over C persistent clusters.  The first floor(T/C)*C tiles go round-robin,
@@ -800,7 +801,7 @@ sparse_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_cons
                 if (!alive) return;
                 tc_fence_after();
                 if constexpr (LORA || Cfg::FP8) {
-                    if (last && p.w_prefetch) griddep_launch_dependents();  // see epilogue.cuh
+                    if (last && p.trigger) griddep_launch_dependents();
                 }
                 if (w.kind == 2) {
                     // wait until every contributing cluster's matching warp has published its rows

@@ -66,6 +66,15 @@ def test_compiled_calls_for_another_torch_or_other_sources_are_not_loaded(monkey
             assert tried == [build.calls_path()]
 
 
+def test_fp8_layers_let_the_next_launch_begin_only_where_their_prune_kernel_has_a_block_per_sm():
+    """That kernel keeps whole rows in shared memory: at least two of them, 2048 elements or longer."""
+    from paper_2605_26632_b200 import binding
+
+    begins = binding.load_library().lynx_gemm_fp8_begins_next
+    assert [begins(k) for k in (256, 1024, 1792, 2048, 2304, 12288, 57600, 57856, 65536)] == [0, 0, 0, 1, 1, 1, 1, 0, 0]
+    assert begins(0) == -1 and begins(300) == -1
+
+
 def test_no_accumulator_hand_back_is_outstanding_when_the_gemm_ends():
     """The MMA issuer's waits, against barriers that complete a phase per hand-back and an epilogue that hands back as
     late as it can: no buffer is filled before its contents were handed back, and when the issuer is through
