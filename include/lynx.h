@@ -344,6 +344,7 @@ LYNX_API lynx_status lynx_selftest_wait_timeout(lynx_ctx* ctx, int64_t limit_us,
  * lynx_gemm_plan returns 1 when, for an (M, N, K) product on a GPU with num_sms SMs, the kernel
  * that runs two 256-row tiles per W stage is chosen (its number of 512-row items and of CTA pairs
  * in *doubles / *clusters), 0 when the single-tile kernel is, -1 on bad arguments.
+ * lynx_gemm_fp8_plan returns the same of an FP8 product.
  * lynx_gemm_split_plan goes before both: for a product of few tiles on a GPU of 148 SMs it returns the tile of the
  * kernel that splits K over the members of a cluster (1: 256 x 128 per CTA pair, 2: 256 x 192, 5: 128 x 128 per CTA;
  * the number of members in *splits), 0 when K is not split, -1 on bad arguments.
@@ -368,6 +369,7 @@ LYNX_API int lynx_gemm_schedule_items(int tiles_m, int tiles_n, int clusters, in
                                       int* items, int capacity);
 LYNX_API int lynx_gemm_split_plan(int fp8, int64_t M, int64_t N, int64_t K, int lora_steps, int* splits);
 LYNX_API int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K);
+LYNX_API int lynx_gemm_fp8_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* doubles, int* clusters);
 LYNX_API int lynx_gemm_fp8_begins_next(int64_t K);
 LYNX_API int lynx_gemm_phase0_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* splits, int* fill);
 LYNX_API int lynx_gemm_register_shares_fit(int regs_per_thread);

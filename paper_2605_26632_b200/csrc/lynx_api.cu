@@ -491,10 +491,8 @@ using Rt2CfgFp8 = Gemm2Cfg<240, 3, true>;
 // stores of 122 KB per CTA slow the next item's first loads).  4352 x 3072 x 3072: one double + one single per
 // cluster 34.9 us, three singles 36.2; 4096 x 3072 x 12288: doubles 121.7, singles 127.1.  Within each class of
 // clusters the one at the first position carries the most singles, so two clusters decide the maximum.
-// FP8 (256-element K blocks): fits to whole layers of 19 shapes at the clocks that calls back to back settle at, single-tile
-// kernel -> two row tiles: 16384 x 12288 x 3072 410 -> 390 us, 4352 x 3072 x 9216 81.5 -> 78.5, 1337 x 3840 x 10240 42.0 -> 40.2,
-// 4096 x 12288 x 3072 104.1 -> 103.7; up to K = 2048 the exposed epilogues cost more than the bytes saved give
-// (8192 x 2048 x 8192 98.5 against 102.4).
+// FP8 (256-element K blocks): fits to whole layers of 19 shapes at the clocks that calls back to back settle at; where they
+// are compared with the single tiles see fp8_rt2_if_faster.
 struct Rt2Cost {
     double t1, t2, e1, e2;
 };
@@ -617,6 +615,18 @@ double gemm_model_time(int num_sms, int64_t M, int64_t N, int64_t K, int lora_st
     double t = 0.0;
     pick_gemm_cfg_model(num_sms, M, N, K, lora_steps, &t);
     return t;
+}
+// The FP8 two-row-tile plan of a product if it is modelled faster than the best single tile.  The fits of FP8_TILES rank single
+// tiles; beside the two-row-tile times the 192-wide one's are too long, so against it the model has to promise 13 %.  Whole layers of
+// 270 shapes (K 1792 ... 15360), both kernels in turn in blocks of 150 ms: where 240 is the best single tile (208) two row tiles
+// take 2.9 % less on average (1792 x 8192 x 8880 -8.1 %, 2560 x 16384 x 12288 -5.6, 3072 x 4352 x 9216 -2.1, K x M x N; launches
+// of one round +-3), where 192 is (62) 3.1 % more (2048 x 16384 x 9216 +8.0 %, 3072 x 2994 x 9216 +10.0, 4864 x 1401 x 3160 +12.6) up to
+// a modelled gain of 12 %, and 2.1 % less from 13 % on (13824 x 270 x 12744 -6.0).
+constexpr double RT2_FP8_OVER_192 = 1.13;
+bool fp8_rt2_if_faster(int num_sms, int64_t M, int64_t N, int64_t K, const Rt2Plan& plan) {
+    double t = 0.0;
+    const TileCost& tile = pick_tile(FP8_TILES, num_sms, M, N, (double)(K / 256), &t);
+    return plan.t_us * (tile.bn == 192 ? RT2_FP8_OVER_192 : 1.0) < t;
 }
 int pick_gemm_cfg(const lynx_ctx* ctx, int64_t M, int64_t N, int64_t K, int lora_steps) {
     if (ctx->gemm_cfg != 0) return ctx->gemm_cfg;
@@ -887,9 +897,7 @@ lynx_status launch_gemm_fp8(lynx_ctx* ctx, const void* values_q, const void* met
     if (ctx->gemm_cfg == 0 && ctx->rt2 != 0 && M > 256) {
         // the two-row-tile kernel where its schedule is modelled faster than the best plain tile
         const Rt2Plan plan = rt2_plan(RT2_FP8, ctx->num_sms, M, N, (double)(K / 256), ctx->rt2_doubles);
-        double t = 0.0;
-        pick_tile(FP8_TILES, ctx->num_sms, M, N, (double)(K / 256), &t);
-        if (ctx->rt2 == 1 || plan.t_us < t)
+        if (ctx->rt2 == 1 || fp8_rt2_if_faster(ctx->num_sms, M, N, K, plan))
             return launch_gemm_rt2<Rt2CfgFp8, false>(ctx, plan, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, nullptr, Y, ldy, st,
                                                      nullptr, layer_call);
     }
@@ -2010,6 +2018,14 @@ int lynx_gemm_split_plan(int fp8, int64_t M, int64_t N, int64_t K, int lora_step
                                : split_plan_if_faster<false>(CLUSTER_CAP_148, 148, M, N, K, lora_steps);
     if (splits) *splits = plan.splits;
     return plan.id;
+}
+
+int lynx_gemm_fp8_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* doubles, int* clusters) {
+    if (num_sms < 2 || M < 1 || N < 8 || K < 256) return -1;
+    const Rt2Plan plan = rt2_plan(RT2_FP8, num_sms, M, N, (double)(K / 256), -1);
+    if (doubles) *doubles = plan.doubles;
+    if (clusters) *clusters = plan.clusters;
+    return (M > 256 && fp8_rt2_if_faster(num_sms, M, N, K, plan)) ? 1 : 0;
 }
 
 int lynx_gemm_fp8_begins_next(int64_t K) { return K < 256 || K % 256 ? -1 : fp8_ring_slots(K) ? 1 : 0; }

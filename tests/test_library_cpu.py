@@ -66,6 +66,17 @@ def test_compiled_calls_for_another_torch_or_other_sources_are_not_loaded(monkey
             assert tried == [build.calls_path()]
 
 
+def test_fp8_two_row_tiles_are_planned_where_they_were_measured_faster():
+    """(M, N, K) of layers timed with both kernels: two row tiles per W stage faster, or a single tile (192 wide) by 6 % and more."""
+    from paper_2605_26632_b200 import binding
+
+    plan = lambda m, n, k: binding.load_library().lynx_gemm_fp8_plan(148, m, n, k, None, None)
+    for shape in [(4096, 3072, 12288), (16384, 3072, 12288), (4352, 9216, 3072), (8192, 8880, 1792), (1393, 10240, 3840), (270, 12744, 13824)]:
+        assert plan(*shape) == 1, shape
+    for shape in [(2994, 9216, 3072), (16384, 9216, 2048), (8192, 12288, 2304), (8321, 3840, 3840), (15102, 3072, 3072), (1401, 3160, 4864)]:
+        assert plan(*shape) == 0, shape
+
+
 def test_fp8_layers_let_the_next_launch_begin_only_where_their_prune_kernel_has_a_block_per_sm():
     """That kernel keeps whole rows in shared memory: at least two of them, 2048 elements or longer."""
     from paper_2605_26632_b200 import binding
