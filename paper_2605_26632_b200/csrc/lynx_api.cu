@@ -634,6 +634,11 @@ int pick_gemm_cfg(const lynx_ctx* ctx, int64_t M, int64_t N, int64_t K, int lora
 }
 // ------------------------------------------------------- K split over a cluster (sparse_gemm_split) -----
 
+// With a quarter of the SMs free the next kernel's CTAs (a prune launch's are small) start there and run their
+// prologue: 256 x 3072 x 3072 layer 10.1 -> 9.8 us.  With fewer they pile up on the few that are: 128 x 3072 x 9216
+// (144 SMs) 16.2 -> 17.6.
+bool split_begins_next(int64_t ctas, int num_sms) { return ctas * 4 <= (int64_t)num_sms * 3; }
+
 template <class Cfg, bool LORA>
 lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, const void* values, const void* meta, int64_t M, int64_t K, const void* W,
                               int64_t N, int64_t ldw, const float* wscale, const void* bias, const lynx_comp* comp,
@@ -682,10 +687,7 @@ lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, const void* values, con
     if (lynx_status as = prepare_gemm_kernel(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
     cudaLaunchConfig_t cfg = {};
     const int grid = p.tiles_m * tiles_n * splits * Cfg::CG;
-    // With a quarter of the SMs free the next kernel's CTAs (a prune launch's are small) start there and run their
-    // prologue: 256 x 3072 x 3072 layer 10.1 -> 9.8 us.  With fewer they pile up on the few that are: 128 x 3072 x 9216
-    // (144 SMs) 16.2 -> 17.6.
-    p.trigger = grid * 4 <= ctx->num_sms * 3 ? 1 : 0;
+    p.trigger = split_begins_next(grid, ctx->num_sms) ? 1 : 0;
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(Cfg::THREADS);
     cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
@@ -726,6 +728,7 @@ constexpr int64_t SPLIT_MAX_ROWS = 2048;
 struct SplitPlan {
     int id = 0, splits = 1;
     double t_us = 1e30;
+    int64_t ctas = 0;
 };
 template <bool FP8>
 SplitPlan split_plan(const int (&cap)[9], int64_t M, int64_t N, int64_t K, int lora_steps) {
@@ -737,7 +740,7 @@ SplitPlan split_plan(const int (&cap)[9], int64_t M, int64_t N, int64_t K, int l
         for (int s = 2; s * c.cg <= 8 && s <= kb; ++s) {
             if (tiles * s * c.cg > cap[s * c.cg]) continue;
             const double t = (double)((kb + s - 1) / s + lora_steps) * c.t_kb + c.fix + 0.3 * c.cg * (s - 2);
-            if (t < best.t_us) best = SplitPlan{c.id, s, t};
+            if (t < best.t_us) best = SplitPlan{c.id, s, t, tiles * s * c.cg};
         }
     }
     return best;
@@ -766,19 +769,31 @@ lynx_status launch_gemm_split_id(lynx_ctx* ctx, const SplitPlan& plan, const voi
     }
 }
 
-// The split plan of a product if it is modelled faster than the other kernels, id 0 if not.
+// The split plan of a product if it is modelled faster than the best single tile (two row tiles never are, where it is), id 0 if not.
+// The model has to promise `least`: what its figures make too good of some forms, measured on 285 layers with both kernels in turn.
+// Two and three splits of single CTAs, pairs of 192 columns: up to there the layers were slower (1498 x 2304 x 256 10.9 -> 11.3 us, 1051 x
+// 2560 x 512 11.2 -> 11.9, 169 x 4608 x 5520 17.0 -> 17.5; FP8 in three splits 280 x 4608 x 1904 11.9 -> 12.6), while four splits and
+// pairs of 128 columns gain from the first tenth on (495 x 2048 x 416 9.7 -> 9.2, 209 x 2304 x 3656 10.1 -> 9.8).  Low-rank: the
+// single-tile kernel lets the next launch begin behind its last MMAs, which splits that hold most of the SMs do not (206 x 3072 x 4320
+// 15.9 -> 17.3, 374 x 3072 x 3072 16.0 -> 17.9, 696 x 3072 x 624 15.7 -> 16.6); the others let it at their start (692 x 2560 x 480
+// 15.1 -> 15.7).
+double split_least(bool fp8, const SplitPlan& plan, int num_sms, int lora_steps) {
+    if (lora_steps) return split_begins_next(plan.ctas, num_sms) ? 1.2 : 2.0;
+    if (fp8) return plan.id == 5 && plan.splits == 3 ? 0.9 : 0.0;
+    return (plan.id == 5 && plan.splits <= 3) || plan.id == 2 ? 0.9 : 0.0;
+}
 template <bool FP8>
 SplitPlan split_plan_if_faster(const int (&cap)[9], int num_sms, int64_t M, int64_t N, int64_t K, int lora_steps) {
     const SplitPlan plan = split_plan<FP8>(cap, M, N, K, lora_steps);
     double t = 0.0;
     if (FP8) pick_tile(FP8_TILES, num_sms, M, N, (double)(K / 256), &t);
     else t = gemm_model_time(num_sms, M, N, K, lora_steps);
-    return plan.t_us < t ? plan : SplitPlan{};
+    return plan.t_us + split_least(FP8, plan, num_sms, lora_steps) < t ? plan : SplitPlan{};
 }
 template <bool FP8>
 SplitPlan choose_split(const lynx_ctx* ctx, int64_t M, int64_t N, int64_t K, int lora_steps) {
     if (ctx->split == 0) return SplitPlan{};
-    if (ctx->split > 0) return SplitPlan{ctx->split / 10, ctx->split % 10, 0.0};
+    if (ctx->split > 0) return SplitPlan{ctx->split / 10, ctx->split % 10, 0.0, 0};
     return split_plan_if_faster<FP8>(ctx->cluster_cap, ctx->num_sms, M, N, K, lora_steps);
 }
 

@@ -331,6 +331,27 @@ def test_bench_launches_its_own_ranks_when_started_plainly():
     assert abs(d["aggregate_tflops"] - 1e12 * 10 * 2 / 15e-3 / 1e12) < 1e-6
 
 
+def test_split_plan_is_not_chosen_where_it_was_measured_slower():
+    """(M, N, K, low-rank steps) of layers timed with and without the split; where it is chosen no two-row-tile plan is."""
+    import random
+
+    from paper_2605_26632_b200 import binding
+
+    for m, n, k, lora in [(1498, 256, 2304, 0), (169, 5520, 4608, 0), (774, 1104, 3328, 0), (206, 4320, 3072, 1), (266, 3072, 3072, 1),
+                          (384, 3072, 3072, 2), (1274, 464, 2560, 2), (692, 480, 2560, 2), (696, 624, 3072, 1)]:
+        assert binding.gemm_split_plan(False, m, n, k, lora) == (0, 1), (m, n, k, lora)
+    for m, n, k, lora in [(256, 3072, 3072, 0), (64, 3072, 3072, 0), (429, 280, 2560, 0), (495, 416, 2048, 0), (209, 3656, 2304, 0), (131, 3072, 3072, 1),
+                          (167, 3072, 3072, 2), (472, 3072, 12288, 1), (80, 3840, 3840, 1)]:
+        assert binding.gemm_split_plan(False, m, n, k, lora)[0] > 0, (m, n, k, lora)
+    assert binding.gemm_split_plan(True, 280, 1904, 4608) == binding.gemm_split_plan(True, 606, 1144, 5376) == (0, 1)
+    assert binding.gemm_split_plan(True, 1858, 376, 4864)[0] > 0 and binding.gemm_split_plan(True, 76, 5744, 6144)[0] > 0
+    rng = random.Random(7)
+    for _ in range(5000):
+        m, k, n, lora = rng.randint(1, 2047), 128 * rng.randint(1, 128), 8 * rng.randint(1, 2688), rng.choice([0, 0, 1, 2])
+        if binding.gemm_split_plan(False, m, n, k, lora)[0]:
+            assert not binding.gemm_plan(148, m, n, k, lora)[0], (m, n, k, lora)
+
+
 def test_split_plan_is_one_round_and_has_a_k_block_for_every_member():
     import random
 
