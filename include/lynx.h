@@ -185,6 +185,10 @@ LYNX_API lynx_status lynx_prune_compress_static(const void* X, int64_t M, int64_
  * where X~ is the matrix (values, meta) encodes, the sum is accumulated in fp32 on the sparse
  * tensor cores, and absent terms (bias == NULL, comp == NULL or its members NULL) are 1 / 0.
  * values / meta must have the layout lynx_prune_compress writes.
+ * The order in which an element's products are added depends on the whole shape (M, N, K, operand type, low-rank branch
+ * or none) and on the GPU: products of few tiles below 2048 rows split K over the CTAs of a thread-block cluster and add
+ * their fp32 partial sums in a fixed order.  Calls of one shape on one GPU repeat bit for bit, but a token row may
+ * differ in its last bits between batches of different sizes.  This holds for every sparse product below.
  */
 LYNX_API lynx_status lynx_sparse_linear(lynx_ctx* ctx, const void* values, const void* meta,
                                         int64_t M, int64_t K, const void* W, int64_t N, int64_t ldw,
@@ -199,7 +203,7 @@ LYNX_API lynx_status lynx_sparse_linear(lynx_ctx* ctx, const void* values, const
  * launch leaves the per-K-split row sums in the scratch and the GEMM's epilogue forms s_m from
  * them, adding in the order lynx_prune_compress itself uses: Y is bit-identical to calling
  * lynx_prune_compress and lynx_sparse_linear one after the other, without the scale hand-over
- * inside the first kernel.
+ * inside the first kernel.  (The order of the product's own additions: see lynx_sparse_linear.)
  */
 LYNX_API lynx_status lynx_act_sparse_linear(lynx_ctx* ctx, const void* X, int64_t M, int64_t K,
                                             int64_t ldx, const void* W, int64_t N, int64_t ldw,
