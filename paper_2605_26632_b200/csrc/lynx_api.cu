@@ -676,7 +676,7 @@ lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, const void* values, con
     p.residual = comp ? static_cast<const uint16_t*>(comp->residual) : nullptr;
     p.ldr = comp ? comp->ldr : 0;
     p.dev_error = ctx->err_dev;
-    constexpr int rows = Cfg::R * Cfg::CG * Cfg::BM;
+    constexpr int rows = Cfg::CG * Cfg::BM;
     p.tiles_m = (int)((M + rows - 1) / rows);
     p.splits = splits;
     p.lora_steps = LORA ? lora->R / 64 : 0;
@@ -762,9 +762,9 @@ lynx_status launch_gemm_split_id(lynx_ctx* ctx, const SplitPlan& plan, const voi
 #undef LYNX_SPLIT_ARGS
     };
     switch (plan.id) {
-        case 1: return go(SplitCfg<1, 128, 2, 5, FP8>{});
-        case 2: return go(SplitCfg<1, 192, 2, FP8 ? 4 : 5, FP8>{});
-        case 5: return go(SplitCfg<1, 128, 1, 4, FP8>{});
+        case 1: return go(SplitCfg<128, 2, 5, FP8>{});
+        case 2: return go(SplitCfg<192, 2, FP8 ? 4 : 5, FP8>{});
+        case 5: return go(SplitCfg<128, 1, 4, FP8>{});
         default: return LYNX_ERR_INVALID_ARG;
     }
 }
@@ -1207,8 +1207,8 @@ lynx_status lynx_create(lynx_ctx** out, int device) {
     }
     {
         // how many CTAs, one per SM, of clusters of 1..8 the GPU holds at once
-        auto kern = sparse_gemm_split_kernel<SplitCfg<1, 128, 2, 5>, false>;
-        constexpr int smem = SplitCfg<1, 128, 2, 5>::SMEM_BYTES;
+        auto kern = sparse_gemm_split_kernel<SplitCfg<128, 2, 5>, false>;
+        constexpr int smem = SplitCfg<128, 2, 5>::SMEM_BYTES;
         const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
         for (int i = 1; i <= 8 && ok; ++i) {
             cudaLaunchConfig_t qc = {};

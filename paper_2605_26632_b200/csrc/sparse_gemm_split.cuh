@@ -13,14 +13,14 @@
 // of the 192-wide one).
 //
 // One tile per cluster, not persistent.  Roles per CTA as in sparse_gemm_kernel: warp 0 TMA producer, warp 1 MMA issuer (of
-// a CTA pair's leader), warps 4..11 epilogue.  R = 2: two row tiles per W stage, as in sparse_gemm_rt2_kernel.
+// a CTA pair's leader), warps 4..11 epilogue.
 //
-// The exchange.  The accumulators of a CTA are R x 8 units, one per (row tile, epilogue warp): the 32 rows of the
-// warp's tensor-memory quarter x its share of the columns.  Unit u belongs to split u * splits / (8 R).  When
-// every member's MMAs are done (first cluster barrier: the rings are free) each warp copies the units that are not its
-// split's, in the register layout of the tensor-memory loads, to the owners' rings (512 contiguous bytes per
-// warp and store); after the second barrier the owners' warps add what they received to their own
-// accumulators, own first, then the others in ascending order, and finish as the other kernels' epilogues do.
+// The exchange.  The accumulator of a CTA is eight units, one per epilogue warp: the 32 rows of the
+// warp's tensor-memory quarter x its share of the columns.  Unit u belongs to split u * splits / 8.  When
+// every member's MMAs are done (first cluster barrier: the rings are free) each warp whose unit is not its split's copies it,
+// in the register layout of the tensor-memory loads, to the owner's ring (512 contiguous bytes per store); after the second
+// barrier the owners' warps add what they received to their own accumulators, own first, then the others in ascending
+// order, and finish as the other kernels' epilogues do.
 #pragma once
 
 #include "epilogue.cuh"
@@ -40,16 +40,16 @@ struct SplitGemmParams {
     const uint16_t* residual;  // [M x N] bf16 (ld = ldr) or nullptr
     int64_t ldr;
     uint32_t* dev_error;
-    int tiles_m;     // tiles of R * CG * 128 rows; consecutive clusters take the row tiles of one column tile
+    int tiles_m;     // tiles of CG * 128 rows; consecutive clusters take the row tiles of one column tile
     int splits;      // members of a cluster: cluster size = CG * splits
     int lora_steps;  // R / 64 dense stages behind the last split's K blocks (0 = no low-rank branch)
     int w_prefetch;  // layer calls: W tiles of the first stages are fetched before the wait for the prune launch
     int trigger;     // the next kernel's CTAs may be placed while this grid works (enough SMs are left for them)
 };
 
-template <int R_, int BN_, int CG_, int STAGES_, bool FP8_ = false>
+template <int BN_, int CG_, int STAGES_, bool FP8_ = false>
 struct SplitCfg {
-    static constexpr int R = R_, BN = BN_, CG = CG_, STAGES = STAGES_;
+    static constexpr int BN = BN_, CG = CG_, STAGES = STAGES_;
     static constexpr bool FP8 = FP8_;
     static constexpr int BM = 128;
     static constexpr int BK = FP8 ? 256 : 128;      // logical K per stage
@@ -60,28 +60,26 @@ struct SplitCfg {
     static constexpr int E_COLS = E_BYTES / 512;
     static constexpr int B_HALF_BYTES = BN_CTA * 128;
     static constexpr int B_BYTES = 2 * B_HALF_BYTES;
-    static constexpr int STAGE_BYTES = R * (A_BYTES + E_BYTES) + B_BYTES;
+    static constexpr int STAGE_BYTES = A_BYTES + E_BYTES + B_BYTES;
     static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
     static constexpr int CH = (BN % 64 == 0) ? 64 : 48;  // epilogue column chunk
     static constexpr int NCH = BN / CH;
     static constexpr int SLOTS = (NCH + 1) / 2;          // most chunks of a unit
-    static constexpr int UNITS = 8 * R;
+    static constexpr int UNITS = 8;                      // one per epilogue warp
     static constexpr int UNIT_BYTES = SLOTS * CH * 128;  // a unit's accumulators: 32 lanes x SLOTS * CH registers
-    static constexpr int E_COL0 = R * BN;
+    static constexpr int E_COL0 = BN;
     static constexpr int TMEM_COLS = 512;
     static constexpr int STRIP_BYTES = BN * 4 * (FP8 ? 2 : 1);
-    static constexpr int NUM_BARS = 2 * STAGES + R;
+    static constexpr int NUM_BARS = 2 * STAGES + 1;
     static constexpr int SMEM_BYTES = 1024 /*align slack*/ + RING_BYTES + STRIP_BYTES + 256;
     static constexpr int THREADS = GEMM_THREADS;
     // units an owner receives from the other splits have to fit into its ring
     static constexpr bool splits_fit(int s) {
-        if (R == 2 && s != 2) return false;  // (a split finishes units of one row tile)
         return s >= 2 && CG * s <= 8 && (UNITS + s - 1) / s * (s - 1) * UNIT_BYTES <= RING_BYTES;
     }
-    static_assert(R == 1 || (R == 2 && !FP8), "row tiles per stage");
     static_assert(BN % CH == 0 && NCH >= 2 && BN % 16 == 0 && BN_CTA % 8 == 0, "tile N");
     static_assert(B_HALF_BYTES % 1024 == 0 && UNIT_BYTES % 1024 == 0, "swizzled tiles and staging boxes stay 1024-byte aligned");
-    static_assert(E_COL0 % 4 == 0 && E_COL0 + R * E_COLS * STAGES <= TMEM_COLS, "tensor memory budget");
+    static_assert(E_COL0 % 4 == 0 && E_COL0 + E_COLS * STAGES <= TMEM_COLS, "tensor memory budget");
     static_assert(8 * NUM_BARS + 16 <= 256, "barrier area");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
     static_assert(splits_fit(2), "exchange area");
@@ -93,14 +91,14 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
                          const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ CUtensorMap tmap_y,
                          const __grid_constant__ CUtensorMap tmap_t, const __grid_constant__ CUtensorMap tmap_la,
                          const SplitGemmParams p) {
-    constexpr int R = Cfg::R, CG = Cfg::CG, STAGES = Cfg::STAGES, BN = Cfg::BN;
+    constexpr int CG = Cfg::CG, STAGES = Cfg::STAGES, BN = Cfg::BN;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-    const uint32_t sA = smem_base;                          // [stage][row tile] A_BYTES
-    const uint32_t sB = sA + STAGES * R * Cfg::A_BYTES;     // [stage] B_BYTES
-    const uint32_t sE = sB + STAGES * Cfg::B_BYTES;         // [stage][row tile] E_BYTES
-    const uint32_t sStrip = sE + STAGES * R * Cfg::E_BYTES;
+    const uint32_t sA = smem_base;                   // [stage] A_BYTES
+    const uint32_t sB = sA + STAGES * Cfg::A_BYTES;  // [stage] B_BYTES
+    const uint32_t sE = sB + STAGES * Cfg::B_BYTES;  // [stage] E_BYTES
+    const uint32_t sStrip = sE + STAGES * Cfg::E_BYTES;
     const uint32_t sBar = sStrip + Cfg::STRIP_BYTES;
     const uint32_t bar_full = sBar, bar_empty = sBar + 8 * STAGES, bar_tfull = sBar + 16 * STAGES;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + (sBar - smem_base) + 8 * Cfg::NUM_BARS);
@@ -116,7 +114,7 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
     const int kb0 = split * kblocks / p.splits, nkb = (split + 1) * kblocks / p.splits - kb0;
     const int lora_steps = (LORA && split == p.splits - 1) ? p.lora_steps : 0;
     const int steps = nkb + lora_steps;
-    const int rb0 = tm * R * CG + sub;  // this CTA's 128-row block of the first row tile; the second: + CG
+    const int rb = tm * CG + sub;  // this CTA's 128-row block
     const int n0_cta = tn * BN + sub * Cfg::BN_CTA;
 
     if (threadIdx.x == 0) {
@@ -125,7 +123,7 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
             mbar_init(bar_full + 8 * s, 1);   // leader's producer arrives once (+ transaction bytes)
             mbar_init(bar_empty + 8 * s, 1);  // one tcgen05.commit
         }
-        for (int r = 0; r < R; ++r) mbar_init(bar_tfull + 8 * r, 1);  // one tcgen05.commit
+        mbar_init(bar_tfull, 1);  // one tcgen05.commit
         fence_mbar_init();
         prefetch_tmap(&tmap_a);
         prefetch_tmap(&tmap_b);
@@ -182,8 +180,8 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
             for (int i = 0; i < steps; ++i) {
                 ok = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1, cta_abort, p.dev_error);
                 if (!ok) break;
-                const uint32_t a_dst = sA + stage * (R * Cfg::A_BYTES), b_dst = sB + stage * Cfg::B_BYTES;
-                const uint32_t e_dst = sE + stage * (R * Cfg::E_BYTES);
+                const uint32_t a_dst = sA + stage * Cfg::A_BYTES, b_dst = sB + stage * Cfg::B_BYTES;
+                const uint32_t e_dst = sE + stage * Cfg::E_BYTES;
                 const uint32_t bar = full0 + 8 * stage;
                 if (!elect_one()) {
                 } else if (i < nkb) {
@@ -191,22 +189,17 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
                     const bool pre = i < npre;  // W tile and byte count went out before the wait
                     // the leader announces the bytes of both CTAs; the peer's bytes may land first
                     if (leader && !pre) mbar_arrive_expect_tx(bar_full + 8 * stage, CG * Cfg::STAGE_BYTES);
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const int rb = rb0 + r * CG;
-                        load(a_dst + r * Cfg::A_BYTES, &tmap_a, kb * Cfg::BOX_X, rb * Cfg::BM, bar);
-                        load(e_dst + r * Cfg::E_BYTES, &tmap_e, 0, E_ROWS * (rb * kblocks + kb), bar);
-                    }
+                    load(a_dst, &tmap_a, kb * Cfg::BOX_X, rb * Cfg::BM, bar);
+                    load(e_dst, &tmap_e, 0, E_ROWS * (rb * kblocks + kb), bar);
                     if (!pre) {
                         load(b_dst, &tmap_b, kb * Cfg::BK, n0_cta, bar);
                         load(b_dst + Cfg::B_HALF_BYTES, &tmap_b, kb * Cfg::BK + Cfg::BOX_X, n0_cta, bar);
                     }
                 } else {
-                    // low-rank stages: T boxes in the A slots, L_A box in the first half of the W slot
+                    // low-rank stages: T box in the A slot, L_A box in the first half of the W slot
                     const int j = i - nkb;
-                    if (leader) mbar_arrive_expect_tx(bar_full + 8 * stage, CG * (R * Cfg::A_BYTES + Cfg::B_HALF_BYTES));
-#pragma unroll
-                    for (int r = 0; r < R; ++r) load(a_dst + r * Cfg::A_BYTES, &tmap_t, j * 64, (rb0 + r * CG) * Cfg::BM, bar);
+                    if (leader) mbar_arrive_expect_tx(bar_full + 8 * stage, CG * (Cfg::A_BYTES + Cfg::B_HALF_BYTES));
+                    load(a_dst, &tmap_t, j * 64, rb * Cfg::BM, bar);
                     load(b_dst, &tmap_la, j * 64, n0_cta, bar);
                 }
                 ++issued;
@@ -239,33 +232,30 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
                 const uint32_t b_lo = b_lo0 + stage * (Cfg::B_BYTES >> 4);
                 const bool sparse = !LORA || i < nkb;
                 if (elect_one()) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const uint32_t d = tmem_base + r * BN, a_lo = a_lo0 + (stage * R + r) * (Cfg::A_BYTES >> 4);
-                        const uint32_t e = tmem_base + Cfg::E_COL0 + (stage * R + r) * Cfg::E_COLS;
-                        const uint64_t e_desc = e_d0 + (uint64_t)((stage * R + r) * (Cfg::E_BYTES >> 4));
-                        if (sparse) {
-                            tmem_cp_128x128b<CG>(e, e_desc);
-                            if constexpr (Cfg::FP8) {
-                                tmem_cp_128x128b<CG>(e + 4, e_desc + (uint64_t)(2048 >> 4));
-                                mma_sp_f8_lh<CG>(d, a_lo, b_lo, desc_hi, e, idesc8, accumulate);
-                                mma_sp_f8_lh<CG>(d, a_lo + 2, b_lo + 4, desc_hi, e + 2, idesc8, 1u);
-                                mma_sp_f8_lh<CG>(d, a_lo + 4, b_lo + BH, desc_hi, e + 4, idesc8, 1u);
-                                mma_sp_f8_lh<CG>(d, a_lo + 6, b_lo + BH + 4, desc_hi, e + 6, idesc8, 1u);
-                            } else {
-                                mma_sp_bf16_lh<CG>(d, a_lo, b_lo, desc_hi, e, idesc0, accumulate);
-                                mma_sp_bf16_lh<CG>(d, a_lo + 2, b_lo + 4, desc_hi, e, idesc1, 1u);
-                                mma_sp_bf16_lh<CG>(d, a_lo + 4, b_lo + BH, desc_hi, e + 2, idesc0, 1u);
-                                mma_sp_bf16_lh<CG>(d, a_lo + 6, b_lo + BH + 4, desc_hi, e + 2, idesc1, 1u);
-                            }
+                    const uint32_t a_lo = a_lo0 + stage * (Cfg::A_BYTES >> 4);
+                    const uint32_t e = tmem_base + Cfg::E_COL0 + stage * Cfg::E_COLS;
+                    const uint64_t e_desc = e_d0 + (uint64_t)(stage * (Cfg::E_BYTES >> 4));
+                    if (sparse) {
+                        tmem_cp_128x128b<CG>(e, e_desc);
+                        if constexpr (Cfg::FP8) {
+                            tmem_cp_128x128b<CG>(e + 4, e_desc + (uint64_t)(2048 >> 4));
+                            mma_sp_f8_lh<CG>(tmem_base, a_lo, b_lo, desc_hi, e, idesc8, accumulate);
+                            mma_sp_f8_lh<CG>(tmem_base, a_lo + 2, b_lo + 4, desc_hi, e + 2, idesc8, 1u);
+                            mma_sp_f8_lh<CG>(tmem_base, a_lo + 4, b_lo + BH, desc_hi, e + 4, idesc8, 1u);
+                            mma_sp_f8_lh<CG>(tmem_base, a_lo + 6, b_lo + BH + 4, desc_hi, e + 6, idesc8, 1u);
                         } else {
-                            mma_bf16_lh<CG>(d, a_lo, b_lo, desc_hi, idesc_dense, accumulate);
-                            mma_bf16_lh<CG>(d, a_lo + 2, b_lo + 2, desc_hi, idesc_dense, 1u);
-                            mma_bf16_lh<CG>(d, a_lo + 4, b_lo + 4, desc_hi, idesc_dense, 1u);
-                            mma_bf16_lh<CG>(d, a_lo + 6, b_lo + 6, desc_hi, idesc_dense, 1u);
+                            mma_sp_bf16_lh<CG>(tmem_base, a_lo, b_lo, desc_hi, e, idesc0, accumulate);
+                            mma_sp_bf16_lh<CG>(tmem_base, a_lo + 2, b_lo + 4, desc_hi, e, idesc1, 1u);
+                            mma_sp_bf16_lh<CG>(tmem_base, a_lo + 4, b_lo + BH, desc_hi, e + 2, idesc0, 1u);
+                            mma_sp_bf16_lh<CG>(tmem_base, a_lo + 6, b_lo + BH + 4, desc_hi, e + 2, idesc1, 1u);
                         }
-                        if (i == steps - 1) commit(bar_tfull + 8 * r);
+                    } else {
+                        mma_bf16_lh<CG>(tmem_base, a_lo, b_lo, desc_hi, idesc_dense, accumulate);
+                        mma_bf16_lh<CG>(tmem_base, a_lo + 2, b_lo + 2, desc_hi, idesc_dense, 1u);
+                        mma_bf16_lh<CG>(tmem_base, a_lo + 4, b_lo + 4, desc_hi, idesc_dense, 1u);
+                        mma_bf16_lh<CG>(tmem_base, a_lo + 6, b_lo + 6, desc_hi, idesc_dense, 1u);
                     }
+                    if (i == steps - 1) commit(bar_tfull);
                     commit(bar_empty + 8 * stage);
                 }
                 accumulate = 1u;
@@ -289,20 +279,15 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
             if constexpr (Cfg::FP8) sts32f(sc + c * 4, (p.col_scale != nullptr && n < p.N) ? p.col_scale[n] : 1.0f);
         }
         bar_sync_named(GEMM_EPI_BARRIER, 32 * GEMM_EPI_WARPS);
-        // unit of row tile r: chunks [c0, c0 + n) of the accumulator; the odd chunk goes to the first warp of the quarter in the
-        // first row tile, to the second in the other
-        auto first_chunk = [&](int r) { return h == 0 ? 0 : (r == 0 ? SLOTS : NCH - SLOTS); };
-        auto num_chunks = [&](int r) { return (h == 0) == (r == 0) ? SLOTS : NCH - SLOTS; };
-        auto owner_of = [&](int r) { return (r * 8 + ew) * p.splits / Cfg::UNITS; };
-        // where split `from` leaves unit (r, this warp) in its owner's ring
-        auto inbox = [&](int r, int owner, int from) {
-            const int local = r * 8 + ew - (owner * Cfg::UNITS + p.splits - 1) / p.splits;
+        // This warp's unit: chunks [c_own, c_own + n_own) of the accumulator; the odd chunk goes to the first warp of the quarter.
+        const int c_own = h == 0 ? 0 : SLOTS, n_own = h == 0 ? SLOTS : NCH - SLOTS, m0 = rb * Cfg::BM + q * 32;
+        const int owner = ew * p.splits / Cfg::UNITS;
+        const bool own = owner == split;
+        // where split `from` leaves the unit in its owner's ring
+        auto inbox = [&](int from) {
+            const int local = ew - (owner * Cfg::UNITS + p.splits - 1) / p.splits;
             return smem_base + (uint32_t)((local * (p.splits - 1) + (from < owner ? from : from - 1)) * Cfg::UNIT_BYTES);
         };
-        // what this warp finishes: its unit of row tile r_own, if that belongs to this split
-        const int r_own = R == 2 ? split : 0;
-        const bool own = owner_of(r_own) == split;
-        const int m0 = (rb0 + r_own * CG) * Cfg::BM + q * 32, n_own = num_chunks(r_own), c_own = first_chunk(r_own);
         float s[4];
         uint32_t packed[SLOTS][2][CH / 4];
         if (own) {
@@ -321,24 +306,19 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
                         epi_load_residual<CH>(p.residual, p.ldr, m0, p.M, tn * BN + (c_own + slot) * CH, p.N, lane, packed[slot]);
             }
         }
-        bool alive = true;
-#pragma unroll
-        for (int r = 0; r < R; ++r) alive = alive && mbar_wait_warp(bar_tfull + 8 * r, 0, cta_abort, p.dev_error);
+        const bool alive = mbar_wait_warp(bar_tfull, 0, cta_abort, p.dev_error);
         tc_fence_after();
         __syncwarp();
         cluster_arrive_release();
         cluster_wait();  // every member's MMAs are done: the rings are free
         const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int owner = owner_of(r);
-            if (!alive || owner == split) continue;
-            const uint32_t dst = mapa(inbox(r, owner, split), (uint32_t)(owner * CG + sub)) + lane * 16;
+        if (alive && !own) {
+            const uint32_t dst = mapa(inbox(split), (uint32_t)(owner * CG + sub)) + lane * 16;
 #pragma unroll
             for (int slot = 0; slot < SLOTS; ++slot) {
-                if (slot >= num_chunks(r)) break;
+                if (slot >= n_own) break;
                 uint32_t v[2][CH / 2];
-                epi_tmem_ld<CH>(t_row + r * BN + (first_chunk(r) + slot) * CH, v);
+                epi_tmem_ld<CH>(t_row + (c_own + slot) * CH, v);
                 tmem_ld_wait();
 #pragma unroll
                 for (int i = 0; i < CH / 4; ++i) {
@@ -358,11 +338,11 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
                     if (slot >= n_own) break;
                     const int c = c_own + slot;
                     uint32_t v[2][CH / 2];
-                    epi_tmem_ld<CH>(t_row + r_own * BN + c * CH, v);
+                    epi_tmem_ld<CH>(t_row + c * CH, v);
                     tmem_ld_wait();
                     for (int from = 0; from < p.splits; ++from) {
                         if (from == split) continue;
-                        const uint32_t src = inbox(r_own, split, from) + lane * 16;
+                        const uint32_t src = inbox(from) + lane * 16;
 #pragma unroll
                         for (int i = 0; i < CH / 4; ++i) {
                             uint32_t a[4];
@@ -378,7 +358,7 @@ sparse_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
             if (p.residual != nullptr) finish(std::true_type{});
             else finish(std::false_type{});
             __syncwarp();  // the unit's inbox has been read: its memory stages the results, a box per chunk
-            const uint32_t box = inbox(r_own, split, split == 0 ? 1 : 0);
+            const uint32_t box = inbox(split == 0 ? 1 : 0);
 #pragma unroll
             for (int slot = 0; slot < SLOTS; ++slot) {
                 if (slot >= n_own) break;
