@@ -60,3 +60,36 @@ def test_fp8_layer(ctx):
     ref = oracle.act_sparse_linear_fp8(u16(X), oq, ows, bias=u16(b), comp_mode=1, Yr=u16(res))
     Wq, ws = ctx.quantize_weights_fp8(W.cuda(), True)
     check_y(ctx.act_sparse_linear_fp8(X.cuda(), Wq, ws, b.cuda(), 1, res.cuda()), ref["Y"])
+
+
+@pytest.mark.parametrize("ctx", FORMS, indirect=True, ids=str)
+def test_whole_tensor_and_group_scales(ctx):
+    X, W, b, res = inputs.make_x(M, K, "outlier", 98), inputs.make_w(N, K, 98), inputs.make_bias(N, 98), inputs.make_residual(M, N, 98)
+    for mode in (2, 3):
+        ref = oracle.act_sparse_linear(u16(X), u16(W), bias=u16(b), comp_mode=mode, Yr=u16(res))
+        check_y(ctx.act_sparse_linear(X.cuda(), W.cuda(), b.cuda(), mode, res.cuda()), ref["Y"])
+
+
+def test_the_forced_form_is_what_runs(monkeypatch):
+    """Every split adds its own K blocks: some last bits differ from the unsplit product's and from another split's.  A form that
+    does not exist is refused."""
+    from paper_2605_26632_b200 import binding
+
+    X, W = inputs.make_x(M, K, "outlier", 99).cuda(), inputs.make_w(N, K, 99).cuda()
+    got = []
+    for form in ("0", "12", "13", "14"):
+        monkeypatch.setenv("LYNX_SPLIT", form)
+        c = binding.Lynx(0)
+        got.append(c.act_sparse_linear(X, W))
+        torch.cuda.synchronize()
+        assert c.last_error() == 0
+        c.close()
+    for i in range(len(got)):
+        for j in range(i):
+            assert not torch.equal(got[i], got[j]), (i, j)
+    for form in ("11", "15", "31", "59"):  # one split, ten CTAs in a cluster, no such tile, nine splits
+        monkeypatch.setenv("LYNX_SPLIT", form)
+        c = binding.Lynx(0)
+        with pytest.raises(binding.LynxError):
+            c.act_sparse_linear(X, W)
+        c.close()
