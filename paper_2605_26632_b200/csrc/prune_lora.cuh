@@ -5,26 +5,28 @@
 //     T[m, r] = bf16( (sum_k X[m,k] L_B[r,k]) / s_m )
 // Both consumers want every element of X exactly once, so X crosses HBM once instead of twice.
 //
-// One CTA per (row block of 128 or 64 rows, K split); the splits of a row block form a thread-block cluster
-// (1 to 8 CTAs).  Warp 0: TMA producer -- a stage is (128-row blocks) 128 rows x 128 K of X
-// (two 128-byte-swizzled boxes of 64 elements) plus the matching R x 128 slice of L_B.  Warp 1
-// issues eight dense tcgen05.mma (K = 16) per stage into a 128 x R fp32 accumulator in tensor
-// memory.  Warps 6..13 each read one 16 x 128 tile of the stage out of shared memory (undoing the
-// swizzle: 16-byte chunk c of row r sits at chunk c ^ (r % 8)) with the lane layout of the
-// stand-alone prune kernel, and run the same selection / compression / store code.  A stage is
-// free again when the MMAs have retired and all eight tiles are in registers.  Warps 2..5 drain
-// the accumulator into the CTA's own shared memory at the end (the L_B half of the ring is free
-// by then); after a cluster barrier every CTA finishes 128 / splits rows of T: it reads those rows
-// of every split's partial and row sums through distributed shared memory, adds them in split order
-// (the result does not depend on timing), divides by the row scale -- the sums added exactly as the
-// GEMM epilogue will add them -- and writes T.  No global round trip, no ticket.
+// One CTA per (row block of BM = 128 or 64 rows, K split); the splits of a row block form a thread-block cluster (1 to 8 CTAs,
+// of 64-row blocks 1 to 4).  Warp 0: TMA producer -- a stage is BM rows x 128 K of X (two 128-byte-swizzled boxes of
+// 64 elements) plus the matching R x 128 slice of L_B.  Warp 1 issues eight dense tcgen05.mma (K = 16) per stage into a
+// 128 x R fp32 accumulator in tensor memory.  Warps 6..13, one 16 x 128 tile of a stage each: with 128 rows all eight share a
+// stage, with 64 the first four take the even stages and the others the odd ones.  A prune warp reads its tile out of
+// shared memory (undoing the swizzle: 16-byte chunk c of row r sits at chunk c ^ (r % 8)) with the lane layout of the
+// stand-alone prune kernel, and runs the same selection / compression / store code.  A stage is free again when the MMAs have
+// retired and all of its tiles are in registers.  Warps 2..5 drain the accumulator into the CTA's own shared memory at the end
+// (the L_B half of the ring is free by then); after a cluster barrier every CTA finishes BM / splits rows of T: it reads those
+// rows of every split's partial and row sums through distributed shared memory, adds them in split order (the result does
+// not depend on timing), divides by the row scale -- the sums added exactly as the GEMM epilogue will add them: one per
+// split of 128-row blocks, two of 64-row blocks -- and writes T.  No global round trip, no ticket.
 //
-// What bounds it: the stream over X is at the HBM rate; what follows the last stage was half of the kernel
-// on 4352 x 3072 (cycles): 2700 in the cluster barrier, whose release waited for every value store of the
-// CTA, and 6400 in the finish, which 4 warps did after a global round trip for the row sums, one
-// dependent load at a time.  Now only the four drain warps release -- the prune warps hand them their row
-// sums in shared memory through a CTA barrier --, twelve warps finish T, and a thread's loads from all splits
-// are in flight together.
+// Which BM: prune_lora_plan (lynx_api.cu), fitted times.  64 rows where they fill more of the GPU: 4352 x 3072 as 136 CTAs instead
+// of 102, 13.2 -> 11.7 us, 1024 x 3072 10.0 -> 8.0; not 4096 x 12288 (31.4 against 33.1).
+//
+// What bounds it: 4352 x 3072 takes 11.7 us against 7 of the prune alone; about 4.5 of it are the first loads, the drain and the
+// cluster's exchange, the rest is the stream over X and the prune warps' ALU work.  What follows the last stage was half of
+// the kernel (cycles): 2700 in the cluster barrier, whose release waited for every value store of the CTA, and 6400 in the
+// finish, which 4 warps did after a global round trip for the row sums, one dependent load at a time.  Now only the four
+// drain warps release -- the prune warps hand them their row sums in shared memory through a CTA barrier --, twelve warps
+// finish T, and a thread's loads from all splits are in flight together.
 #pragma once
 
 #include "lora_down.cuh"
@@ -38,7 +40,7 @@ struct PruneLoraParams {
     int kb_per_split;   // 128-element K blocks per split (the last split may get fewer)
     uint16_t* values;   // [M x K/2] bf16
     uint8_t* meta;      // tensor-core order, 128 x 128 blocks of 2048 bytes
-    float* scale_partial;  // [row blocks of 16][splits][16][2] fp32 row sums (SUMS) or nullptr
+    float* scale_partial;  // [row blocks of 16][splits * TURNS][16][2] fp32 row sums (SUMS) or nullptr
     uint16_t* T;           // [M x R] bf16, leading dimension ldt
     int64_t ldt;
     uint32_t* dev_error;
@@ -176,7 +178,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     } else if (warp >= 6) {
         // ------------------------------------------------------------------ prune warps -------
         const int pw = (warp - 6) % Cfg::TILES, turn = (warp - 6) / Cfg::TILES, r = lane >> 2, q = lane & 3;
-        const int rowA_in = 16 * pw + r;                      // row inside the 128-row block; row B = + 8
+        const int rowA_in = 16 * pw + r;                      // row inside the row block; row B = + 8
         const int64_t rowA = (int64_t)tm * Cfg::BM + rowA_in, rowB = rowA + 8;
         const bool okA = rowA < p.M, okB = rowB < p.M;        // rows past M arrive as zeros (TMA fill)
         // this lane's 32 elements: box q / 2, chunks (q % 2) * 4 + 0..3 of the row's 128-byte line
@@ -235,7 +237,7 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         bar_sync_named(3, Cfg::TAIL_THREADS);
     } else {
         // ------------------------------------------------------------------ drain -------------
-        // accumulator -> this CTA's shared memory, float4 (row, 4 columns j) at (j * 128 + row) * 16:
+        // accumulator -> this CTA's shared memory, float4 (row, 4 columns j) at (j * BM + row) * 16:
         // consecutive lanes write consecutive 16-byte slots
         const int q = warp & 3;  // tensor-memory lane quarter this warp may read
         const int r_in_tile = q * 32 + lane;
@@ -266,8 +268,8 @@ prune_lora_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     else cluster_arrive_relaxed();
     cluster_wait();
     if (warp >= 2) {
-        // this CTA finishes rows [split * 128 / splits, (split + 1) * 128 / splits) of the row block
-        // (integer division: the shares differ by a row when splits does not divide 128)
+        // this CTA finishes rows [split * BM / splits, (split + 1) * BM / splits) of the row block
+        // (integer division: the shares differ by a row when splits does not divide BM)
         const int t = threadIdx.x - 64;
         const int row_first = split * Cfg::BM / p.splits;
         const int rows_per = (split + 1) * Cfg::BM / p.splits - row_first;
