@@ -479,6 +479,51 @@ lynx_status launch_gemm_cfg(lynx_ctx* ctx, const void* values, const void* meta,
     return LYNX_OK;
 }
 
+// Tensor maps and common parameters of the two-row-tile and the K-splitting kernel, from their configurations.
+struct GemmMaps {
+    CUtensorMap a, b, e, y, t, la;
+};
+template <class Cfg, bool LORA>
+bool make_gemm_maps(lynx_ctx* ctx, GemmMaps* m, const void* values, const void* meta, int64_t M, int64_t K, const void* W, int64_t N,
+                    int64_t ldw, const LoraArgs* lora, void* Y, int64_t ldy, int store_rows, CUtensorMapSwizzle store_swizzle) {
+    constexpr CUtensorMapDataType op_type = Cfg::FP8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    constexpr int op_bytes = Cfg::FP8 ? 1 : 2;
+    const uint64_t rb = (uint64_t)((M + 127) / 128), kb128 = (uint64_t)(K / 128);
+    if (!make_tmap_2d(ctx, &m->a, op_type, op_bytes, values, (uint64_t)M, (uint64_t)(K / 2), (uint64_t)(K / 2) * op_bytes, Cfg::BOX_X,
+                      Cfg::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_tmap_2d(ctx, &m->b, op_type, op_bytes, W, (uint64_t)N, (uint64_t)K, (uint64_t)ldw * op_bytes, Cfg::BOX_X, Cfg::BN_CTA,
+                      CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_tmap_2d(ctx, &m->e, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, meta, rb * kb128 * 2, 256, 1024, 256, Cfg::E_BYTES / 1024,
+                      CU_TENSOR_MAP_SWIZZLE_NONE) ||
+        !make_tmap_2d(ctx, &m->y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, (uint64_t)M, (uint64_t)N, (uint64_t)ldy * 2, Cfg::CH, store_rows,
+                      store_swizzle))
+        return false;
+    if (!LORA) {
+        m->t = m->a;  // never read: lora_steps = 0
+        m->la = m->b;
+        return true;
+    }
+    return make_tmap_2d(ctx, &m->t, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->T, (uint64_t)M, (uint64_t)lora->R, (uint64_t)lora->ldt * 2,
+                        64, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
+           make_tmap_2d(ctx, &m->la, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->LA, (uint64_t)N, (uint64_t)lora->R,
+                        (uint64_t)lora->ldla * 2, 64, Cfg::BN_CTA, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+template <class P>
+void set_gemm_params(P& p, const lynx_ctx* ctx, int64_t M, int64_t N, int64_t K, const float* wscale, const void* bias,
+                     const lynx_comp* comp, const ScaleSrc* ss, int lora_steps, bool layer_call) {
+    p.M = M; p.N = N; p.K = K;
+    p.row_scale = comp ? comp->row_scale : nullptr;
+    p.scale_partial = ss ? ss->partial : nullptr;
+    p.scale_ks = ss ? ss->ks : 0;
+    p.col_scale = wscale;
+    p.bias = static_cast<const uint16_t*>(bias);
+    p.residual = comp ? static_cast<const uint16_t*>(comp->residual) : nullptr;
+    p.ldr = comp ? comp->ldr : 0;
+    p.dev_error = ctx->err_dev;
+    p.lora_steps = lora_steps;
+    p.w_prefetch = layer_call ? 1 : 0;
+}
+
 // ------------------------------------------------------- two-row-tile GEMM kernel (sparse_gemm_rt2) -----
 
 using Rt2Cfg = Gemm2Cfg<240, 3>;
@@ -544,42 +589,12 @@ lynx_status launch_gemm_rt2(lynx_ctx* ctx, const Rt2Plan& plan, const void* valu
                             int64_t K, const void* W, int64_t N, int64_t ldw, const float* wscale, const void* bias,
                             const lynx_comp* comp, const LoraArgs* lora, void* Y, int64_t ldy, cudaStream_t st,
                             const ScaleSrc* ss, bool layer_call) {
-    constexpr CUtensorMapDataType op_type = Cfg::FP8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    constexpr int op_bytes = Cfg::FP8 ? 1 : 2;
-    CUtensorMap ta, tb, te, ty, tt, tla;
-    const uint64_t rb = (uint64_t)((M + 127) / 128), kb128 = (uint64_t)(K / 128);
-    if (!make_tmap_2d(ctx, &ta, op_type, op_bytes, values, (uint64_t)M, (uint64_t)(K / 2), (uint64_t)(K / 2) * op_bytes, Cfg::BOX_X,
-                      Cfg::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_tmap_2d(ctx, &tb, op_type, op_bytes, W, (uint64_t)N, (uint64_t)K, (uint64_t)ldw * op_bytes, Cfg::BOX_X, Cfg::BN_CTA,
-                      CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_tmap_2d(ctx, &te, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, meta, rb * kb128 * 2, 256, 1024, 256, Cfg::E_BYTES / 1024,
-                      CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !make_tmap_2d(ctx, &ty, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, (uint64_t)M, (uint64_t)N, (uint64_t)ldy * 2, Cfg::CH,
-                      Cfg::BOX_ROWS, CU_TENSOR_MAP_SWIZZLE_NONE))
+    GemmMaps m;
+    if (!make_gemm_maps<Cfg, LORA>(ctx, &m, values, meta, M, K, W, N, ldw, lora, Y, ldy, Cfg::BOX_ROWS, CU_TENSOR_MAP_SWIZZLE_NONE))
         return LYNX_ERR_CUDA;
-    if (LORA) {
-        if (!make_tmap_2d(ctx, &tt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->T, (uint64_t)M, (uint64_t)lora->R,
-                          (uint64_t)lora->ldt * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !make_tmap_2d(ctx, &tla, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->LA, (uint64_t)N, (uint64_t)lora->R,
-                          (uint64_t)lora->ldla * 2, 64, Cfg::BN_CTA, CU_TENSOR_MAP_SWIZZLE_128B))
-            return LYNX_ERR_CUDA;
-    } else {
-        tt = ta;  // never read: lora_steps = 0
-        tla = tb;
-    }
     Gemm2Params p;
-    p.M = M; p.N = N; p.K = K;
-    p.row_scale = comp ? comp->row_scale : nullptr;
-    p.scale_partial = ss ? ss->partial : nullptr;
-    p.scale_ks = ss ? ss->ks : 0;
-    p.col_scale = wscale;
-    p.bias = static_cast<const uint16_t*>(bias);
-    p.residual = comp ? static_cast<const uint16_t*>(comp->residual) : nullptr;
-    p.ldr = comp ? comp->ldr : 0;
-    p.dev_error = ctx->err_dev;
+    set_gemm_params(p, ctx, M, N, K, wscale, bias, comp, ss, LORA ? lora->R / 64 : 0, layer_call);
     p.sched.init((int)((M + 255) / 256), (int)((N + Cfg::BN - 1) / Cfg::BN), plan.clusters, plan.doubles, 8);
-    p.lora_steps = LORA ? lora->R / 64 : 0;
-    p.w_prefetch = layer_call ? 1 : 0;
     auto kern = sparse_gemm_rt2_kernel<Cfg, LORA>;
     static bool attr_set[MAX_CTX_DEVICES] = {};  // per instantiation
     if (lynx_status as = prepare_gemm_kernel(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
@@ -597,7 +612,7 @@ lynx_status launch_gemm_rt2(lynx_ctx* ctx, const Rt2Plan& plan, const void* valu
     attr[1].val.programmaticStreamSerializationAllowed = ctx->pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, te, ty, tt, tla, p) != cudaSuccess) return LYNX_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, kern, m.a, m.b, m.e, m.y, m.t, m.la, p) != cudaSuccess) return LYNX_ERR_CUDA;
     ctx->launches++;
     return LYNX_OK;
 }
@@ -643,44 +658,15 @@ template <class Cfg, bool LORA>
 lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, const void* values, const void* meta, int64_t M, int64_t K, const void* W,
                               int64_t N, int64_t ldw, const float* wscale, const void* bias, const lynx_comp* comp,
                               const LoraArgs* lora, void* Y, int64_t ldy, cudaStream_t st, const ScaleSrc* ss, bool layer_call) {
-    constexpr CUtensorMapDataType op_type = Cfg::FP8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    constexpr int op_bytes = Cfg::FP8 ? 1 : 2;
-    CUtensorMap ta, tb, te, ty, tt, tla;
-    const uint64_t rb = (uint64_t)((M + 127) / 128), kb128 = (uint64_t)(K / 128);
-    if (!make_tmap_2d(ctx, &ta, op_type, op_bytes, values, (uint64_t)M, (uint64_t)(K / 2), (uint64_t)(K / 2) * op_bytes, Cfg::BOX_X,
-                      Cfg::BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_tmap_2d(ctx, &tb, op_type, op_bytes, W, (uint64_t)N, (uint64_t)K, (uint64_t)ldw * op_bytes, Cfg::BOX_X, Cfg::BN_CTA,
-                      CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_tmap_2d(ctx, &te, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, meta, rb * kb128 * 2, 256, 1024, 256, Cfg::E_BYTES / 1024,
-                      CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !make_tmap_2d(ctx, &ty, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, (uint64_t)M, (uint64_t)N, (uint64_t)ldy * 2, Cfg::CH, 32,
-                      Cfg::CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE))
+    GemmMaps m;
+    if (!make_gemm_maps<Cfg, LORA>(ctx, &m, values, meta, M, K, W, N, ldw, lora, Y, ldy, 32,
+                                   Cfg::CH == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE))
         return LYNX_ERR_CUDA;
-    if (LORA) {
-        if (!make_tmap_2d(ctx, &tt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->T, (uint64_t)M, (uint64_t)lora->R,
-                          (uint64_t)lora->ldt * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !make_tmap_2d(ctx, &tla, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, lora->LA, (uint64_t)N, (uint64_t)lora->R,
-                          (uint64_t)lora->ldla * 2, 64, Cfg::BN_CTA, CU_TENSOR_MAP_SWIZZLE_128B))
-            return LYNX_ERR_CUDA;
-    } else {
-        tt = ta;  // never read: lora_steps = 0
-        tla = tb;
-    }
     SplitGemmParams p;
-    p.M = M; p.N = N; p.K = K;
-    p.row_scale = comp ? comp->row_scale : nullptr;
-    p.scale_partial = ss ? ss->partial : nullptr;
-    p.scale_ks = ss ? ss->ks : 0;
-    p.col_scale = wscale;
-    p.bias = static_cast<const uint16_t*>(bias);
-    p.residual = comp ? static_cast<const uint16_t*>(comp->residual) : nullptr;
-    p.ldr = comp ? comp->ldr : 0;
-    p.dev_error = ctx->err_dev;
+    set_gemm_params(p, ctx, M, N, K, wscale, bias, comp, ss, LORA ? lora->R / 64 : 0, layer_call);
     constexpr int rows = Cfg::CG * Cfg::BM;
     p.tiles_m = (int)((M + rows - 1) / rows);
     p.splits = splits;
-    p.lora_steps = LORA ? lora->R / 64 : 0;
-    p.w_prefetch = layer_call ? 1 : 0;
     const int tiles_n = (int)((N + Cfg::BN - 1) / Cfg::BN);
     auto kern = sparse_gemm_split_kernel<Cfg, LORA>;
     static bool attr_set[MAX_CTX_DEVICES] = {};  // per instantiation
@@ -701,7 +687,7 @@ lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, const void* values, con
     attr[1].val.programmaticStreamSerializationAllowed = ctx->pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, kern, ta, tb, te, ty, tt, tla, p) != cudaSuccess) return LYNX_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, kern, m.a, m.b, m.e, m.y, m.t, m.la, p) != cudaSuccess) return LYNX_ERR_CUDA;
     ctx->launches++;
     return LYNX_OK;
 }
