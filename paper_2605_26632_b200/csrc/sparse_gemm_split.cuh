@@ -6,11 +6,11 @@
 // output tile, each takes a contiguous range of its K blocks, and the fp32 accumulators are added in the
 // cluster's shared memory: no global partials, no ticket, and the order of the additions is fixed.
 //
-// What bounds it: from 96 SMs on the stream of W out of HBM (256 x 12288 x 3072: 75 MB in 16 us of 20), before that
-// the operand stream per SM.  What it adds to a tile is the exchange: ~1.1 us in two splits (24 tiles of 256 x 128, K = 3072:
-// 5.6 us besides the K blocks against 4.5).  Measured and not built: two row tiles per W stage, as in sparse_gemm_rt2_kernel
-// (an exchange of 123 KB per CTA costs ~5 us: 1024 x 12288 x 3072 44 us against 39.4 unsplit); 240- and 256-wide tiles (within 4 %
-// of the 192-wide one).
+// What bounds it (256 x K x 3072 in two splits, 96 SMs): 5.5 us that no K block is in -- launch, first loads, the exchange (~1.1
+// us), epilogue -- and 0.30 us per K block of a split, W out of HBM at 5.2 TB/s (80 % of the copy rate): 12288 is 20.0 us, of which
+// the stream alone would be 11.5.  With W in the L2 a K block takes 0.20 us, the operand stream of an SM.
+// Measured and not built: two row tiles per W stage, as in sparse_gemm_rt2_kernel (an exchange of 123 KB per CTA costs ~5 us: 1024 x
+// 12288 x 3072 44 us against 39.4 unsplit); 240- and 256-wide tiles (within 4 % of the 192-wide one).
 //
 // One tile per cluster, not persistent.  Roles per CTA as in sparse_gemm_kernel: warp 0 TMA producer, warp 1 MMA issuer (of
 // a CTA pair's leader), warps 4..11 epilogue.
