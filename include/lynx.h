@@ -354,6 +354,7 @@ LYNX_API lynx_status lynx_selftest_wait_timeout(lynx_ctx* ctx, int64_t limit_us,
  * the number of members in *splits), 0 when K is not split, -1 on bad arguments.
  * lynx_gemm_fp8_tile returns the width of the tiles (256 x 128, 192 or 240) of an FP8 product in the single-tile kernel, or -1.
  * lynx_gemm_fp8_begins_next says whether that kernel, in a layer call of that K, lets the next launch begin behind its last MMAs.
+ * lynx_gemm_split_begins_next says whether a plain layer whose K is split lets it begin while its GEMM works (148 SMs).
  * lynx_gemm_schedule_items lists the work items of CTA pair `cluster` for `tiles_m` x `tiles_n`
  * tiles of 256 x 240 over `clusters` pairs with `doubles` 512-row items: items[4i..4i+3] = first
  * row tile, column tile, row tiles (1 or 2), ordinal among the pair's single-tile items; returns
@@ -374,6 +375,7 @@ LYNX_API int lynx_gemm_schedule_items(int tiles_m, int tiles_n, int clusters, in
 LYNX_API int lynx_gemm_split_plan(int fp8, int64_t M, int64_t N, int64_t K, int lora_steps, int* splits);
 LYNX_API int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K);
 LYNX_API int lynx_gemm_fp8_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* doubles, int* clusters);
+LYNX_API int lynx_gemm_split_begins_next(lynx_comp_mode mode, int64_t M, int64_t N, int64_t K);
 LYNX_API int lynx_gemm_fp8_begins_next(int64_t K);
 LYNX_API int lynx_gemm_phase0_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* splits, int* fill);
 LYNX_API int lynx_gemm_register_shares_fit(int regs_per_thread);

@@ -28,8 +28,8 @@ EXPORTS = [
     "lynx_reserve_lora", "lynx_lora_down", "lynx_prune_compress_lora", "lynx_sparse_linear_lora", "lynx_act_sparse_linear_lora",
     "lynx_quantize_weights_fp8", "lynx_prune_compress_fp8", "lynx_sparse_linear_fp8",
     "lynx_act_sparse_linear_fp8", "lynx_gemm_plan", "lynx_gemm_schedule_items", "lynx_gemm_accumulator_waits",
-    "lynx_gemm_register_shares_fit", "lynx_gemm_split_plan", "lynx_gemm_fp8_tile", "lynx_gemm_fp8_plan", "lynx_gemm_fp8_begins_next",
-    "lynx_gemm_phase0_plan", "lynx_selftest_wait_timeout",
+    "lynx_gemm_register_shares_fit", "lynx_gemm_split_plan", "lynx_gemm_fp8_tile", "lynx_gemm_fp8_plan",
+    "lynx_gemm_fp8_begins_next", "lynx_gemm_split_begins_next", "lynx_gemm_phase0_plan", "lynx_selftest_wait_timeout",
 ]
 
 
@@ -113,6 +113,7 @@ def load_library() -> ctypes.CDLL:
     lib.lynx_gemm_fp8_tile.argtypes = [i32, i64, i64, i64]
     lib.lynx_gemm_fp8_plan.argtypes = [i32, i64, i64, i64, ctypes.POINTER(i32), ctypes.POINTER(i32)]
     lib.lynx_gemm_fp8_begins_next.argtypes = [i64]
+    lib.lynx_gemm_split_begins_next.argtypes = [i32, i64, i64, i64]
     lib.lynx_gemm_phase0_plan.argtypes = [i32, i64, i64, i64, ctypes.POINTER(i32), ctypes.POINTER(i32)]
     lib.lynx_selftest_wait_timeout.argtypes = [vp, i64, vp]
     lib.lynx_launch_count.argtypes = [vp]

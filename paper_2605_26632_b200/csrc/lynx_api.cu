@@ -653,9 +653,15 @@ int pick_gemm_cfg(const lynx_ctx* ctx, int64_t M, int64_t N, int64_t K, int lora
 // prologue: 256 x 3072 x 3072 layer 10.1 -> 9.8 us.  With fewer they pile up on the few that are: 128 x 3072 x 9216
 // (144 SMs) 16.2 -> 17.6.
 bool split_begins_next(int64_t ctas, int num_sms) { return ctas * 4 <= (int64_t)num_sms * 3; }
+// In a plain layer also only where the next prune launch is short: its blocks take the free SMs before the others are done, and from
+// some number of them on that is where most of its work stays.  NONE and ROW up to 512 rows (442 x 2816 x 336 9.9 us without, 9.4 with
+// it, 250 x 5120 x 680 11.1, 10.5; but 700 x 3072 x 424 10.5, 11.2 and 1500 x 3072 x 256 11.3, 12.3); not where its kernel does more
+// per element or another launch follows it (GROUP 700 x 3072 x 424 13.3, 15.4, 150 x 5120 x 3072 14.8, 15.7; TENSOR 14.4, 16.0
+// and 14.9, 15.8).  The low-rank and FP8 layers' prune kernels have a block per SM: they gain at every size.
+bool plain_layer_begins_next(lynx_comp_mode mode, int64_t M) { return (mode == LYNX_COMP_NONE || mode == LYNX_COMP_ROW) && M <= 512; }
 
 template <class Cfg, bool LORA>
-lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, const void* values, const void* meta, int64_t M, int64_t K, const void* W,
+lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, bool next_early, const void* values, const void* meta, int64_t M, int64_t K, const void* W,
                               int64_t N, int64_t ldw, const float* wscale, const void* bias, const lynx_comp* comp,
                               const LoraArgs* lora, void* Y, int64_t ldy, cudaStream_t st, const ScaleSrc* ss, bool layer_call) {
     GemmMaps m;
@@ -673,7 +679,7 @@ lynx_status launch_gemm_split(lynx_ctx* ctx, int splits, const void* values, con
     if (lynx_status as = prepare_gemm_kernel(kern, Cfg::SMEM_BYTES, ctx->device, attr_set); as != LYNX_OK) return as;
     cudaLaunchConfig_t cfg = {};
     const int grid = p.tiles_m * tiles_n * splits * Cfg::CG;
-    p.trigger = split_begins_next(grid, ctx->num_sms) ? 1 : 0;
+    p.trigger = next_early && split_begins_next(grid, ctx->num_sms) ? 1 : 0;
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(Cfg::THREADS);
     cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
@@ -715,6 +721,7 @@ struct SplitPlan {
     int id = 0, splits = 1;
     double t_us = 1e30;
     int64_t ctas = 0;
+    bool next_early = true;  // the next launch may begin while this one works, if it leaves enough SMs
 };
 template <bool FP8>
 SplitPlan split_plan(const int (&cap)[9], int64_t M, int64_t N, int64_t K, int lora_steps) {
@@ -726,7 +733,7 @@ SplitPlan split_plan(const int (&cap)[9], int64_t M, int64_t N, int64_t K, int l
         for (int s = 2; s * c.cg <= 8 && s <= kb; ++s) {
             if (tiles * s * c.cg > cap[s * c.cg]) continue;
             const double t = (double)((kb + s - 1) / s + lora_steps) * c.t_kb + c.fix + 0.3 * c.cg * (s - 2);
-            if (t < best.t_us) best = SplitPlan{c.id, s, t, tiles * s * c.cg};
+            if (t < best.t_us) best = SplitPlan{c.id, s, t, tiles * s * c.cg, true};
         }
     }
     return best;
@@ -740,7 +747,7 @@ lynx_status launch_gemm_split_id(lynx_ctx* ctx, const SplitPlan& plan, const voi
         using Cfg = decltype(cfg);
         const int splits = plan.splits;
         if (!Cfg::splits_fit(splits) || splits > K / Cfg::BK) return LYNX_ERR_INVALID_ARG;
-#define LYNX_SPLIT_ARGS ctx, splits, values, meta, M, K, W, N, ldw, wscale, bias, comp, lora, Y, ldy, st, ss, layer_call
+#define LYNX_SPLIT_ARGS ctx, splits, plan.next_early, values, meta, M, K, W, N, ldw, wscale, bias, comp, lora, Y, ldy, st, ss, layer_call
         if constexpr (!FP8) {
             if (lora) return launch_gemm_split<Cfg, true>(LYNX_SPLIT_ARGS);
         }
@@ -779,7 +786,7 @@ SplitPlan split_plan_if_faster(const int (&cap)[9], int num_sms, int64_t M, int6
 template <bool FP8>
 SplitPlan choose_split(const lynx_ctx* ctx, int64_t M, int64_t N, int64_t K, int lora_steps) {
     if (ctx->split == 0) return SplitPlan{};
-    if (ctx->split > 0) return SplitPlan{ctx->split / 10, ctx->split % 10, 0.0, 0};
+    if (ctx->split > 0) return SplitPlan{ctx->split / 10, ctx->split % 10, 0.0, 0, true};
     return split_plan_if_faster<FP8>(ctx->cluster_cap, ctx->num_sms, M, N, K, lora_steps);
 }
 
@@ -789,10 +796,11 @@ bool cfg_supports_l0(int cfg) { return cfg >= 1 && cfg <= 8 && cfg != 6; }
 lynx_status launch_gemm(lynx_ctx* ctx, const void* values, const void* meta, int64_t M, int64_t K, const void* W,
                         int64_t N, int64_t ldw, const void* bias, const lynx_comp* comp, const LoraArgs* lora, void* Y,
                         int64_t ldy, cudaStream_t st, int cfg = 0, const ScaleSrc* ss = nullptr, bool layer_call = false,
-                        bool split_ok = true) {
+                        bool split_ok = true, bool next_early = true) {
     const int lora_steps = lora ? lora->R / 64 : 0;
     if (split_ok && cfg == 0 && ctx->gemm_cfg == 0 && ctx->rt2 != 1 && !ctx->streamk && !(lora && lora->X)) {
-        const SplitPlan plan = choose_split<false>(ctx, M, N, K, lora_steps);
+        SplitPlan plan = choose_split<false>(ctx, M, N, K, lora_steps);
+        plan.next_early = next_early;
         if (plan.id)
             return launch_gemm_split_id<false>(ctx, plan, values, meta, M, K, W, N, ldw, nullptr, bias, comp, lora, Y, ldy, st, ss, layer_call);
     }
@@ -890,7 +898,8 @@ lynx_status launch_gemm_fp8(lynx_ctx* ctx, const void* values_q, const void* met
                             const void* Wq, int64_t N, int64_t ldwq, const float* wscale, const void* bias,
                             const lynx_comp* comp, void* Y, int64_t ldy, cudaStream_t st, bool layer_call = false) {
     if (ctx->gemm_cfg == 0 && ctx->rt2 != 1) {
-        const SplitPlan plan = choose_split<true>(ctx, M, N, K, 0);
+        SplitPlan plan = choose_split<true>(ctx, M, N, K, 0);
+        plan.next_early = !layer_call || (ctx->fp8_ring && fp8_ring_slots(K));
         if (plan.id)
             return launch_gemm_split_id<true>(ctx, plan, values_q, meta, M, K, Wq, N, ldwq, wscale, bias, comp, nullptr, Y, ldy, st, nullptr,
                                               layer_call);
@@ -1513,7 +1522,7 @@ static lynx_status act_sparse_linear_impl(lynx_ctx* ctx, const void* X, int64_t 
     comp.ldr = ldr;
     if ((s = check_device_error(ctx)) == LYNX_OK)
         s = launch_gemm(ctx, values, meta, M, K, W, N, ldw, bias, &comp, nullptr, Y, ldy,
-                        static_cast<cudaStream_t>(stream), 0, &ss, true, split_ok);
+                        static_cast<cudaStream_t>(stream), 0, &ss, true, split_ok, plain_layer_begins_next(mode, M));
     clear_deferred(ctx);  // the sums in the scratch belonged to this call
     return s;
 }
@@ -2030,6 +2039,12 @@ int lynx_gemm_fp8_plan(int num_sms, int64_t M, int64_t N, int64_t K, int* double
 }
 
 int lynx_gemm_fp8_begins_next(int64_t K) { return K < 256 || K % 256 ? -1 : fp8_ring_slots(K) ? 1 : 0; }
+
+int lynx_gemm_split_begins_next(lynx_comp_mode mode, int64_t M, int64_t N, int64_t K) {
+    if (M < 1 || N < 8 || K < 128) return -1;
+    const SplitPlan plan = split_plan_if_faster<false>(CLUSTER_CAP_148, 148, M, N, K, 0);
+    return plan.id && plain_layer_begins_next(mode, M) && split_begins_next(plan.ctas, 148) ? 1 : 0;
+}
 
 int lynx_gemm_fp8_tile(int num_sms, int64_t M, int64_t N, int64_t K) {
     if (num_sms < 2 || M < 1 || N < 8 || K < 256) return -1;

@@ -352,6 +352,17 @@ def test_split_plan_is_not_chosen_where_it_was_measured_slower():
             assert not binding.gemm_plan(148, m, n, k, lora)[0], (m, n, k, lora)
 
 
+def test_split_layers_let_the_next_launch_begin_only_before_a_short_prune_launch():
+    from paper_2605_26632_b200 import binding
+
+    begins = binding.load_library().lynx_gemm_split_begins_next
+    for mode, early in ((binding.COMP_NONE, 1), (binding.COMP_ROW, 1), (binding.COMP_TENSOR, 0), (binding.COMP_GROUP, 0)):
+        assert begins(mode, 256, 3072, 3072) == begins(mode, 442, 336, 2816) == begins(mode, 512, 256, 5120) == early
+        assert begins(mode, 700, 424, 3072) == begins(mode, 1500, 256, 3072) == begins(mode, 513, 256, 5120) == 0
+        assert begins(mode, 226, 3840, 3840) == 0  # 120 SMs are held
+        assert begins(mode, 256, 512, 512) == 0  # K is not split
+
+
 def test_split_plan_is_one_round_and_has_a_k_block_for_every_member():
     import random
 
